@@ -275,8 +275,8 @@ constexpr uint32_t kLPoolPerKey = 40;  // words of coefficient rows per shard ke
 // rows take ~0.0011 m words per key.
 constexpr uint32_t kLgeBigShard = 24576;
 struct LgeOffsets {
-    uint64_t cev, porder, proff, f0, f1, cand, core, eqst, inc_off, inc_cur, inc_list, vstate, act, actv,
-        solves, soff, srec, dense, lc, L, lpool, total;
+    uint64_t ev, prec, proff, lists, core, eqst, inc_off, inc_list, vstate, act, actv, solves, soff, srec, dense, lc,
+        L, lpool, total;
     uint32_t a_cap;  // active variables a shard may have
 };
 
@@ -289,27 +289,24 @@ __host__ __device__ constexpr uint64_t lge_take(uint64_t& p, uint64_t words) {
 __host__ __device__ constexpr LgeOffsets lge_offsets(uint32_t m, uint32_t V) {
     LgeOffsets o{};
     uint64_t p = 0;
-    o.cev = lge_take(p, 3ull * m);
-    o.porder = lge_take(p, m);
+    o.ev = lge_take(p, 2ull * m);     // vertices of an edge, 16 bits each
+    o.prec = lge_take(p, 2ull * m);   // one uint2 per peeled edge
     o.proff = lge_take(p, V + 2ull);
-    o.f0 = lge_take(p, V);
-    o.f1 = lge_take(p, V);
-    o.cand = lge_take(p, V);
-    o.core = lge_take(p, m);
+    o.lists = lge_take(p, 3 * ((V + 1ull) / 2));  // frontiers and candidates (16 bits), then round queues
+    o.core = lge_take(p, (m + 1ull) / 2);
     o.eqst = lge_take(p, m);
     o.inc_off = lge_take(p, V + 1ull);
-    o.inc_cur = lge_take(p, V);
-    o.inc_list = lge_take(p, 3ull * m);
+    o.inc_list = lge_take(p, (3ull * m + 1) / 2);
     o.vstate = lge_take(p, V);
-    o.act = lge_take(p, V);
+    o.act = lge_take(p, (V + 1ull) / 2);
     const uint64_t big = m > kLgeBigShard ? m - kLgeBigShard : 0;
     o.a_cap = uint32_t(kMaxActive + big / 8);
     o.actv = lge_take(p, o.a_cap);
     o.solves = lge_take(p, m);
     o.soff = lge_take(p, uint64_t(m) + V + 4);
-    o.srec = lge_take(p, 4ull * m);  // one uint4 per solve
+    o.srec = lge_take(p, 2ull * m);   // one uint2 per solve
     o.dense = lge_take(p, m);
-    o.lc = lge_take(p, m);
+    o.lc = lge_take(p, uint64_t(m) + o.a_cap);
     o.lpool = uint64_t(m) * (kLPoolPerKey + big / 500) + 4096;
     o.L = lge_take(p, o.lpool);
     o.total = p;

@@ -64,31 +64,53 @@ __device__ __forceinline__ uint32_t xr_of(const uint32_t* xrw, uint32_t v) {
     return (xrw[v >> 1] >> ((v & 1u) * 16u)) & 0xFFFFu;
 }
 
-// Inclusive-to-exclusive scan of arr[0..len) in global memory by one CTA.
-__device__ void cta_exclusive_scan(uint32_t* arr, uint32_t len, uint32_t* s_part) {
-    const uint32_t T = blockDim.x, tid = threadIdx.x;
+// Exclusive scan of cnt[0..len) by one CTA; part: one word per warp of scratch.
+// Each thread takes a run of consecutive entries.
+__device__ void cta_exclusive_scan(uint32_t* cnt, uint32_t len, uint32_t* part) {
+    const uint32_t T = blockDim.x, tid = threadIdx.x, lane = tid & 31u;
     const uint32_t chunk = (len + T - 1) / T;
     const uint32_t lo = min(len, tid * chunk), hi = min(len, lo + chunk);
     uint32_t sum = 0;
-    for (uint32_t i = lo; i < hi; i++) sum += arr[i];
-    s_part[tid] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t run = 0;
-        for (uint32_t t = 0; t < T; t++) {
-            uint32_t x = s_part[t];
-            s_part[t] = run;
-            run += x;
-        }
+    for (uint32_t i = lo; i < hi; i++) sum += cnt[i];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= uint32_t(d)) incl += y;
     }
+    if (lane == 31) part[tid >> 5] = incl;
     __syncthreads();
-    uint32_t run = s_part[tid];
+    uint32_t run = incl - sum;
+    for (uint32_t w = 0; w < (tid >> 5); w++) run += part[w];
     for (uint32_t i = lo; i < hi; i++) {
-        uint32_t x = arr[i];
-        arr[i] = run;
+        const uint32_t x = cnt[i];
+        cnt[i] = run;
         run += x;
     }
     __syncthreads();
+}
+
+// A slot of *ctr for every lane with `p` (one shared atomic per warp; all
+// lanes of the warp call it).
+__device__ __forceinline__ uint32_t warp_slot(uint32_t* ctr, bool p) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, p);
+    if (m == 0) return 0;
+    const unsigned lane = threadIdx.x & 31u;
+    const int lead = __ffs(m) - 1;
+    uint32_t at = 0;
+    if (int(lane) == lead) at = atomicAdd(ctr, uint32_t(__popc(m)));
+    return __shfl_sync(0xFFFFFFFFu, at, lead) + __popc(m & ((1u << lane) - 1u));
+}
+
+// The same for counters that differ by lane (key: which one): one atomic per
+// distinct key of the warp's lanes with `p`.
+__device__ __forceinline__ uint32_t warp_slot_by(uint32_t* ctrs, uint32_t key, bool p) {
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, p ? key : kNone);
+    const unsigned lane = threadIdx.x & 31u;
+    const int lead = __ffs(peers) - 1;
+    uint32_t at = 0;
+    if (p && int(lane) == lead) at = atomicAdd(ctrs + key, uint32_t(__popc(peers)));
+    return __shfl_sync(0xFFFFFFFFu, at, lead) + __popc(peers & ((1u << lane) - 1u));
 }
 
 // Drops the 128-byte L2 lines wholly inside [p, p + words) without writing
@@ -108,23 +130,20 @@ __device__ __forceinline__ void discard_words(const uint32_t* p, uint64_t words)
 // words of coefficient rows (and slab-resident dense system) it wrote.
 __device__ void discard_slab(const uint32_t* scr, const LgeOffsets& o, uint32_t m, uint32_t V, uint64_t lused) {
     const uint64_t mm = m, vv = V;
-    discard_words(scr + o.cev, 3 * mm);
-    discard_words(scr + o.porder, mm);
+    discard_words(scr + o.ev, 2 * mm);
+    discard_words(scr + o.prec, 2 * mm);
     discard_words(scr + o.proff, vv + 2);
-    discard_words(scr + o.f0, vv);
-    discard_words(scr + o.f1, vv);
-    discard_words(scr + o.cand, vv);
-    discard_words(scr + o.core, mm);
+    discard_words(scr + o.lists, 3 * ((vv + 1) / 2));
+    discard_words(scr + o.core, mm / 2);
     discard_words(scr + o.eqst, mm);
     discard_words(scr + o.inc_off, vv + 1);
-    discard_words(scr + o.inc_cur, vv);
-    discard_words(scr + o.inc_list, 3 * mm);
+    discard_words(scr + o.inc_list, 3 * mm / 2);
     discard_words(scr + o.vstate, vv);
-    discard_words(scr + o.act, vv);
+    discard_words(scr + o.act, vv / 2);
     discard_words(scr + o.actv, o.a_cap);
     discard_words(scr + o.solves, mm);
     discard_words(scr + o.soff, mm + vv + 4);
-    discard_words(scr + o.srec, 4 * mm);
+    discard_words(scr + o.srec, 2 * mm);
     discard_words(scr + o.dense, mm);
     discard_words(scr + o.lc, mm);
     discard_words(scr + o.L, lused < o.lpool ? lused : o.lpool);
@@ -143,30 +162,30 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     extern __shared__ __align__(16) uint32_t sm[];
     __shared__ uint32_t s_shard, s_fail;
     __shared__ uint32_t s_cnt[4];
-    __shared__ uint32_t s_C, s_rem, s_A, s_S, s_D, s_r, s_apos, s_nact, s_nbatch, s_piv, s_lo, s_dup;
+    __shared__ uint32_t s_C, s_rem, s_A, s_S, s_D, s_r, s_apos, s_nact, s_nbatch, s_lo, s_dup;
     __shared__ uint32_t s_hist[256];
     __shared__ uint32_t s_batch[kMaxBatch];
     __shared__ uint32_t s_part[kLT];
+    __shared__ __align__(16) uint32_t s_cand[2][kLT / 32 + 2];  // pivot candidates, one per warp
+    __shared__ uint32_t s_piv[32];                               // pivot rows of a panel
 
     const uint32_t tid = threadIdx.x, T = blockDim.x;
+    const unsigned lane = tid & 31u, warp = tid >> 5;
     const LgeOffsets o = lge_offsets(a.m_cap, a.v_cap);
     uint32_t* scr = a.scratch + uint64_t(blockIdx.x) * a.scratch_words_per_cta;
-    uint32_t* cev = scr + o.cev;
-    uint32_t* porder = scr + o.porder;
+    uint2* ev = reinterpret_cast<uint2*>(scr + o.ev);      // an edge's vertices: v0 | v1 << 16, v2
+    uint2* prec = reinterpret_cast<uint2*>(scr + o.prec);  // a peeled edge: its vertex | edge << 16, other | other << 16
     uint32_t* proff = scr + o.proff;
-    uint32_t* fr[2] = {scr + o.f0, scr + o.f1};
-    uint32_t* cand = scr + o.cand;
-    uint32_t* core = scr + o.core;
+    uint16_t* core = reinterpret_cast<uint16_t*>(scr + o.core);
     uint32_t* eqst = scr + o.eqst;
     uint32_t* inc_off = scr + o.inc_off;
-    uint32_t* inc_cur = scr + o.inc_cur;
-    uint32_t* inc_list = scr + o.inc_list;
+    uint16_t* inc_list = reinterpret_cast<uint16_t*>(scr + o.inc_list);
     uint32_t* vstate = scr + o.vstate;
-    uint32_t* act = scr + o.act;
+    uint16_t* act = reinterpret_cast<uint16_t*>(scr + o.act);
     uint32_t* actv = scr + o.actv;
     uint32_t* solves = scr + o.solves;
     uint32_t* soff = scr + o.soff;
-    uint4* srec = reinterpret_cast<uint4*>(scr + o.srec);
+    uint2* srec = reinterpret_cast<uint2*>(scr + o.srec);  // a solve: variable | edge << 16, other | other << 16
     uint32_t* dense = scr + o.dense;
     uint32_t* lc = scr + o.lc;
     uint32_t* L = scr + o.L;
@@ -219,6 +238,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         gg.kind = task.kind;
         gg.fpb = task.fpb;
         gg.fps = task.fps;
+        gg.k = 3;
         if (m > a.m_cap || V > a.v_cap || V > 65535u || m > 65535u) {
             // (nothing was written to the slab: prev_m, prev_v stay 0)
             if (tid == 0) {
@@ -242,17 +262,25 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             __syncthreads();
             continue;
         }
+        // frontier lists and the edges read off them: behind the counters when they fit
+        const uint32_t lw = (V + 1) / 2;
+        uint16_t* lists = reinterpret_cast<uint16_t*>(pw + 3 * lw <= kLgeSmemWords ? sm + pw : scr + o.lists);
+        uint16_t* const cand = lists + 4 * lw;
         for (uint32_t i = tid; i < pw; i += T) sm[i] = 0;
         prev_m = m;  // the slab is written from here on
         prev_v = V;
+        if (tid == 0) {
+            s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
+            proff[0] = 0;
+        }
         __syncthreads();
         for (uint32_t e = tid; e < m; e += T) {
             uint64_t v[4];
             edge_of(gg, __ldg(a.loc + e0 + e), v);
+            ev[e] = make_uint2(uint32_t(v[0]) | uint32_t(v[1]) << 16, uint32_t(v[2]));
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 uint32_t vk = uint32_t(v[k]);
-                cev[3 * e + k] = vk;
                 uint32_t sh8 = (vk & 3u) * 8u;
                 uint32_t old = atomicAdd(&degw[vk >> 2], 1u << sh8);
                 if (((old >> sh8) & 255u) == 255u) s_fail = 1;
@@ -270,41 +298,45 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         }
 
         // -------------------------------------------------------------------- 2. peel
-        if (tid == 0) {
-            s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
-            proff[0] = 0;
+        for (uint32_t v0 = tid & ~31u; v0 < V; v0 += T) {
+            const uint32_t v = v0 + lane;
+            const bool one = v < V && deg_of(degw, v) == 1u;
+            const uint32_t at = warp_slot(&s_cnt[0], one);
+            if (one) lists[at] = uint16_t(v);
         }
-        __syncthreads();
-        for (uint32_t v = tid; v < V; v += T)
-            if (deg_of(degw, v) == 1u) fr[0][atomicAdd(&s_cnt[0], 1u)] = v;
         __syncthreads();
         uint32_t fi = 0;
         for (;;) {
             const uint32_t nF = s_cnt[fi];
             if (nF == 0) break;
-            const uint32_t* F = fr[fi];
-            uint32_t* G = fr[fi ^ 1];
+            const uint16_t* F = lists + (fi ? 2 * lw : 0u);
+            uint16_t* G = lists + (fi ? 0u : 2 * lw);
+            // 65535 stands for none: an edge index is at most 65534
             for (uint32_t i = tid; i < nF; i += T) {
-                uint32_t v = __ldcg(&F[i]);
-                cand[i] = deg_of(degw, v) == 1u ? xr_of(xrw, v) : kNone;
+                const uint32_t v = F[i];
+                cand[i] = uint16_t(deg_of(degw, v) == 1u ? xr_of(xrw, v) : 0xFFFFu);
             }
             __syncthreads();
-            for (uint32_t i = tid; i < nF; i += T) {
-                uint32_t e = __ldcg(&cand[i]);
-                if (e == kNone) continue;
-                uint32_t bit = 1u << (e & 31u);
-                if (atomicOr(&clm[e >> 5], bit) & bit) continue;
-                uint32_t v = __ldcg(&F[i]);
-                uint32_t side = __ldcg(&cev[3 * e]) == v ? 0u : __ldcg(&cev[3 * e + 1]) == v ? 1u : 2u;
-                porder[atomicAdd(&s_cnt[2], 1u)] = (e << 2) | side;
+            for (uint32_t i0 = tid & ~31u; i0 < nF; i0 += T) {
+                const uint32_t i = i0 + lane;
+                const uint32_t e = i < nF ? cand[i] : 0xFFFFu;
+                const uint32_t bit = 1u << (e & 31u);
+                const bool mine = e != 0xFFFFu && !(atomicOr(&clm[e >> 5], bit) & bit);
+                const uint32_t at = warp_slot(&s_cnt[2], mine);
+                if (mine) {
+                    const uint32_t v = F[i];
+                    const uint2 x = __ldcg(ev + e);
+                    const uint32_t a0 = x.x & 0xFFFFu, a1 = x.x >> 16;
+                    const uint32_t u0 = a0 == v ? a1 : a0, u1 = x.y == v ? a1 : x.y;
+                    prec[at] = make_uint2(v | e << 16, u0 | u1 << 16);
 #pragma unroll
-                for (uint32_t k = 0; k < 3; k++) {
-                    if (k == side) continue;
-                    uint32_t u = __ldcg(&cev[3 * e + k]);
-                    uint32_t sh8 = (u & 3u) * 8u;
-                    uint32_t old = atomicSub(&degw[u >> 2], 1u << sh8);
-                    atomicXor(&xrw[u >> 1], e << ((u & 1u) * 16u));
-                    if (((old >> sh8) & 255u) == 2u) G[atomicAdd(&s_cnt[fi ^ 1], 1u)] = u;
+                    for (int k = 0; k < 2; k++) {
+                        const uint32_t u = k ? u1 : u0;
+                        const uint32_t sh8 = (u & 3u) * 8u;
+                        const uint32_t old = atomicSub(&degw[u >> 2], 1u << sh8);
+                        atomicXor(&xrw[u >> 1], e << ((u & 1u) * 16u));
+                        if (((old >> sh8) & 255u) == 2u) G[atomicAdd(&s_cnt[fi ^ 1], 1u)] = uint16_t(u);
+                    }
                 }
             }
             __syncthreads();
@@ -320,61 +352,104 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         const uint32_t prounds = s_cnt[3];
 
         // ---------------------------------------------------- 3. lazy Gaussian elimination
-        uint32_t C = 0;
+        uint32_t C = 0, A = 0, S = 0, D = 0, R = 0;
         if (peeled < m) {
             if (tid == 0) s_C = 0;
             __syncthreads();
-            for (uint32_t e = tid; e < m; e += T)
-                if (!((clm[e >> 5] >> (e & 31u)) & 1u)) core[atomicAdd(&s_C, 1u)] = e;
-            for (uint32_t v = tid; v <= V; v += T) inc_off[v] = 0;
+            for (uint32_t f0 = tid & ~31u; f0 < m; f0 += T) {
+                const uint32_t e = f0 + lane;
+                const bool open = e < m && !((clm[e >> 5] >> (e & 31u)) & 1u);
+                const uint32_t at = warp_slot(&s_C, open);
+                if (open) core[at] = uint16_t(e);
+            }
             __syncthreads();
             C = s_C;
             // Variable states and equation states move to shared memory when they
             // fit (the peel's arrays are dead now); otherwise they stay in the slab.
             // Equation word: bits 0-1 idle count, bit 2 done, bits 3.. XOR of its idle variables.
             const bool in_smem = uint64_t(V) + C <= kLgeSmemWords;
-            uint32_t* vst = in_smem ? sm : vstate;
+            uint32_t* vst = in_smem ? sm : vstate;  // first the core degrees, then the list cursors
             uint32_t* est = in_smem ? sm + V : eqst;
-            for (uint32_t j = tid; j < C; j += T) {
-                const uint32_t* evp = cev + 3 * __ldcg(&core[j]);
-                const uint32_t ev[3] = {__ldcg(evp), __ldcg(evp + 1), __ldcg(evp + 2)};
-                atomicAdd(&inc_off[ev[0]], 1u);
-                atomicAdd(&inc_off[ev[1]], 1u);
-                atomicAdd(&inc_off[ev[2]], 1u);
-                est[j] = ((ev[0] ^ ev[1] ^ ev[2]) << 3) | 3u;
-            }
             for (uint32_t v = tid; v < V; v += T) vst[v] = 0;
             for (uint32_t i = tid; i < 256; i += T) s_hist[i] = 0;
             __syncthreads();
-            // activation order: core degree, heaviest first (counting sort)
-            for (uint32_t v = tid; v < V; v += T) {
-                uint32_t d = __ldcg(&inc_off[v]);
-                if (d) atomicAdd(&s_hist[min(d, 255u)], 1u);
-            }
-            cta_exclusive_scan(inc_off, V + 1, s_part);
-            for (uint32_t v = tid; v < V; v += T) inc_cur[v] = __ldcg(&inc_off[v]);
-            if (tid == 0) {
-                uint32_t run = 0;
-                for (int d = 255; d >= 1; d--) {
-                    uint32_t x = s_hist[d];
-                    s_hist[d] = run;
-                    run += x;
-                }
-                s_nact = run;
-            }
-            __syncthreads();
-            for (uint32_t v = tid; v < V; v += T) {
-                uint32_t d = __ldcg(&inc_off[v + 1]) - __ldcg(&inc_off[v]);
-                if (d) act[atomicAdd(&s_hist[min(d, 255u)], 1u)] = v;
-            }
             for (uint32_t j = tid; j < C; j += T) {
-                const uint32_t* evp = cev + 3 * __ldcg(&core[j]);
-                const uint32_t ev[3] = {__ldcg(evp), __ldcg(evp + 1), __ldcg(evp + 2)};
-                inc_list[atomicAdd(&inc_cur[ev[0]], 1u)] = j;
-                inc_list[atomicAdd(&inc_cur[ev[1]], 1u)] = j;
-                inc_list[atomicAdd(&inc_cur[ev[2]], 1u)] = j;
+                const uint2 x = __ldcg(ev + core[j]);
+                const uint32_t v0 = x.x & 0xFFFFu, v1 = x.x >> 16, v2 = x.y;
+                atomicAdd(&vst[v0], 1u);
+                atomicAdd(&vst[v1], 1u);
+                atomicAdd(&vst[v2], 1u);
+                est[j] = ((v0 ^ v1 ^ v2) << 3) | 3u;
             }
             __syncthreads();
+            // activation order: core degree, heaviest first (counting sort)
+            for (uint32_t v0 = tid & ~31u; v0 < V; v0 += T) {
+                const uint32_t d = v0 + lane < V ? vst[v0 + lane] : 0u;
+                warp_slot_by(s_hist, min(d, 255u), d != 0);
+            }
+            __syncthreads();
+            if (warp == 0) {  // s_hist[d]: variables of larger core degree
+                uint32_t x[8], sum = 0;
+#pragma unroll
+                for (int k = 0; k < 8; k++) {
+                    x[k] = s_hist[255 - (8 * lane + k)];
+                    sum += x[k];
+                }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                    if (lane >= unsigned(d)) incl += y;
+                }
+                uint32_t run = incl - sum;
+#pragma unroll
+                for (int k = 0; k < 8; k++) {
+                    s_hist[255 - (8 * lane + k)] = run;
+                    run += x[k];
+                }
+                if (lane == 31) s_nact = run;
+            }
+            __syncthreads();
+            for (uint32_t v0 = tid & ~31u; v0 < V; v0 += T) {
+                const uint32_t v = v0 + lane;
+                const uint32_t d = v < V ? vst[v] : 0u;
+                const uint32_t at = warp_slot_by(s_hist, min(d, 255u), d != 0);
+                if (d) act[at] = uint16_t(v);
+            }
+            __syncthreads();
+            cta_exclusive_scan(vst, V, s_part);
+            // The incidence offsets (at most 3C) go to shared memory as 16-bit
+            // entries after the states when they fit, and so does the incidence
+            // list: the elimination rounds then wait on no memory beyond it.
+            uint16_t* ioff16 = nullptr;
+            uint32_t used = V + C;
+            if (in_smem && 3ull * C < 65536 && uint64_t(used) + (V + 2) / 2 <= kLgeSmemWords) {
+                ioff16 = reinterpret_cast<uint16_t*>(sm + used);
+                used += (V + 2) / 2;
+            }
+            constexpr uint32_t kQueueRoom = 1024;  // words kept for the round queues
+            uint16_t* ilist = inc_list;
+            if (ioff16 && uint64_t(used) + (3 * C + 1) / 2 + kQueueRoom <= kLgeSmemWords) {
+                ilist = reinterpret_cast<uint16_t*>(sm + used);
+                used += (3 * C + 1) / 2;
+            }
+            if (ioff16) {
+                for (uint32_t v = tid; v < V; v += T) ioff16[v] = uint16_t(vst[v]);
+                if (tid == 0) ioff16[V] = uint16_t(3 * C);
+            } else {
+                for (uint32_t v = tid; v < V; v += T) inc_off[v] = vst[v];
+                if (tid == 0) inc_off[V] = 3 * C;
+            }
+            __syncthreads();
+            for (uint32_t j = tid; j < C; j += T) {
+                const uint2 x = __ldcg(ev + core[j]);
+                ilist[atomicAdd(&vst[x.x & 0xFFFFu], 1u)] = uint16_t(j);
+                ilist[atomicAdd(&vst[x.x >> 16], 1u)] = uint16_t(j);
+                ilist[atomicAdd(&vst[x.y], 1u)] = uint16_t(j);
+            }
+            auto off_of = [&](uint32_t v) -> uint32_t { return ioff16 ? uint32_t(ioff16[v]) : __ldcg(&inc_off[v]); };
+            __syncthreads();
+            for (uint32_t v = tid; v < V; v += T) vst[v] = 0;
             // Duplicate keys (Sec. 4.4-4.5): equal local signatures in a shard are
             // the same key. Identical edges never peel, so every duplicate is in
             // the core, next to its copies in the incidence list of its first
@@ -383,19 +458,22 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // values agree; a key with two values has no solution at any seed
             // and ends the build (kErrDupKey). A copy that differs from the first
             // copy differs from the earlier copy it meets, so one comparison each
-            // finds every conflict.
+            // finds every conflict. Copies have the same vertices, hence equation
+            // words with the same XOR: only then are their signatures compared.
             for (uint32_t j = tid; j < C; j += T) {
-                const uint32_t e = __ldcg(&core[j]);
-                const uint64_t x = __ldg(a.loc + e0 + e);
-                const uint32_t v = __ldcg(&cev[3 * e]);
-                const uint32_t q1 = __ldcg(&inc_off[v + 1]);
-                for (uint32_t q = __ldcg(&inc_off[v]); q < q1; q++) {
-                    const uint32_t e2 = __ldcg(&core[__ldcg(&inc_list[q])]);
-                    if (e2 < e && __ldg(a.loc + e0 + e2) == x) {
+                const uint32_t w = est[j] >> 3;
+                const uint32_t e = core[j];
+                const uint32_t v = __ldcg(ev + e).x & 0xFFFFu;
+                const uint32_t q1 = off_of(v + 1);
+                for (uint32_t q = off_of(v); q < q1; q++) {
+                    const uint32_t j2 = ilist[q];
+                    if (j2 == j || (est[j2] >> 3) != w) continue;
+                    const uint32_t e2 = core[j2];
+                    if (e2 < e && __ldg(a.loc + e0 + e2) == __ldg(a.loc + e0 + e)) {
                         if (task.kind == 0 && __ldg(a.val + e0 + e2) != __ldg(a.val + e0 + e)) {
                             s_fail = 3;
                         } else {
-                            est[j] |= 4u;  // done: no equation of its own
+                            atomicOr(&est[j], 4u);  // done: no equation of its own
                             atomicAdd(&s_dup, 1u);
                         }
                         break;
@@ -411,43 +489,34 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 __syncthreads();
                 continue;
             }
-            // The incidence offsets (at most 3C) go to shared memory as 16-bit
-            // entries after the states when they fit: the elimination rounds then
-            // read only the incidence list itself from the slab.
-            uint16_t* ioff16 = nullptr;
-            if (in_smem && 3ull * C < 65536 && uint64_t(V) + C + (V + 2) / 2 <= kLgeSmemWords) {
-                ioff16 = reinterpret_cast<uint16_t*>(sm + V + C);
-                for (uint32_t v = tid; v <= V; v += T) ioff16[v] = uint16_t(__ldcg(&inc_off[v]));
-            }
-            auto off_of = [&](uint32_t v) -> uint32_t { return ioff16 ? uint32_t(ioff16[v]) : __ldcg(&inc_off[v]); };
             // The rest of shared memory holds the first qcap entries of the two
             // round queues; entries beyond stay in the slab's queues.
             uint32_t qcap = 0;
             uint32_t* sq0 = nullptr;
             if (in_smem) {
-                const uint32_t used = (V + C + (ioff16 ? (V + 2) / 2 : 0) + 3) & ~3u;
+                used = (used + 3) & ~3u;
                 qcap = used < kLgeSmemWords ? (kLgeSmemWords - used) / 2 : 0;
                 sq0 = sm + used;
             }
+            uint16_t* const gq = reinterpret_cast<uint16_t*>(scr + o.lists);
+            const uint32_t gq1 = 2 * ((a.v_cap + 1) / 2);
             auto qpush = [&](uint32_t q, uint32_t k) {
                 const uint32_t idx = atomicAdd(&s_cnt[q], 1u);
                 if (idx < qcap) sq0[q * qcap + idx] = k;
-                else fr[q][idx] = k;
+                else gq[(q ? gq1 : 0u) + idx] = uint16_t(k);
             };
-            auto qread = [&](uint32_t q, uint32_t i) -> uint32_t {
-                return i < qcap ? sq0[q * qcap + i] : __ldcg(&fr[q][i]);
-            };
+            auto qread = [&](uint32_t q, uint32_t i) -> uint32_t { return i < qcap ? sq0[q * qcap + i] : gq[(q ? gq1 : 0u) + i]; };
             // Removes variable u (now solved from equation `skip`, or active) from
             // every other open equation; an equation left with one idle variable
             // joins the next round's queue, one left with none joins the dense
             // system. Incidence entries are loaded four at a time, before any
-            // equation is touched, so their global loads overlap.
-            auto remove_var = [&](uint32_t u, uint32_t skip, uint32_t gq) {
+            // equation is touched, so their loads overlap.
+            auto remove_var = [&](uint32_t u, uint32_t skip, uint32_t gqi) {
                 const uint32_t q1 = off_of(u + 1);
                 for (uint32_t q = off_of(u); q < q1; q += 4) {
                     uint32_t ks[4];
 #pragma unroll
-                    for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? __ldcg(&inc_list[q + t]) : kNone;
+                    for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? uint32_t(ilist[q + t]) : kNone;
 #pragma unroll
                     for (uint32_t t = 0; t < 4; t++) {
                         const uint32_t k = ks[t];
@@ -456,7 +525,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                         atomicXor(&est[k], u << 3);
                         const uint32_t c = (old & 3u) - 1u;
                         if (c == 1u) {
-                            qpush(gq, k);
+                            qpush(gqi, k);
                         } else if (c == 0u) {
                             atomicOr(&est[k], 4u);
                             dense[atomicAdd(&s_D, 1u)] = k;
@@ -473,7 +542,6 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             }
             fi = 0;
             const uint32_t max_rounds = m + V + 2;
-            const unsigned lane = tid & 31u, warp = tid >> 5;
             __syncthreads();
             for (;;) {
                 if (s_rem == 0 || s_fail) break;
@@ -497,13 +565,13 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     bool elig = false;
                     uint32_t v = 0;
                     if (tid < wn) {
-                        v = __ldcg(&act[base + tid]);
+                        v = act[base + tid];
                         if (vst[v] == 0) {
                             const uint32_t q1 = off_of(v + 1);
                             for (uint32_t q = off_of(v); q < q1 && !elig; q += 4) {
                                 uint32_t ks[4];
 #pragma unroll
-                                for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? __ldcg(&inc_list[q + t]) : kNone;
+                                for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? uint32_t(ilist[q + t]) : kNone;
 #pragma unroll
                                 for (uint32_t t = 0; t < 4; t++) elig |= ks[t] != kNone && (est[ks[t]] & 4u) == 0;
                             }
@@ -512,18 +580,12 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     const unsigned bal = __ballot_sync(0xFFFFFFFFu, elig);
                     if (lane == 0) s_part[warp] = __popc(bal);
                     __syncthreads();
-                    if (tid == 0) {
-                        uint32_t run = 0;
-                        for (uint32_t w = 0; w < (T + 31) / 32; w++) {
-                            const uint32_t x = s_part[w];
-                            s_part[w] = run;
-                            run += x;
-                        }
-                        s_part[kLT - 1] = run;  // total eligible
+                    uint32_t rank = __popc(bal & ((1u << lane) - 1u)), tot = 0;
+                    for (uint32_t w = 0; w < kLT / 32; w++) {
+                        const uint32_t x = s_part[w];
+                        if (w < warp) rank += x;
+                        tot += x;
                     }
-                    __syncthreads();
-                    const uint32_t rank = s_part[warp] + __popc(bal & ((1u << lane) - 1u));
-                    const uint32_t tot = s_part[kLT - 1];
                     if (elig && rank < K) s_batch[rank] = v;
                     if (elig && rank == K - 1) s_nbatch = base + tid + 1;  // new scan position
                     __syncthreads();
@@ -588,150 +650,215 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 __syncthreads();
                 continue;
             }
-            // the affine rows and the dense system need shared memory: states go back to the slab
-            if (in_smem)
-                for (uint32_t v = tid; v < V; v += T) vstate[v] = vst[v];
+            A = s_A, S = s_S, D = s_D, R = s_r;
             __syncthreads();
-            const uint32_t A = s_A, S = s_S, D = s_D, R = s_r;
-            const uint32_t AW = (A + 31) / 32;
-            const uint32_t RS = AW | 1u;  // odd row stride: conflict-free shared-memory rows
-            // The dense system (rows, right-hand sides, pivot flags, column map) is
-            // solved in shared memory when it fits, else in the slab after the
-            // affine rows (large shards only; L2-resident, slower).
-            const uint64_t rows_off = (uint64_t(S) * AW + 3) & ~uint64_t(3);
-            const uint64_t dense_words = uint64_t(D) * RS + 2ull * D + A;
-            const bool dense_smem = dense_words <= kLgeSmemWords;
-            if (uint64_t(S) * AW > o.lpool || (!dense_smem && rows_off + dense_words > o.lpool)) {
-                if (tid == 0) {
-                    atomicOr(a.err, kErrLgeSize);
-                    atomicOr(a.item_fail + task.item, kErrLgeSize);
+        }
+        const uint32_t AW = (A + 31) / 32, DW = (D + 31) / 32;
+        const uint32_t RS = AW | 1u;  // odd row stride: conflict-free shared-memory rows
+        // The dense system: rows, then right-hand sides, panel words, combinations
+        // and pivot flags (a word per row each), the column map and a panel's
+        // pivot rows. In shared memory when it fits, else in the slab behind the
+        // column-major matrix (large shards only).
+        const uint64_t cm_words = (uint64_t(A) * DW + 3) & ~uint64_t(3);
+        const uint64_t rows_words = uint64_t(D) * RS;
+        const uint32_t small_words = 4 * D + A + 32 * AW;
+        if (small_words > kLgeSmemWords && spill_task(a, s)) {  // nothing of this shard has left the slab yet
+            __syncthreads();
+            continue;
+        }
+        if (uint64_t(S) * AW > o.lpool || cm_words + rows_words > o.lpool || small_words > kLgeSmemWords) {
+            if (tid == 0) {
+                atomicOr(a.err, kErrLgeSize);
+                atomicOr(a.item_fail + task.item, kErrLgeSize);
+            }
+            __syncthreads();
+            continue;
+        }
+        // ------------------------------------------------------ 4. dense system, values
+        // Shared memory: the solve records and the rounds' offsets when they fit
+        // beside the largest of what follows, then one region for the values (one
+        // word per variable) and the dense system in turn.
+        const uint32_t region = max(V, uint32_t(min(rows_words, uint64_t(kLgeSmemWords))) + small_words);
+        const uint32_t rec_words = (2 * S + 3) & ~3u, off_words = (R / 2 + 4) & ~3u;
+        const bool rec_smem = uint64_t(rec_words) + off_words + region <= kLgeSmemWords;
+        uint2* const rec = rec_smem ? reinterpret_cast<uint2*>(sm) : srec;
+        uint16_t* const off16 = rec_smem ? reinterpret_cast<uint16_t*>(sm + rec_words) : nullptr;
+        const uint32_t rb = rec_smem ? rec_words + off_words : 0;
+        uint32_t* const vx = rb + V <= kLgeSmemWords ? sm + rb : vstate;
+        auto round_off = [&](uint32_t r) -> uint32_t { return off16 ? uint32_t(off16[r]) : __ldcg(&soff[r]); };
+        // One record per solve, gathered for all solves at once: the variable, its
+        // equation's edge and the two other variables.
+        for (uint32_t si = tid; si < S; si += T) {
+            const uint32_t sv = __ldcg(&solves[si]);
+            const uint32_t x = sv & 0xFFFFu, e = core[sv >> 16];
+            const uint2 q = __ldcg(ev + e);
+            const uint32_t a0 = q.x & 0xFFFFu, a1 = q.x >> 16;
+            rec[si] = make_uint2(x | e << 16, (a0 == x ? a1 : a0) | (q.y == x ? a1 : q.y) << 16);
+        }
+        if (off16)
+            for (uint32_t r = tid; r <= R; r += T) off16[r] = uint16_t(__ldcg(&soff[r]));
+        __syncthreads();
+        // Values of the solved variables, round by round: vx[x] starts as its
+        // equation's right-hand side, the active variables as given.
+        auto forward = [&]() {
+            for (uint32_t r = 0; r < R; r++) {
+                const uint32_t lo = round_off(r), hi = round_off(r + 1);
+                if (hi == lo) continue;
+                for (uint32_t si = lo + tid; si < hi; si += T) {
+                    const uint2 q = rec[si];
+                    vx[q.x & 0xFFFFu] ^= vx[q.y & 0xFFFFu] ^ vx[q.y >> 16];
                 }
                 __syncthreads();
-                continue;
             }
-            prev_l = dense_smem ? uint64_t(S) * AW : rows_off + dense_words;
-            // One record per solve, gathered for all solves at once: the solved
-            // cell x, its equation's edge e, the two other cells and their states
-            // (final when x was solved: active, or solved in an earlier round). The
-            // rounds below then wait on two dependent loads instead of five.
-            // Shared memory is idle until the dense system is built: the affine
-            // rounds read the records from its top end when they fit, and so does
-            // the back-substitution if the dense system leaves them room.
-            uint4* const srs = 4ull * S <= kLgeSmemWords ? reinterpret_cast<uint4*>(sm + (kLgeSmemWords - 4 * S)) : nullptr;
+        };
+        if (D > 0) {
+            // constant terms: every active variable 0
+            for (uint32_t v = tid; v < V; v += T) vx[v] = 0;
+            __syncthreads();
             for (uint32_t si = tid; si < S; si += T) {
-                const uint32_t sv = __ldcg(&solves[si]);
-                const uint32_t x = sv & 0xFFFFu, e = __ldcg(&core[sv >> 16]);
-                const uint32_t c0 = __ldcg(&cev[3 * e]), c1 = __ldcg(&cev[3 * e + 1]), c2 = __ldcg(&cev[3 * e + 2]);
-                const uint32_t u1 = c0 == x ? c1 : c0, u2 = c2 == x ? c1 : c2;
-                const uint4 rec = make_uint4(x | (e << 16), u1 | (u2 << 16), __ldcg(&vstate[u1]), __ldcg(&vstate[u2]));
-                srec[si] = rec;
-                if (srs) srs[si] = rec;
+                const uint32_t q = rec[si].x;
+                vx[q & 0xFFFFu] = rhs_of(a, task, e0 + (q >> 16));
             }
             __syncthreads();
-            // the elimination's arrays are dead from here on (their lines are
-            // dropped instead of being written back when evicted)
-            discard_words(fr[0], V);
-            discard_words(fr[1], V);
-            discard_words(cand, V);
-            discard_words(inc_off, V + 1ull);
-            discard_words(inc_cur, V);
-            discard_words(inc_list, 3ull * m);
-            discard_words(act, V);
-            discard_words(eqst, m);
-            discard_words(solves, m);
-            // solved variables as affine functions of the active ones, round by round
-            for (uint32_t r = 0; r < R; r++) {
-                const uint32_t lo = __ldcg(&soff[r]), hi = __ldcg(&soff[r + 1]);
-                if (hi == lo) continue;
-                const uint32_t items = (hi - lo) * AW;
-                for (uint32_t it = tid; it < items; it += T) {
-                    const uint32_t si = lo + it / AW, w = it % AW;
-                    const uint4 q = srs ? srs[si] : __ldcg(&srec[si]);
-                    const uint32_t st[2] = {q.z, q.w};
-                    uint32_t acc = 0, c = 0;
-#pragma unroll
-                    for (int k = 0; k < 2; k++) {
-                        if ((st[k] & 3u) == 1u) {
-                            const uint32_t ai = st[k] >> 2;
-                            if ((ai >> 5) == w) acc ^= 1u << (ai & 31u);
-                        } else {
-                            acc ^= __ldcg(&L[uint64_t(st[k] >> 2) * AW + w]);
-                            if (w == 0) c ^= __ldcg(&lc[st[k] >> 2]);
+            forward();
+            for (uint32_t d = tid; d < D; d += T) {
+                const uint32_t e = core[__ldcg(&dense[d])];
+                const uint2 q = __ldcg(ev + e);
+                lc[d] = rhs_of(a, task, e0 + e) ^ vx[q.x & 0xFFFFu] ^ vx[q.x >> 16] ^ vx[q.y];
+            }
+            // Coefficients: 32 dense equations at a time are carried back through the
+            // solves in reverse order (bit d of vx[v]: equation d contains v): a
+            // solved variable's bits pass to the two others of its equation. What
+            // is left stands on active variables: a column of the system each.
+            // (Carrying the columns forward, one coefficient row per solve, takes
+            // as many bits per solve as there are active variables, 2.5 times the
+            // dense equations, and the rows do not fit in shared memory.)
+            for (uint32_t w = 0; w < DW; w++) {
+                __syncthreads();
+                for (uint32_t v = tid; v < V; v += T) vx[v] = 0;
+                __syncthreads();
+                if (tid < 32 && 32 * w + tid < D) {
+                    const uint2 q = __ldcg(ev + core[__ldcg(&dense[32 * w + tid])]);
+                    atomicXor(&vx[q.x & 0xFFFFu], 1u << tid);
+                    atomicXor(&vx[q.x >> 16], 1u << tid);
+                    atomicXor(&vx[q.y], 1u << tid);
+                }
+                __syncthreads();
+                for (uint32_t r = R; r-- > 0;) {
+                    const uint32_t lo = round_off(r), hi = round_off(r + 1);
+                    if (hi == lo) continue;
+                    for (uint32_t si = lo + tid; si < hi; si += T) {
+                        const uint2 q = rec[si];
+                        const uint32_t c = vx[q.x & 0xFFFFu];
+                        if (c) {
+                            atomicXor(&vx[q.y & 0xFFFFu], c);
+                            atomicXor(&vx[q.y >> 16], c);
                         }
                     }
-                    L[uint64_t(si) * AW + w] = acc;
-                    if (w == 0) lc[si] = c ^ rhs_of(a, task, e0 + (q.x >> 16));
+                    __syncthreads();
                 }
-                __syncthreads();
+                for (uint32_t c = tid; c < A; c += T) L[uint64_t(w) * A + c] = vx[__ldcg(&actv[c])];
             }
-            uint32_t* rows = dense_smem ? sm : L + rows_off;
-            uint32_t* rhs = rows + uint64_t(D) * RS;
-            uint32_t* pivf = rhs + D;
-            uint32_t* colrow = pivf + D;
-            for (uint32_t it = tid; it < D * AW; it += T) {
-                const uint32_t d = it / AW, w = it % AW;
-                const uint32_t e = __ldcg(&core[__ldcg(&dense[d])]);
-                uint32_t acc = 0, c = 0;
+            __syncthreads();
+            const bool rows_smem = rb + rows_words + small_words <= kLgeSmemWords;
+            uint32_t* const small = sm + rb;
+            uint32_t* const rhs = small;
+            uint32_t* const pan = rhs + D;    // a panel's word of each row
+            uint32_t* const comb = pan + D;   // the panel's pivot rows to add to each row
+            uint32_t* const pivf = comb + D;
+            uint32_t* const colrow = pivf + D;
+            uint32_t* const pbuf = colrow + A;  // pivot rows as the panel found them: 32 rows of AW words
+            uint32_t* const rows = rows_smem ? small + small_words : L + cm_words;
+            if (!rows_smem) prev_l = cm_words + rows_words;
+            else prev_l = cm_words;
+            // rows from columns: a warp turns 32 columns x 32 rows with ballots
+            for (uint32_t blk = warp; blk < AW * DW; blk += kLT / 32) {
+                const uint32_t cw = blk / DW, w = blk % DW;
+                const uint32_t c = 32 * cw + lane;
+                const uint32_t bits = c < A ? __ldcg(&L[uint64_t(w) * A + c]) : 0u;
+                uint32_t mine = 0;
 #pragma unroll
-                for (int k = 0; k < 3; k++) {
-                    uint32_t st = __ldcg(&vstate[__ldcg(&cev[3 * e + k])]);
-                    if ((st & 3u) == 1u) {
-                        uint32_t ai = st >> 2;
-                        if ((ai >> 5) == w) acc ^= 1u << (ai & 31u);
-                    } else {
-                        acc ^= __ldcg(&L[uint64_t(st >> 2) * AW + w]);
-                        c ^= __ldcg(&lc[st >> 2]);
-                    }
+                for (uint32_t d = 0; d < 32; d++) {
+                    const uint32_t row = __ballot_sync(0xFFFFFFFFu, (bits >> d) & 1u);
+                    if (lane == d) mine = row;
                 }
-                rows[d * RS + w] = acc;
-                if (w == 0) {
-                    rhs[d] = c ^ rhs_of(a, task, e0 + e);
-                    pivf[d] = 0;
-                }
+                if (32 * w + lane < D) rows[uint64_t(32 * w + lane) * RS + cw] = mine;
+            }
+            for (uint32_t d = tid; d < D; d += T) {
+                rhs[d] = __ldcg(&lc[d]);
+                pivf[d] = 0;
             }
             for (uint32_t c = tid; c < A; c += T) colrow[c] = kNone;
             __syncthreads();
-            // the affine rows (and what built the dense rows) are dead now
-            discard_words(L, uint64_t(S) * AW);
-            discard_words(lc, S);
-            discard_words(core, m);
-            discard_words(dense, m);
-            discard_words(vstate, V);
-            // Gauss-Jordan over GF(2): pivot = lowest unused row with the column bit
-            // once every row is a pivot no later column can have one (its active
-            // variable stays free, 0): the loop ends there
-            for (uint32_t col = 0, npiv = 0; col < A && npiv < D; col++) {
-                const uint32_t cw = col >> 5, cb = 1u << (col & 31u);
-                if (tid == 0) s_piv = kNone;
-                __syncthreads();
-                for (uint32_t d = tid; d < D; d += T)
-                    if (!pivf[d] && (rows[d * RS + cw] & cb)) atomicMin(&s_piv, d);
-                __syncthreads();
-                const uint32_t p = s_piv;
-                if (p == kNone) {
-                    __syncthreads();
-                    continue;
-                }
+            // Gauss-Jordan over GF(2), a word of columns (a panel) at a time; pivot =
+            // lowest unused row with the column bit. Within the panel only its word
+            // of each row is kept up to date, one barrier per column, and which of
+            // the panel's pivot rows, as they were before the panel, each row has
+            // to take up; the rest of every row is brought up to date once per
+            // panel. Once every row is a pivot no later column can have one (its
+            // active variable stays free, 0): the loop ends there.
+            uint32_t npiv = 0, step = 0;
+            for (uint32_t cw = 0; cw < AW && npiv < D; cw++) {
                 for (uint32_t d = tid; d < D; d += T) {
-                    if (d == p || !(rows[d * RS + cw] & cb)) continue;
-                    // rows d and p never alias: four words of each are loaded
-                    // before any is stored, so the round trips overlap
-                    uint32_t* rd = rows + d * RS;
-                    const uint32_t* rp = rows + p * RS;
-                    uint32_t w = cw;
-                    for (; w + 4 <= AW; w += 4) {
-                        const uint32_t a0 = rd[w], a1 = rd[w + 1], a2 = rd[w + 2], a3 = rd[w + 3];
-                        const uint32_t b0 = rp[w], b1 = rp[w + 1], b2 = rp[w + 2], b3 = rp[w + 3];
-                        rd[w] = a0 ^ b0, rd[w + 1] = a1 ^ b1, rd[w + 2] = a2 ^ b2, rd[w + 3] = a3 ^ b3;
+                    pan[d] = rows[uint64_t(d) * RS + cw];
+                    comb[d] = 0;
+                }
+                uint32_t k = 0;  // the panel's pivots so far
+                const uint32_t cols = min(32u, A - 32 * cw);
+                for (uint32_t c = 0; c < cols && npiv + k < D; c++, step++) {
+                    uint32_t best = kNone;  // this thread's rows are its own until the barrier
+                    for (uint32_t d = tid; d < D && best == kNone; d += T)
+                        if (!pivf[d] && ((pan[d] >> c) & 1u)) best = d;
+                    best = __reduce_min_sync(0xFFFFFFFFu, best);
+                    if (lane == 0) s_cand[step & 1u][warp] = best;
+                    __syncthreads();
+                    uint32_t p = kNone;
+#pragma unroll
+                    for (uint32_t w = 0; w < kLT / 32; w++) p = min(p, s_cand[step & 1u][w]);
+                    if (p == kNone) continue;
+                    const uint32_t pw2 = pan[p], pc = comb[p] ^ (1u << k);
+                    for (uint32_t d = tid; d < D; d += T) {
+                        if (d == p) {
+                            pivf[d] = 1;
+                            s_piv[k] = p;
+                            colrow[32 * cw + c] = p;
+                        } else if ((pan[d] >> c) & 1u) {
+                            pan[d] ^= pw2;
+                            comb[d] ^= pc;
+                        }
                     }
-                    for (; w < AW; w++) rd[w] ^= rp[w];
-                    rhs[d] ^= rhs[p];
+                    k++;
                 }
-                if (tid == 0) {
-                    pivf[p] = 1;
-                    colrow[col] = p;
+                npiv += k;
+                __syncthreads();
+                const uint32_t w0 = cw + 1, wn = AW - w0;  // words still to be brought up to date
+                for (uint32_t i = tid; i < k * (wn + 1); i += T) {
+                    const uint32_t j = i / (wn + 1), w = i % (wn + 1);
+                    pbuf[j * AW + w] = w < wn ? rows[uint64_t(s_piv[j]) * RS + w0 + w] : rhs[s_piv[j]];
                 }
-                npiv++;
+                __syncthreads();
+                const uint32_t quads = (wn + 1 + 3) / 4;
+                for (uint32_t i = tid; i < D * quads; i += T) {
+                    const uint32_t d = i % D, q = i / D;
+                    uint32_t c = comb[d];
+                    if (!c) continue;
+                    uint32_t x0 = 0, x1 = 0, x2 = 0, x3 = 0;
+                    const uint32_t* pb = pbuf + 4 * q;
+                    for (uint32_t j = 0; j < k; j++, pb += AW) {
+                        const uint32_t f = 0u - ((c >> j) & 1u);
+                        x0 ^= f & pb[0];
+                        if (4 * q + 1 <= wn) x1 ^= f & pb[1];
+                        if (4 * q + 2 <= wn) x2 ^= f & pb[2];
+                        if (4 * q + 3 <= wn) x3 ^= f & pb[3];
+                    }
+                    uint32_t* row = rows + uint64_t(d) * RS + w0 + 4 * q;
+                    const uint32_t xs[4] = {x0, x1, x2, x3};
+#pragma unroll
+                    for (uint32_t t = 0; t < 4; t++) {
+                        if (4 * q + t < wn) row[t] ^= xs[t];
+                        else if (4 * q + t == wn) rhs[d] ^= xs[t];
+                    }
+                }
                 __syncthreads();
             }
             for (uint32_t d = tid; d < D; d += T)
@@ -745,39 +872,36 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 __syncthreads();
                 continue;
             }
-            for (uint32_t c = tid; c < A; c += T)
-                cell_put_zero(data, b, cbase + __ldcg(&actv[c]), colrow[c] != kNone ? rhs[colrow[c]] : 0u);
+            // the active variables' values leave the region before the values enter it
+            for (uint32_t c = tid; c < A; c += T) lc[c] = colrow[c] != kNone ? rhs[colrow[c]] : 0u;
             __syncthreads();
-            const uint4* const srs_bs =
-                srs && (!dense_smem || dense_words + 4ull * S <= kLgeSmemWords) ? srs : nullptr;
-            // solved variables, in solve order (their equations as generated)
-            for (uint32_t r = 0; r < R; r++) {
-                const uint32_t lo = __ldcg(&soff[r]), hi = __ldcg(&soff[r + 1]);
-                if (hi == lo) continue;
-                for (uint32_t si = lo + tid; si < hi; si += T) {
-                    const uint4 q = srs_bs ? srs_bs[si] : __ldcg(&srec[si]);
-                    const uint32_t val = rhs_of(a, task, e0 + (q.x >> 16)) ^ cell_get_cg(data, b, cbase + (q.y & 0xFFFFu)) ^
-                                         cell_get_cg(data, b, cbase + (q.y >> 16));
-                    cell_put_zero(data, b, cbase + (q.x & 0xFFFFu), val);
-                }
-                __syncthreads();
-            }
         }
-
-        // -------------------------------------------- 4. reverse peel-order assignment
+        // Values of every variable: active, solved in solve order, then the peeled
+        // edges' vertices in reverse peel order.
+        for (uint32_t v = tid; v < V; v += T) vx[v] = 0;
+        __syncthreads();
+        if (D > 0)
+            for (uint32_t c = tid; c < A; c += T) vx[__ldcg(&actv[c])] = __ldcg(&lc[c]);
+        for (uint32_t si = tid; si < S; si += T) {
+            const uint32_t q = rec[si].x;
+            vx[q & 0xFFFFu] = rhs_of(a, task, e0 + (q >> 16));
+        }
+        for (uint32_t i = tid; i < peeled; i += T) {
+            const uint32_t q = __ldcg(prec + i).x;
+            vx[q & 0xFFFFu] = rhs_of(a, task, e0 + (q >> 16));
+        }
+        __syncthreads();
+        forward();
         for (uint32_t r = prounds; r-- > 0;) {
             const uint32_t lo = __ldcg(&proff[r]), hi = __ldcg(&proff[r + 1]);
             for (uint32_t i = lo + tid; i < hi; i += T) {
-                const uint32_t ent = __ldcg(&porder[i]);
-                const uint32_t e = ent >> 2, side = ent & 3u;
-                uint32_t val = rhs_of(a, task, e0 + e);
-#pragma unroll
-                for (uint32_t k = 0; k < 3; k++)
-                    if (k != side) val ^= cell_get_cg(data, b, cbase + __ldcg(&cev[3 * e + k]));
-                cell_put_zero(data, b, cbase + __ldcg(&cev[3 * e + side]), val);
+                const uint2 q = __ldcg(prec + i);
+                vx[q.x & 0xFFFFu] ^= vx[q.y & 0xFFFFu] ^ vx[q.y >> 16];
             }
             __syncthreads();
         }
+        const uint32_t vmask = b == 32 ? 0xFFFFFFFFu : ((1u << b) - 1u);
+        for (uint32_t v = tid; v < V; v += T) cell_put_zero(data, b, cbase + v, vx[v] & vmask);
         if (tid == 0) {
             atomicAdd(&a.stats[0], peeled);
             atomicAdd(&a.stats[1], C - s_dup);
