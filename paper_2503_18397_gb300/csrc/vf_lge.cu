@@ -34,6 +34,7 @@
 // error that ends the build rather than a retry.
 #include <algorithm>
 #include <atomic>
+#include <cstdlib>
 
 #include "vf_internal.h"
 
@@ -166,8 +167,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     __shared__ uint32_t s_hist[256];
     __shared__ uint32_t s_batch[kMaxBatch];
     __shared__ uint32_t s_part[kLT];
-    __shared__ __align__(16) uint32_t s_cand[2][kLT / 32 + 2];  // pivot candidates, one per warp
-    __shared__ uint32_t s_piv[32];                               // pivot rows of a panel
+    __shared__ uint4 s_piv[32];    // a panel's pivots: row, reduced panel word, combination with itself, column
+    __shared__ uint32_t s_pool[64];  // the rows it is looked for in
 
     const uint32_t tid = threadIdx.x, T = blockDim.x;
     const unsigned lane = tid & 31u, warp = tid >> 5;
@@ -189,6 +190,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     uint32_t* dense = scr + o.dense;
     uint32_t* lc = scr + o.lc;
     uint32_t* L = scr + o.L;
+    // the small configurations hand on a shard whose arrays do not all fit
+    constexpr bool kSpills = kLgeSmemWords != kBigWords;
     constexpr uint32_t kBad = kErrUnsolvable | kErrCapacity | kErrLgeSize | kErrDegOverflow | kErrDupKey;
 
     // The large configuration behind a small one takes its tasks from the
@@ -254,7 +257,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         uint32_t* xrw = degw + (V + 3) / 4;
         uint32_t* clm = xrw + (V + 1) / 2;
         const uint32_t pw = (V + 3) / 4 + (V + 1) / 2 + (m + 31) / 32;
-        if (pw > kLgeSmemWords) {
+        // (or of one whose solve records, ~0.6 a key, will not fit beside its values)
+        if (pw > kLgeSmemWords || (kSpills && V + 6u * m / 5u > kLgeSmemWords && a.spill)) {
             if (!spill_task(a, s) && tid == 0) {
                 atomicOr(a.err, kErrCapacity);
                 atomicOr(a.item_fail + task.item, kErrCapacity);
@@ -368,19 +372,38 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // fit (the peel's arrays are dead now); otherwise they stay in the slab.
             // Equation word: bits 0-1 idle count, bit 2 done, bits 3.. XOR of its idle variables.
             const bool in_smem = uint64_t(V) + C <= kLgeSmemWords;
-            uint32_t* vst = in_smem ? sm : vstate;  // first the core degrees, then the list cursors
-            uint32_t* est = in_smem ? sm + V : eqst;
+            if (kSpills && !in_smem && spill_task(a, s)) {
+                __syncthreads();
+                continue;
+            }
+            // core equations with their vertices, four loads of a thread in flight
+            auto for_core = [&](auto&& f) {
+                for (uint32_t j0 = tid; j0 < C; j0 += 4 * T) {
+                    uint32_t e[4];
+                    uint2 x[4];
+#pragma unroll
+                    for (uint32_t t = 0; t < 4; t++) e[t] = j0 + t * T < C ? core[j0 + t * T] : 0u;
+#pragma unroll
+                    for (uint32_t t = 0; t < 4; t++) x[t] = __ldcg(ev + e[t]);
+#pragma unroll
+                    for (uint32_t t = 0; t < 4; t++)
+                        if (j0 + t * T < C) f(j0 + t * T, x[t]);
+                }
+            };
+            // vst: first the core degrees, then the list cursors, then the variable
+            // states. Written for both places they may be in (the compiler then
+            // uses shared-memory instructions for the usual one).
+            auto eliminate_all = [&](uint32_t* const vst, uint32_t* const est) {
             for (uint32_t v = tid; v < V; v += T) vst[v] = 0;
             for (uint32_t i = tid; i < 256; i += T) s_hist[i] = 0;
             __syncthreads();
-            for (uint32_t j = tid; j < C; j += T) {
-                const uint2 x = __ldcg(ev + core[j]);
+            for_core([&](uint32_t j, uint2 x) {
                 const uint32_t v0 = x.x & 0xFFFFu, v1 = x.x >> 16, v2 = x.y;
                 atomicAdd(&vst[v0], 1u);
                 atomicAdd(&vst[v1], 1u);
                 atomicAdd(&vst[v2], 1u);
                 est[j] = ((v0 ^ v1 ^ v2) << 3) | 3u;
-            }
+            });
             __syncthreads();
             // activation order: core degree, heaviest first (counting sort)
             for (uint32_t v0 = tid & ~31u; v0 < V; v0 += T) {
@@ -441,12 +464,11 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 if (tid == 0) inc_off[V] = 3 * C;
             }
             __syncthreads();
-            for (uint32_t j = tid; j < C; j += T) {
-                const uint2 x = __ldcg(ev + core[j]);
+            for_core([&](uint32_t j, uint2 x) {
                 ilist[atomicAdd(&vst[x.x & 0xFFFFu], 1u)] = uint16_t(j);
                 ilist[atomicAdd(&vst[x.x >> 16], 1u)] = uint16_t(j);
                 ilist[atomicAdd(&vst[x.y], 1u)] = uint16_t(j);
-            }
+            });
             auto off_of = [&](uint32_t v) -> uint32_t { return ioff16 ? uint32_t(ioff16[v]) : __ldcg(&inc_off[v]); };
             __syncthreads();
             for (uint32_t v = tid; v < V; v += T) vst[v] = 0;
@@ -460,15 +482,13 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // copy differs from the earlier copy it meets, so one comparison each
             // finds every conflict. Copies have the same vertices, hence equation
             // words with the same XOR: only then are their signatures compared.
-            for (uint32_t j = tid; j < C; j += T) {
-                const uint32_t w = est[j] >> 3;
-                const uint32_t e = core[j];
-                const uint32_t v = __ldcg(ev + e).x & 0xFFFFu;
+            for_core([&](uint32_t j, uint2 x) {
+                const uint32_t v = x.x & 0xFFFFu, w = est[j] >> 3;
                 const uint32_t q1 = off_of(v + 1);
                 for (uint32_t q = off_of(v); q < q1; q++) {
                     const uint32_t j2 = ilist[q];
                     if (j2 == j || (est[j2] >> 3) != w) continue;
-                    const uint32_t e2 = core[j2];
+                    const uint32_t e = core[j], e2 = core[j2];
                     if (e2 < e && __ldg(a.loc + e0 + e2) == __ldg(a.loc + e0 + e)) {
                         if (task.kind == 0 && __ldg(a.val + e0 + e2) != __ldg(a.val + e0 + e)) {
                             s_fail = 3;
@@ -479,16 +499,9 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                         break;
                     }
                 }
-            }
+            });
             __syncthreads();
-            if (s_fail == 3) {
-                if (tid == 0) {
-                    atomicOr(a.err, kErrDupKey);
-                    atomicOr(a.item_fail + task.item, kErrDupKey);
-                }
-                __syncthreads();
-                continue;
-            }
+            if (s_fail == 3) return;
             // The rest of shared memory holds the first qcap entries of the two
             // round queues; entries beyond stay in the slab's queues.
             uint32_t qcap = 0;
@@ -642,10 +655,14 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 fi ^= 1;
                 __syncthreads();
             }
+            };
+            if (kSpills || in_smem) eliminate_all(sm, sm + V);
+            else eliminate_all(vstate, eqst);
             if (s_fail) {
+                const uint32_t bad = s_fail == 3 ? kErrDupKey : kErrLgeSize;
                 if (tid == 0) {
-                    atomicOr(a.err, kErrLgeSize);
-                    atomicOr(a.item_fail + task.item, kErrLgeSize);
+                    atomicOr(a.err, bad);
+                    atomicOr(a.item_fail + task.item, bad);
                 }
                 __syncthreads();
                 continue;
@@ -656,12 +673,14 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         const uint32_t AW = (A + 31) / 32, DW = (D + 31) / 32;
         const uint32_t RS = AW | 1u;  // odd row stride: conflict-free shared-memory rows
         // The dense system: rows, then right-hand sides, panel words, combinations
-        // and pivot flags (a word per row each), the column map and a panel's
-        // pivot rows. In shared memory when it fits, else in the slab behind the
-        // column-major matrix (large shards only).
+        // and pivot flags (a word per row each), the column map, a panel's pivot
+        // rows and their sums in fours. In shared memory when it fits, else its
+        // rows are in the slab behind the column-major matrix (large shards only).
         const uint64_t cm_words = (uint64_t(A) * DW + 3) & ~uint64_t(3);
         const uint64_t rows_words = uint64_t(D) * RS;
-        const uint32_t small_words = 4 * D + A + 32 * AW;
+        const uint32_t PS = (AW + 3) & ~3u;  // stride of a panel's pivot rows
+        const uint32_t flat_words = (4 * D + A + 3u) & ~3u;
+        const uint32_t small_words = flat_words + (32 + 128) * PS;
         if (small_words > kLgeSmemWords && spill_task(a, s)) {  // nothing of this shard has left the slab yet
             __syncthreads();
             continue;
@@ -675,17 +694,17 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             continue;
         }
         // ------------------------------------------------------ 4. dense system, values
-        // Shared memory: the solve records and the rounds' offsets when they fit
-        // beside the largest of what follows, then one region for the values (one
-        // word per variable) and the dense system in turn.
-        const uint32_t region = max(V, uint32_t(min(rows_words, uint64_t(kLgeSmemWords))) + small_words);
+        // Shared memory holds the solve records, the rounds' offsets and one word
+        // per variable when they fit; the dense system takes their place in between.
         const uint32_t rec_words = (2 * S + 3) & ~3u, off_words = (R / 2 + 4) & ~3u;
-        const bool rec_smem = uint64_t(rec_words) + off_words + region <= kLgeSmemWords;
-        uint2* const rec = rec_smem ? reinterpret_cast<uint2*>(sm) : srec;
-        uint16_t* const off16 = rec_smem ? reinterpret_cast<uint16_t*>(sm + rec_words) : nullptr;
-        const uint32_t rb = rec_smem ? rec_words + off_words : 0;
-        uint32_t* const vx = rb + V <= kLgeSmemWords ? sm + rb : vstate;
-        auto round_off = [&](uint32_t r) -> uint32_t { return off16 ? uint32_t(off16[r]) : __ldcg(&soff[r]); };
+        const uint32_t rb = rec_words + off_words;
+        const bool rec_smem = uint64_t(rb) + V <= kLgeSmemWords;
+        const bool rows_smem = rows_words + small_words <= kLgeSmemWords;
+        if (kSpills && !(rec_smem && rows_smem) && spill_task(a, s)) {  // nothing of this shard has left the slab yet
+            __syncthreads();
+            continue;
+        }
+        uint16_t* const off16 = reinterpret_cast<uint16_t*>(sm + rec_words);
         // One record per solve, gathered for all solves at once: the variable, its
         // equation's edge and the two other variables.
         for (uint32_t si = tid; si < S; si += T) {
@@ -693,24 +712,56 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             const uint32_t x = sv & 0xFFFFu, e = core[sv >> 16];
             const uint2 q = __ldcg(ev + e);
             const uint32_t a0 = q.x & 0xFFFFu, a1 = q.x >> 16;
-            rec[si] = make_uint2(x | e << 16, (a0 == x ? a1 : a0) | (q.y == x ? a1 : q.y) << 16);
+            srec[si] = make_uint2(x | e << 16, (a0 == x ? a1 : a0) | (q.y == x ? a1 : q.y) << 16);
         }
-        if (off16)
-            for (uint32_t r = tid; r <= R; r += T) off16[r] = uint16_t(__ldcg(&soff[r]));
         __syncthreads();
-        // Values of the solved variables, round by round: vx[x] starts as its
-        // equation's right-hand side, the active variables as given.
-        auto forward = [&]() {
-            for (uint32_t r = 0; r < R; r++) {
-                const uint32_t lo = round_off(r), hi = round_off(r + 1);
-                if (hi == lo) continue;
-                for (uint32_t si = lo + tid; si < hi; si += T) {
-                    const uint2 q = rec[si];
-                    vx[q.x & 0xFFFFu] ^= vx[q.y & 0xFFFFu] ^ vx[q.y >> 16];
+        // Written for every place its arrays may be in, as the elimination.
+        // false: the system has no solution.
+        auto solve_all = [&](uint32_t* const vx, uint2* const rec, auto&& round_off, uint32_t* const rows) -> bool {
+        auto load_records = [&]() {
+            if (!rec_smem) return;
+            for (uint32_t si = tid; si < S; si += T) rec[si] = __ldcg(srec + si);
+            for (uint32_t r = tid; r <= R; r += T) off16[r] = uint16_t(__ldcg(&soff[r]));
+        };
+        // The rounds of solves from `first` in steps of `dir`, a barrier behind each.
+        // A round is short (some 60 solves), so its latency counts: the next
+        // round's offsets and records are read before this one's barrier.
+        auto walk = [&](bool back, auto&& f) {
+            uint32_t lo = 0, hi = 0, r = back ? R : 0;
+            uint2 q = make_uint2(0, 0);
+            auto next = [&](uint32_t& nlo, uint32_t& nhi, uint2& nq) {
+                nlo = nhi = 0;
+                while (back ? r > 0 : r < R) {
+                    if (back) r--;
+                    nlo = round_off(r), nhi = round_off(r + 1);
+                    if (!back) r++;
+                    if (nhi > nlo) break;
+                }
+                if (nlo + tid < nhi) nq = rec[nlo + tid];
+            };
+            next(lo, hi, q);
+            while (hi > lo) {
+                uint32_t nlo, nhi;
+                uint2 nq = make_uint2(0, 0);
+                const bool on = lo + tid < hi;
+                const uint32_t c = on ? vx[q.x & 0xFFFFu] : 0u;
+                next(nlo, nhi, nq);
+                if (on) f(q, c);
+                for (uint32_t si = lo + tid + T; si < hi; si += T) {
+                    const uint2 x = rec[si];
+                    f(x, vx[x.x & 0xFFFFu]);
                 }
                 __syncthreads();
+                lo = nlo, hi = nhi, q = nq;
             }
         };
+        // Values of the solved variables: vx[x] starts as its equation's
+        // right-hand side, the active variables as given.
+        auto forward = [&]() {
+            walk(false, [&](uint2 q, uint32_t c) { vx[q.x & 0xFFFFu] = c ^ vx[q.y & 0xFFFFu] ^ vx[q.y >> 16]; });
+        };
+        load_records();
+        __syncthreads();
         if (D > 0) {
             // constant terms: every active variable 0
             for (uint32_t v = tid; v < V; v += T) vx[v] = 0;
@@ -744,33 +795,23 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     atomicXor(&vx[q.y], 1u << tid);
                 }
                 __syncthreads();
-                for (uint32_t r = R; r-- > 0;) {
-                    const uint32_t lo = round_off(r), hi = round_off(r + 1);
-                    if (hi == lo) continue;
-                    for (uint32_t si = lo + tid; si < hi; si += T) {
-                        const uint2 q = rec[si];
-                        const uint32_t c = vx[q.x & 0xFFFFu];
-                        if (c) {
-                            atomicXor(&vx[q.y & 0xFFFFu], c);
-                            atomicXor(&vx[q.y >> 16], c);
-                        }
+                walk(true, [&](uint2 q, uint32_t c) {
+                    if (c) {
+                        atomicXor(&vx[q.y & 0xFFFFu], c);
+                        atomicXor(&vx[q.y >> 16], c);
                     }
-                    __syncthreads();
-                }
+                });
                 for (uint32_t c = tid; c < A; c += T) L[uint64_t(w) * A + c] = vx[__ldcg(&actv[c])];
             }
             __syncthreads();
-            const bool rows_smem = rb + rows_words + small_words <= kLgeSmemWords;
-            uint32_t* const small = sm + rb;
+            uint32_t* const small = sm;
             uint32_t* const rhs = small;
             uint32_t* const pan = rhs + D;    // a panel's word of each row
             uint32_t* const comb = pan + D;   // the panel's pivot rows to add to each row
             uint32_t* const pivf = comb + D;
             uint32_t* const colrow = pivf + D;
-            uint32_t* const pbuf = colrow + A;  // pivot rows as the panel found them: 32 rows of AW words
-            uint32_t* const rows = rows_smem ? small + small_words : L + cm_words;
-            if (!rows_smem) prev_l = cm_words + rows_words;
-            else prev_l = cm_words;
+            uint32_t* const pbuf = small + flat_words;  // pivot rows as the panel found them
+            uint32_t* const tab = pbuf + 32 * PS;       // every sum of pivot rows 4g .. 4g + 3, 16 each
             // rows from columns: a warp turns 32 columns x 32 rows with ballots
             for (uint32_t blk = warp; blk < AW * DW; blk += kLT / 32) {
                 const uint32_t cw = blk / DW, w = blk % DW;
@@ -790,91 +831,135 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             }
             for (uint32_t c = tid; c < A; c += T) colrow[c] = kNone;
             __syncthreads();
-            // Gauss-Jordan over GF(2), a word of columns (a panel) at a time; pivot =
-            // lowest unused row with the column bit. Within the panel only its word
-            // of each row is kept up to date, one barrier per column, and which of
-            // the panel's pivot rows, as they were before the panel, each row has
-            // to take up; the rest of every row is brought up to date once per
-            // panel. Once every row is a pivot no later column can have one (its
-            // active variable stays free, 0): the loop ends there.
-            uint32_t npiv = 0, step = 0;
+            // Gauss-Jordan over GF(2), a word of columns (a panel) at a time. One warp
+            // reduces the panel's words of 64 unused rows in registers, two a lane,
+            // and finds up to 32 pivots with no barrier (64 random rows hardly ever
+            // lack one for a column); what every other row has to take up then
+            // follows from its own panel word, and the rest of every row is brought
+            // up to date once, from the sums of the pivot rows in fours. Columns
+            // the 64 rows had no pivot for are looked at again with the rows that
+            // still have bits in them. Once every row is a pivot no later column
+            // can have one (its active variable stays free, 0): the loop ends there.
+            uint32_t npiv = 0;
             for (uint32_t cw = 0; cw < AW && npiv < D; cw++) {
-                for (uint32_t d = tid; d < D; d += T) {
-                    pan[d] = rows[uint64_t(d) * RS + cw];
-                    comb[d] = 0;
-                }
-                uint32_t k = 0;  // the panel's pivots so far
-                const uint32_t cols = min(32u, A - 32 * cw);
-                for (uint32_t c = 0; c < cols && npiv + k < D; c++, step++) {
-                    uint32_t best = kNone;  // this thread's rows are its own until the barrier
-                    for (uint32_t d = tid; d < D && best == kNone; d += T)
-                        if (!pivf[d] && ((pan[d] >> c) & 1u)) best = d;
-                    best = __reduce_min_sync(0xFFFFFFFFu, best);
-                    if (lane == 0) s_cand[step & 1u][warp] = best;
+                for (uint32_t d = tid; d < D; d += T) pan[d] = rows[uint64_t(d) * RS + cw];
+                const uint32_t w0 = cw + 1, wn = AW - w0;  // words behind the panel
+                for (;;) {
+                    if (tid == 0) s_cnt[0] = 0;
                     __syncthreads();
-                    uint32_t p = kNone;
+                    for (uint32_t d0 = tid & ~31u; d0 < D; d0 += T) {
+                        const uint32_t d = d0 + lane;
+                        const bool cand = d < D && !pivf[d] && pan[d];
+                        const uint32_t at = warp_slot(&s_cnt[0], cand);
+                        if (cand && at < 64) s_pool[at] = d;
+                    }
+                    __syncthreads();
+                    const uint32_t np = min(s_cnt[0], 64u);
+                    if (np == 0) break;
+                    if (warp == 0) {
+                        uint32_t row[2], x[2], y[2] = {0, 0}, mine[2] = {kNone, kNone};
 #pragma unroll
-                    for (uint32_t w = 0; w < kLT / 32; w++) p = min(p, s_cand[step & 1u][w]);
-                    if (p == kNone) continue;
-                    const uint32_t pw2 = pan[p], pc = comb[p] ^ (1u << k);
+                        for (int t = 0; t < 2; t++) {
+                            const uint32_t i = lane + 32 * t;
+                            row[t] = i < np ? s_pool[i] : kNone;
+                            x[t] = i < np ? pan[row[t]] : 0u;
+                        }
+                        uint32_t k = 0;
+                        for (uint32_t c = 0; c < 32; c++) {
+                            const unsigned h0 = __ballot_sync(0xFFFFFFFFu, mine[0] == kNone && ((x[0] >> c) & 1u));
+                            const unsigned h1 = __ballot_sync(0xFFFFFFFFu, mine[1] == kNone && ((x[1] >> c) & 1u));
+                            if (!(h0 | h1)) continue;
+                            const int p = __ffs(h0 ? h0 : h1) - 1;
+                            const uint32_t px = __shfl_sync(0xFFFFFFFFu, h0 ? x[0] : x[1], p);
+                            const uint32_t py = __shfl_sync(0xFFFFFFFFu, h0 ? y[0] : y[1], p) ^ (1u << k);
+#pragma unroll
+                            for (int t = 0; t < 2; t++) {
+                                if (int(lane) == p && (t == 0) == (h0 != 0)) {
+                                    mine[t] = k | (c << 8);
+                                } else if ((x[t] >> c) & 1u) {
+                                    x[t] ^= px;
+                                    y[t] ^= py;
+                                }
+                            }
+                            k++;
+                        }
+#pragma unroll
+                        for (int t = 0; t < 2; t++)
+                            if (mine[t] != kNone) {
+                                const uint32_t j = mine[t] & 255u, c = mine[t] >> 8;
+                                s_piv[j] = make_uint4(row[t], x[t], y[t] ^ (1u << j), c);
+                                pivf[row[t]] = 2u + j;  // a pivot of this panel
+                                colrow[32 * cw + c] = row[t];
+                            }
+                        if (lane == 0) s_cnt[1] = k;
+                    }
+                    __syncthreads();
+                    const uint32_t k = s_cnt[1];
+                    npiv += k;
                     for (uint32_t d = tid; d < D; d += T) {
-                        if (d == p) {
+                        const uint32_t own = pivf[d];
+                        uint32_t x = pan[d], y = 0;
+                        if (own >= 2) {
+                            y = s_piv[own - 2].z ^ (1u << (own - 2));
+                            x = 0;  // its columns are done
                             pivf[d] = 1;
-                            s_piv[k] = p;
-                            colrow[32 * cw + c] = p;
-                        } else if ((pan[d] >> c) & 1u) {
-                            pan[d] ^= pw2;
-                            comb[d] ^= pc;
+                        } else {
+                            const uint32_t was = x;
+                            for (uint32_t j = 0; j < k; j++) {
+                                const uint4 p = s_piv[j];
+                                const uint32_t f = 0u - ((was >> p.w) & 1u);
+                                x ^= f & p.y;
+                                y ^= f & p.z;
+                            }
+                        }
+                        pan[d] = x;
+                        comb[d] = y;
+                    }
+                    for (uint32_t j = warp; j < k; j += kLT / 32)
+                        for (uint32_t w = lane; w <= wn; w += 32)
+                            pbuf[j * PS + w] = w < wn ? rows[uint64_t(s_piv[j].x) * RS + w0 + w] : rhs[s_piv[j].x];
+                    __syncthreads();
+                    const uint32_t groups = (k + 3) / 4;
+                    for (uint32_t i = warp; i < groups * 16; i += kLT / 32) {
+                        const uint32_t j0 = i / 16 * 4, n4 = min(4u, k - j0);
+                        const uint32_t* pb = pbuf + j0 * PS;
+                        for (uint32_t w = lane; w <= wn; w += 32) {
+                            uint32_t x = 0;
+#pragma unroll
+                            for (uint32_t t = 0; t < 4; t++)
+                                if (t < n4 && ((i >> t) & 1u)) x ^= pb[t * PS + w];
+                            tab[i * PS + w] = x;
                         }
                     }
-                    k++;
-                }
-                npiv += k;
-                __syncthreads();
-                const uint32_t w0 = cw + 1, wn = AW - w0;  // words still to be brought up to date
-                for (uint32_t i = tid; i < k * (wn + 1); i += T) {
-                    const uint32_t j = i / (wn + 1), w = i % (wn + 1);
-                    pbuf[j * AW + w] = w < wn ? rows[uint64_t(s_piv[j]) * RS + w0 + w] : rhs[s_piv[j]];
-                }
-                __syncthreads();
-                const uint32_t quads = (wn + 1 + 3) / 4;
-                for (uint32_t i = tid; i < D * quads; i += T) {
-                    const uint32_t d = i % D, q = i / D;
-                    uint32_t c = comb[d];
-                    if (!c) continue;
-                    uint32_t x0 = 0, x1 = 0, x2 = 0, x3 = 0;
-                    const uint32_t* pb = pbuf + 4 * q;
-                    for (uint32_t j = 0; j < k; j++, pb += AW) {
-                        const uint32_t f = 0u - ((c >> j) & 1u);
-                        x0 ^= f & pb[0];
-                        if (4 * q + 1 <= wn) x1 ^= f & pb[1];
-                        if (4 * q + 2 <= wn) x2 ^= f & pb[2];
-                        if (4 * q + 3 <= wn) x3 ^= f & pb[3];
-                    }
-                    uint32_t* row = rows + uint64_t(d) * RS + w0 + 4 * q;
-                    const uint32_t xs[4] = {x0, x1, x2, x3};
+                    __syncthreads();
+                    for (uint32_t q = 0; 4 * q <= wn; q++)
+                        for (uint32_t d = tid; d < D; d += T) {
+                            const uint32_t c = comb[d];
+                            if (!c) continue;
+                            uint32_t x[4] = {0, 0, 0, 0};
+                            for (uint32_t g = 0; g < groups; g++) {
+                                const uint4 y = *reinterpret_cast<const uint4*>(tab + (g * 16 + ((c >> (4 * g)) & 15u)) * PS + 4 * q);
+                                x[0] ^= y.x, x[1] ^= y.y, x[2] ^= y.z, x[3] ^= y.w;
+                            }
+                            uint32_t* row = rows + uint64_t(d) * RS + w0 + 4 * q;
 #pragma unroll
-                    for (uint32_t t = 0; t < 4; t++) {
-                        if (4 * q + t < wn) row[t] ^= xs[t];
-                        else if (4 * q + t == wn) rhs[d] ^= xs[t];
-                    }
+                            for (uint32_t t = 0; t < 4; t++) {
+                                if (4 * q + t < wn) row[t] ^= x[t];
+                                else if (4 * q + t == wn) rhs[d] ^= x[t];
+                            }
+                        }
+                    if (k == 32 || npiv == D) break;
                 }
                 __syncthreads();
             }
             for (uint32_t d = tid; d < D; d += T)
                 if (!pivf[d] && rhs[d] != 0) s_fail = 1;
             __syncthreads();
-            if (s_fail) {
-                if (tid == 0) {
-                    atomicOr(a.err, kErrUnsolvable);
-                    atomicOr(a.item_fail + task.item, kErrUnsolvable);
-                }
-                __syncthreads();
-                continue;
-            }
+            if (s_fail) return false;
             // the active variables' values leave the region before the values enter it
             for (uint32_t c = tid; c < A; c += T) lc[c] = colrow[c] != kNone ? rhs[colrow[c]] : 0u;
             __syncthreads();
+            load_records();
         }
         // Values of every variable: active, solved in solve order, then the peeled
         // edges' vertices in reverse peel order.
@@ -902,6 +987,23 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         }
         const uint32_t vmask = b == 32 ? 0xFFFFFFFFu : ((1u << b) - 1u);
         for (uint32_t v = tid; v < V; v += T) cell_put_zero(data, b, cbase + v, vx[v] & vmask);
+        return true;
+        };
+        auto off_smem = [&](uint32_t r) -> uint32_t { return off16[r]; };
+        auto off_any = [&](uint32_t r) -> uint32_t { return rec_smem ? uint32_t(off16[r]) : __ldcg(&soff[r]); };
+        prev_l = rows_smem ? cm_words : cm_words + rows_words;
+        bool solved;
+        if (kSpills || (rec_smem && rows_smem)) solved = solve_all(sm + rb, reinterpret_cast<uint2*>(sm), off_smem, sm + small_words);
+        else solved = solve_all(rec_smem ? sm + rb : V <= kLgeSmemWords ? sm : vstate, rec_smem ? reinterpret_cast<uint2*>(sm) : srec,
+                                off_any, rows_smem ? sm + small_words : L + cm_words);
+        if (!solved) {
+            if (tid == 0) {
+                atomicOr(a.err, kErrUnsolvable);
+                atomicOr(a.item_fail + task.item, kErrUnsolvable);
+            }
+            __syncthreads();
+            continue;
+        }
         if (tid == 0) {
             atomicAdd(&a.stats[0], peeled);
             atomicAdd(&a.stats[1], C - s_dup);
@@ -951,8 +1053,12 @@ uint32_t lge_partition(std::vector<LgeTask>& tasks, uint64_t small_keys) {
 
 cudaError_t launch_lge(const LgeArgs& a, unsigned grid, cudaStream_t st) {
     if (a.ntasks == 0) return cudaSuccess;
-    if (!a.spill) {  // large configuration alone
+    // the large configuration alone: no spill list, or no more shards than SMs
+    // (a shard on an SM of its own is done sooner by 512 threads)
+    if (!a.spill || (a.ntasks <= unsigned(num_sms()) && !getenv("VF_NOBIG"))) {
         LgeArgs only = a;
+        only.spill = nullptr;
+        only.spilled = nullptr;
         only.task_lo = 0;
         only.ctr = 2;
         VF_LGE_BIG<<<std::min(grid, resident(kCfgBig)), kBigT, kBigWords * 4, st>>>(only);
