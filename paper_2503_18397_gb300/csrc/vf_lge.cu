@@ -34,7 +34,7 @@
 // error that ends the build rather than a retry.
 #include <algorithm>
 #include <atomic>
-#include <cstdlib>
+#include <type_traits>
 
 #include "vf_internal.h"
 
@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     __shared__ uint32_t s_part[kLT];
     __shared__ uint4 s_piv[32];    // a panel's pivots: row, reduced panel word, combination with itself, column
     __shared__ uint32_t s_pool[64];  // the rows it is looked for in
+    __shared__ uint32_t s_tz[128];   // sums of four pivots' combinations, 16 for each four
 
     const uint32_t tid = threadIdx.x, T = blockDim.x;
     const unsigned lane = tid & 31u, warp = tid >> 5;
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             C = s_C;
             // Variable states and equation states move to shared memory when they
             // fit (the peel's arrays are dead now); otherwise they stay in the slab.
-            // Equation word: bits 0-1 idle count, bit 2 done, bits 3.. XOR of its idle variables.
+            // Equation word: bits 0-1 idle count, bit 2 done, bits 3.. sum of its idle variables.
             const bool in_smem = uint64_t(V) + C <= kLgeSmemWords;
             if (kSpills && !in_smem && spill_task(a, s)) {
                 __syncthreads();
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 atomicAdd(&vst[v0], 1u);
                 atomicAdd(&vst[v1], 1u);
                 atomicAdd(&vst[v2], 1u);
-                est[j] = ((v0 ^ v1 ^ v2) << 3) | 3u;
+                est[j] = ((v0 + v1 + v2) << 3) | 3u;
             });
             __syncthreads();
             // activation order: core degree, heaviest first (counting sort)
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // and ends the build (kErrDupKey). A copy that differs from the first
             // copy differs from the earlier copy it meets, so one comparison each
             // finds every conflict. Copies have the same vertices, hence equation
-            // words with the same XOR: only then are their signatures compared.
+            // words with the same sum: only then are their signatures compared.
             for_core([&](uint32_t j, uint2 x) {
                 const uint32_t v = x.x & 0xFFFFu, w = est[j] >> 3;
                 const uint32_t q1 = off_of(v + 1);
@@ -522,27 +523,29 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // Removes variable u (now solved from equation `skip`, or active) from
             // every other open equation; an equation left with one idle variable
             // joins the next round's queue, one left with none joins the dense
-            // system. Incidence entries are loaded four at a time, before any
-            // equation is touched, so their loads overlap.
+            // system. Four entries at a time: their loads, then their updates (one
+            // fetch-and-add each, whose result says all) are in flight together. An
+            // equation that is done takes the update too (it is never read again).
             auto remove_var = [&](uint32_t u, uint32_t skip, uint32_t gqi) {
-                const uint32_t q1 = off_of(u + 1);
+                const uint32_t q1 = off_of(u + 1), dec = (u << 3) + 1u;
                 for (uint32_t q = off_of(u); q < q1; q += 4) {
-                    uint32_t ks[4];
+                    uint32_t ks[4], old[4];
 #pragma unroll
                     for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? uint32_t(ilist[q + t]) : kNone;
 #pragma unroll
                     for (uint32_t t = 0; t < 4; t++) {
-                        const uint32_t k = ks[t];
-                        if (k == kNone || k == skip || (est[k] & 4u)) continue;
-                        const uint32_t old = atomicSub(&est[k], 1u);
-                        atomicXor(&est[k], u << 3);
-                        const uint32_t c = (old & 3u) - 1u;
+                        if (ks[t] == skip) ks[t] = kNone;
+                        old[t] = ks[t] != kNone ? atomicSub(&est[ks[t]], dec) : 4u;
+                    }
+#pragma unroll
+                    for (uint32_t t = 0; t < 4; t++) {
+                        if (old[t] & 4u) continue;
+                        const uint32_t c = (old[t] & 3u) - 1u;
                         if (c == 1u) {
-                            qpush(gqi, k);
+                            qpush(gqi, ks[t]);
                         } else if (c == 0u) {
-                            atomicOr(&est[k], 4u);
-                            dense[atomicAdd(&s_D, 1u)] = k;
-                            atomicSub(&s_rem, 1u);
+                            atomicOr(&est[ks[t]], 4u);
+                            dense[atomicAdd(&s_D, 1u)] = ks[t];
                         }
                     }
                 }
@@ -622,18 +625,18 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 } else {
                     const uint32_t lo = s_lo;  // solves of earlier rounds; s_S moves below
                     uint32_t mine = kNone;     // this thread's solve (rounds of at most T entries)
-                    for (uint32_t i = tid; i < nF; i += T) {
-                        const uint32_t j = qread(fi, i);
-                        const uint32_t w = est[j];
-                        if ((w & 4u) || (w & 3u) != 1u) continue;
+                    for (uint32_t i0 = tid & ~31u; i0 < nF; i0 += T) {
+                        const uint32_t i = i0 + lane;
+                        const uint32_t j = i < nF ? qread(fi, i) : 0u;
+                        const uint32_t w = i < nF ? est[j] : 4u;
                         const uint32_t x = w >> 3;
-                        if (atomicCAS(&vst[x], 0u, 3u) != 0u) continue;
-                        const uint32_t si = atomicAdd(&s_S, 1u);
-                        vst[x] = 2u | (si << 2);
-                        mine = (j << 16) | x;
-                        solves[si] = mine;
-                        atomicOr(&est[j], 4u);
-                        atomicSub(&s_rem, 1u);
+                        const bool won = (w & 7u) == 1u && atomicCAS(&vst[x], 0u, 2u) == 0u;
+                        const uint32_t si = warp_slot(&s_S, won);
+                        if (won) {
+                            mine = (j << 16) | x;
+                            solves[si] = mine;
+                            atomicOr(&est[j], 4u);
+                        }
                     }
                     __syncthreads();
                     // eliminate each variable solved this round from its other equations
@@ -650,6 +653,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     s_r++;
                     soff[s_r] = s_S;
                     s_lo = s_S;
+                    s_rem = C - s_dup - s_S - s_D;
                     s_cnt[fi] = 0;
                 }
                 fi ^= 1;
@@ -717,48 +721,76 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         __syncthreads();
         // Written for every place its arrays may be in, as the elimination.
         // false: the system has no solution.
-        auto solve_all = [&](uint32_t* const vx, uint2* const rec, auto&& round_off, uint32_t* const rows) -> bool {
+        auto solve_all = [&](uint32_t* const vx, uint2* const rec, uint32_t* const rows) -> bool {
+        // (and the first solve of every round that has one, s_cnt[3] rounds)
         auto load_records = [&]() {
             if (!rec_smem) return;
+            if (warp == 0) {
+                uint32_t n = 0;
+                for (uint32_t r0 = 0; r0 < R; r0 += 32) {
+                    const uint32_t r = r0 + lane;
+                    const uint32_t o0 = r < R ? __ldcg(&soff[r]) : 0u, o1 = r < R ? __ldcg(&soff[r + 1]) : 0u;
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, o1 > o0);
+                    if (o1 > o0) off16[n + __popc(m & ((1u << lane) - 1u))] = uint16_t(o0);
+                    n += __popc(m);
+                }
+                if (lane == 0) {
+                    off16[n] = uint16_t(S);
+                    s_cnt[3] = n;
+                }
+            }
             for (uint32_t si = tid; si < S; si += T) rec[si] = __ldcg(srec + si);
-            for (uint32_t r = tid; r <= R; r += T) off16[r] = uint16_t(__ldcg(&soff[r]));
         };
-        // The rounds of solves from `first` in steps of `dir`, a barrier behind each.
-        // A round is short (some 60 solves), so its latency counts: the next
-        // round's offsets and records are read before this one's barrier.
-        auto walk = [&](bool back, auto&& f) {
-            uint32_t lo = 0, hi = 0, r = back ? R : 0;
-            uint2 q = make_uint2(0, 0);
-            auto next = [&](uint32_t& nlo, uint32_t& nhi, uint2& nq) {
-                nlo = nhi = 0;
-                while (back ? r > 0 : r < R) {
-                    if (back) r--;
-                    nlo = round_off(r), nhi = round_off(r + 1);
-                    if (!back) r++;
-                    if (nhi > nlo) break;
+        // The rounds of solves, first to last or back, with a barrier behind each. A
+        // round is short (some 60 solves), so its latency is what counts: the next
+        // round's records and the bounds of the one after are on their way while
+        // this one is worked on (420 -> 160 cycles a round).
+        auto walk = [&](auto back_c, auto&& f) {
+            constexpr bool back = decltype(back_c)::value;
+            if (rec_smem) {
+                const uint32_t n = s_cnt[3];
+                uint32_t k = 0;
+                auto bound = [&](uint32_t i) -> uint32_t {  // i-th bound met on the way
+                    const uint32_t j = min(i, n);
+                    return off16[back ? n - j : j];
+                };
+                uint32_t b0 = bound(0), b1 = bound(1), b2 = bound(2);
+                auto first = [&](uint32_t x, uint32_t y) { return (back ? y : x) + tid; };
+                auto last = [&](uint32_t x, uint32_t y) { return back ? x : y; };
+                uint2 q = make_uint2(0, 0);
+                if (first(b0, b1) < last(b0, b1)) q = rec[first(b0, b1)];
+                for (; k < n; k++) {
+                    const uint32_t si = first(b0, b1), hi = last(b0, b1);
+                    const bool on = si < hi;
+                    const uint32_t c = on ? vx[q.x & 0xFFFFu] : 0u;
+                    uint2 nq = make_uint2(0, 0);
+                    if (first(b1, b2) < last(b1, b2)) nq = rec[first(b1, b2)];
+                    const uint32_t b3 = bound(k + 3);
+                    if (on) f(q, c);
+                    for (uint32_t sj = si + T; sj < hi; sj += T) {
+                        const uint2 x = rec[sj];
+                        f(x, vx[x.x & 0xFFFFu]);
+                    }
+                    __syncthreads();
+                    q = nq, b0 = b1, b1 = b2, b2 = b3;
                 }
-                if (nlo + tid < nhi) nq = rec[nlo + tid];
-            };
-            next(lo, hi, q);
-            while (hi > lo) {
-                uint32_t nlo, nhi;
-                uint2 nq = make_uint2(0, 0);
-                const bool on = lo + tid < hi;
-                const uint32_t c = on ? vx[q.x & 0xFFFFu] : 0u;
-                next(nlo, nhi, nq);
-                if (on) f(q, c);
-                for (uint32_t si = lo + tid + T; si < hi; si += T) {
-                    const uint2 x = rec[si];
-                    f(x, vx[x.x & 0xFFFFu]);
+            } else {
+                for (uint32_t k = 0; k < R; k++) {
+                    const uint32_t r = back ? R - 1 - k : k;
+                    const uint32_t lo = __ldcg(&soff[r]), hi = __ldcg(&soff[r + 1]);
+                    if (hi == lo) continue;
+                    for (uint32_t si = lo + tid; si < hi; si += T) {
+                        const uint2 x = rec[si];
+                        f(x, vx[x.x & 0xFFFFu]);
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
-                lo = nlo, hi = nhi, q = nq;
             }
         };
         // Values of the solved variables: vx[x] starts as its equation's
         // right-hand side, the active variables as given.
         auto forward = [&]() {
-            walk(false, [&](uint2 q, uint32_t c) { vx[q.x & 0xFFFFu] = c ^ vx[q.y & 0xFFFFu] ^ vx[q.y >> 16]; });
+            walk(std::false_type{}, [&](uint2 q, uint32_t c) { vx[q.x & 0xFFFFu] = c ^ vx[q.y & 0xFFFFu] ^ vx[q.y >> 16]; });
         };
         load_records();
         __syncthreads();
@@ -795,7 +827,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     atomicXor(&vx[q.y], 1u << tid);
                 }
                 __syncthreads();
-                walk(true, [&](uint2 q, uint32_t c) {
+                walk(std::true_type{}, [&](uint2 q, uint32_t c) {
                     if (c) {
                         atomicXor(&vx[q.y & 0xFFFFu], c);
                         atomicXor(&vx[q.y >> 16], c);
@@ -896,6 +928,16 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     __syncthreads();
                     const uint32_t k = s_cnt[1];
                     npiv += k;
+                    if (k == 32) {  // pivot j stands in column j: its combinations in fours, too
+                        if (tid < 128) {
+                            uint32_t z = 0;
+#pragma unroll
+                            for (uint32_t t = 0; t < 4; t++)
+                                if ((tid >> t) & 1u) z ^= s_piv[tid / 16 * 4 + t].z;
+                            s_tz[tid] = z;
+                        }
+                        __syncthreads();
+                    }
                     for (uint32_t d = tid; d < D; d += T) {
                         const uint32_t own = pivf[d];
                         uint32_t x = pan[d], y = 0;
@@ -903,6 +945,10 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                             y = s_piv[own - 2].z ^ (1u << (own - 2));
                             x = 0;  // its columns are done
                             pivf[d] = 1;
+                        } else if (k == 32) {
+#pragma unroll
+                            for (uint32_t g = 0; g < 8; g++) y ^= s_tz[g * 16 + ((x >> (4 * g)) & 15u)];
+                            x = 0;
                         } else {
                             const uint32_t was = x;
                             for (uint32_t j = 0; j < k; j++) {
@@ -989,13 +1035,11 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         for (uint32_t v = tid; v < V; v += T) cell_put_zero(data, b, cbase + v, vx[v] & vmask);
         return true;
         };
-        auto off_smem = [&](uint32_t r) -> uint32_t { return off16[r]; };
-        auto off_any = [&](uint32_t r) -> uint32_t { return rec_smem ? uint32_t(off16[r]) : __ldcg(&soff[r]); };
         prev_l = rows_smem ? cm_words : cm_words + rows_words;
         bool solved;
-        if (kSpills || (rec_smem && rows_smem)) solved = solve_all(sm + rb, reinterpret_cast<uint2*>(sm), off_smem, sm + small_words);
+        if (kSpills || (rec_smem && rows_smem)) solved = solve_all(sm + rb, reinterpret_cast<uint2*>(sm), sm + small_words);
         else solved = solve_all(rec_smem ? sm + rb : V <= kLgeSmemWords ? sm : vstate, rec_smem ? reinterpret_cast<uint2*>(sm) : srec,
-                                off_any, rows_smem ? sm + small_words : L + cm_words);
+                                rows_smem ? sm + small_words : L + cm_words);
         if (!solved) {
             if (tid == 0) {
                 atomicOr(a.err, kErrUnsolvable);
@@ -1055,7 +1099,7 @@ cudaError_t launch_lge(const LgeArgs& a, unsigned grid, cudaStream_t st) {
     if (a.ntasks == 0) return cudaSuccess;
     // the large configuration alone: no spill list, or no more shards than SMs
     // (a shard on an SM of its own is done sooner by 512 threads)
-    if (!a.spill || (a.ntasks <= unsigned(num_sms()) && !getenv("VF_NOBIG"))) {
+    if (!a.spill || (a.ntasks <= unsigned(num_sms()))) {
         LgeArgs only = a;
         only.spill = nullptr;
         only.spilled = nullptr;
