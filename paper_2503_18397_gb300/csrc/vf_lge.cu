@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     extern __shared__ __align__(16) uint32_t sm[];
     __shared__ uint32_t s_shard, s_fail;
     __shared__ uint32_t s_cnt[4];
-    __shared__ uint32_t s_C, s_rem, s_A, s_S, s_D, s_r, s_apos, s_nact, s_nbatch, s_lo, s_dup;
+    __shared__ uint32_t s_C, s_nact, s_nbatch, s_dup;
+    __shared__ uint32_t s_queue[4], s_solved[4], s_dense[4];  // the elimination's rounds
     __shared__ uint32_t s_hist[256];
     __shared__ uint32_t s_batch[kMaxBatch];
     __shared__ uint32_t s_part[kLT];
@@ -514,59 +515,48 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             }
             uint16_t* const gq = reinterpret_cast<uint16_t*>(scr + o.lists);
             const uint32_t gq1 = 2 * ((a.v_cap + 1) / 2);
-            auto qpush = [&](uint32_t q, uint32_t k) {
-                const uint32_t idx = atomicAdd(&s_cnt[q], 1u);
-                if (idx < qcap) sq0[q * qcap + idx] = k;
-                else gq[(q ? gq1 : 0u) + idx] = uint16_t(k);
-            };
+            // Counters of a round, one set for each r mod 4 (a set is cleared two
+            // rounds before its round and read after its round's only barrier):
+            // queue entries for the round, its solves, its dense equations.
             auto qread = [&](uint32_t q, uint32_t i) -> uint32_t { return i < qcap ? sq0[q * qcap + i] : gq[(q ? gq1 : 0u) + i]; };
+            uint32_t r = 0, ns = 0, nd = 0, na = 0, apos = 0;  // round; solves, dense equations, active variables so far
             // Removes variable u (now solved from equation `skip`, or active) from
-            // every other open equation; an equation left with one idle variable
-            // joins the next round's queue, one left with none joins the dense
-            // system. Four entries at a time: their loads, then their updates (one
-            // fetch-and-add each, whose result says all) are in flight together. An
-            // equation that is done takes the update too (it is never read again).
-            auto remove_var = [&](uint32_t u, uint32_t skip, uint32_t gqi) {
+            // its other equations, four lanes taking an entry each of its incidence
+            // list: an equation left with one idle variable joins the next round's
+            // queue, one left with none joins the dense system. One fetch-and-add
+            // per entry, whose result says all; an equation that is done takes the
+            // update too (it is never read again).
+            auto remove_var = [&](uint32_t u, uint32_t skip) {
                 const uint32_t q1 = off_of(u + 1), dec = (u << 3) + 1u;
-                for (uint32_t q = off_of(u); q < q1; q += 4) {
-                    uint32_t ks[4], old[4];
-#pragma unroll
-                    for (uint32_t t = 0; t < 4; t++) ks[t] = q + t < q1 ? uint32_t(ilist[q + t]) : kNone;
-#pragma unroll
-                    for (uint32_t t = 0; t < 4; t++) {
-                        if (ks[t] == skip) ks[t] = kNone;
-                        old[t] = ks[t] != kNone ? atomicSub(&est[ks[t]], dec) : 4u;
-                    }
-#pragma unroll
-                    for (uint32_t t = 0; t < 4; t++) {
-                        if (old[t] & 4u) continue;
-                        const uint32_t c = (old[t] & 3u) - 1u;
-                        if (c == 1u) {
-                            qpush(gqi, ks[t]);
-                        } else if (c == 0u) {
-                            atomicOr(&est[ks[t]], 4u);
-                            dense[atomicAdd(&s_D, 1u)] = ks[t];
-                        }
+                for (uint32_t q = off_of(u) + (lane & 3u); q < q1; q += 4) {
+                    const uint32_t k = ilist[q];
+                    if (k == skip) continue;
+                    const uint32_t old = atomicSub(&est[k], dec);
+                    if (old & 4u) continue;
+                    const uint32_t c = (old & 3u) - 1u;
+                    if (c == 1u) {
+                        const uint32_t idx = atomicAdd(&s_queue[(r + 1) & 3u], 1u), nq = (r + 1) & 1u;
+                        if (idx < qcap) sq0[nq * qcap + idx] = k;
+                        else gq[(nq ? gq1 : 0u) + idx] = uint16_t(k);
+                    } else if (c == 0u) {
+                        atomicOr(&est[k], 4u);
+                        dense[nd + atomicAdd(&s_dense[r & 3u], 1u)] = k;
                     }
                 }
             };
-            if (tid == 0) {
-                s_rem = C - s_dup;
-                s_A = s_S = s_D = s_r = s_apos = s_lo = 0;
-                s_cnt[0] = s_cnt[1] = 0;
-                soff[0] = 0;
-            }
-            fi = 0;
+            if (tid < 4) s_queue[tid] = s_solved[tid] = s_dense[tid] = 0;
+            if (tid == 0) soff[0] = 0;
             const uint32_t max_rounds = m + V + 2;
             __syncthreads();
+            const uint32_t open = C - s_dup;
             for (;;) {
-                if (s_rem == 0 || s_fail) break;
-                if (s_r >= max_rounds) {
+                const uint32_t rem = open - ns - nd;
+                if (rem == 0) break;
+                if (r >= max_rounds) {
                     if (tid == 0) s_fail = 2;
-                    __syncthreads();
                     break;
                 }
-                const uint32_t nF = s_cnt[fi];
+                const uint32_t nF = s_queue[r & 3u];
                 if (nF == 0) {
                     // Activate the next heaviest idle variables that still occur in
                     // open equations: the block examines a window of the activation
@@ -575,13 +565,12 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     // slightly fewer active variables but need many more rounds (per
                     // 9.8K-key shard, 1%: 194 rounds, 655 active; 2.5%: 112 and 704,
                     // 4% fewer cycles)
-                    const uint32_t K = max(1u, min(kMaxBatch, s_rem / 40u));
-                    const uint32_t base = s_apos;
-                    const uint32_t wn = min(T, s_nact - base);
+                    const uint32_t K = max(1u, min(kMaxBatch, rem / 40u));
+                    const uint32_t wn = min(T, s_nact - apos);
                     bool elig = false;
                     uint32_t v = 0;
                     if (tid < wn) {
-                        v = act[base + tid];
+                        v = act[apos + tid];
                         if (vst[v] == 0) {
                             const uint32_t q1 = off_of(v + 1);
                             for (uint32_t q = off_of(v); q < q1 && !elig; q += 4) {
@@ -603,62 +592,62 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                         tot += x;
                     }
                     if (elig && rank < K) s_batch[rank] = v;
-                    if (elig && rank == K - 1) s_nbatch = base + tid + 1;  // new scan position
+                    if (elig && rank == K - 1) s_nbatch = apos + tid + 1;  // new scan position
                     __syncthreads();
-                    if (tid == 0) {
-                        const uint32_t nb = min(K, tot);
-                        s_apos = tot >= K ? s_nbatch : base + wn;
-                        s_nbatch = nb;
-                        if (s_A + nb > o.a_cap || (nb == 0 && s_apos >= s_nact)) s_fail = 2;
+                    const uint32_t nb = min(K, tot);
+                    apos = tot >= K ? s_nbatch : apos + wn;
+                    if (na + nb > o.a_cap || (nb == 0 && apos >= s_nact)) {
+                        if (tid == 0) s_fail = 2;
+                        break;
                     }
-                    __syncthreads();
-                    if (s_fail) break;
-                    const uint32_t nb = s_nbatch, abase = s_A;
-                    for (uint32_t i = tid; i < nb; i += T) {
+                    for (uint32_t i = tid / 4; i < nb; i += kLT / 4) {
                         const uint32_t u = s_batch[i];
-                        vst[u] = 1u | ((abase + i) << 2);
-                        actv[abase + i] = u;
-                        remove_var(u, kNone, fi ^ 1);
+                        if ((tid & 3u) == 0) {
+                            vst[u] = 1;
+                            actv[na + i] = u;
+                        }
+                        remove_var(u, kNone);
                     }
-                    __syncthreads();
-                    if (tid == 0) s_A += nb;
+                    na += nb;
                 } else {
-                    const uint32_t lo = s_lo;  // solves of earlier rounds; s_S moves below
-                    uint32_t mine = kNone;     // this thread's solve (rounds of at most T entries)
-                    for (uint32_t i0 = tid & ~31u; i0 < nF; i0 += T) {
-                        const uint32_t i = i0 + lane;
-                        const uint32_t j = i < nF ? qread(fi, i) : 0u;
+                    // Queue entries dealt out over the warps; a warp then takes its
+                    // solves eight at a time. (No barrier in between: an equation of
+                    // this queue has one idle variable, and whoever solves that
+                    // variable elsewhere leaves the equation with none.)
+                    for (uint32_t i0 = 0; i0 < nF; i0 += kLT) {
+                        const uint32_t i = i0 + lane * (kLT / 32) + warp;
+                        const uint32_t j = i < nF ? qread(r & 1u, i) : 0u;
                         const uint32_t w = i < nF ? est[j] : 4u;
                         const uint32_t x = w >> 3;
                         const bool won = (w & 7u) == 1u && atomicCAS(&vst[x], 0u, 2u) == 0u;
-                        const uint32_t si = warp_slot(&s_S, won);
+                        const unsigned mw = __ballot_sync(0xFFFFFFFFu, won);
+                        if (mw == 0) continue;
+                        uint32_t at = 0;
+                        if (lane == 0) at = atomicAdd(&s_solved[r & 3u], uint32_t(__popc(mw)));
+                        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+                        const uint32_t mine = __popc(mw & ((1u << lane) - 1u));
                         if (won) {
-                            mine = (j << 16) | x;
-                            solves[si] = mine;
+                            s_part[32 * warp + mine] = (j << 16) | x;
+                            solves[ns + at + mine] = (j << 16) | x;
                             atomicOr(&est[j], 4u);
                         }
+                        __syncwarp();
+                        for (uint32_t g = lane / 4; g < uint32_t(__popc(mw)); g += 8) {
+                            const uint32_t sv = s_part[32 * warp + g];
+                            remove_var(sv & 0xFFFFu, sv >> 16);
+                        }
+                        __syncwarp();
                     }
-                    __syncthreads();
-                    // eliminate each variable solved this round from its other equations
-                    auto eliminate = [&](uint32_t sv) { remove_var(sv & 0xFFFFu, sv >> 16, fi ^ 1); };
-                    if (nF <= T) {  // each solve is still in the register of the thread that made it
-                        if (mine != kNone) eliminate(mine);
-                    } else {
-                        const uint32_t hi = s_S;
-                        for (uint32_t si = lo + tid; si < hi; si += T) eliminate(__ldcg(&solves[si]));
-                    }
-                    __syncthreads();
                 }
-                if (tid == 0) {
-                    s_r++;
-                    soff[s_r] = s_S;
-                    s_lo = s_S;
-                    s_rem = C - s_dup - s_S - s_D;
-                    s_cnt[fi] = 0;
-                }
-                fi ^= 1;
+                if (tid == 0) s_queue[(r + 2) & 3u] = s_solved[(r + 2) & 3u] = s_dense[(r + 2) & 3u] = 0;
                 __syncthreads();
+                ns += s_solved[r & 3u];
+                nd += s_dense[r & 3u];
+                r++;
+                if (tid == 0) soff[r] = ns;
             }
+            __syncthreads();
+            A = na, S = ns, D = nd, R = r;
             };
             if (kSpills || in_smem) eliminate_all(sm, sm + V);
             else eliminate_all(vstate, eqst);
@@ -671,8 +660,6 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                 __syncthreads();
                 continue;
             }
-            A = s_A, S = s_S, D = s_D, R = s_r;
-            __syncthreads();
         }
         const uint32_t AW = (A + 31) / 32, DW = (D + 31) / 32;
         const uint32_t RS = AW | 1u;  // odd row stride: conflict-free shared-memory rows
