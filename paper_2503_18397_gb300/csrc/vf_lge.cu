@@ -51,6 +51,10 @@ constexpr uint32_t kMidWords = 27 * 1024;
 constexpr int kSmallT = 192;
 constexpr uint32_t kSmallWords = 18 * 1024;
 constexpr uint32_t kNone = 0xFFFFFFFFu;
+// equation words: the sum of up to three 16-bit variables in bits 3..20, and a mark
+constexpr uint32_t kSumMask = 0x001FFFF8u;
+constexpr uint32_t kTwin = 0x80000000u;
+constexpr uint32_t kLgSeen = 16, kSeenWords = 1u << (kLgSeen - 5);
 
 uint64_t lge_scratch_words_per_cta(uint32_t m_cap, uint32_t v_cap) { return lge_offsets(m_cap, v_cap).total; }
 
@@ -89,6 +93,11 @@ __device__ void cta_exclusive_scan(uint32_t* cnt, uint32_t len, uint32_t* part) 
         run += x;
     }
     __syncthreads();
+}
+
+// Barrier `id` (1..15) of n threads.
+__device__ __forceinline__ void bar_some(uint32_t id, uint32_t n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
 // A slot of *ctr for every lane with `p` (one shared atomic per warp; all
@@ -192,6 +201,10 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
     uint32_t* dense = scr + o.dense;
     uint32_t* lc = scr + o.lc;
     uint32_t* L = scr + o.L;
+    // threads of the elimination's rounds: a round has ~50 solves, and a warp
+    // without one still issues the round's instructions
+    constexpr int kET = kLT < 256 ? kLT : 256;
+    constexpr int kGT = kLT % 128 ? kLT / 2 : 128;  // and of a walk over the solves
     // the small configurations hand on a shard whose arrays do not all fit
     constexpr bool kSpills = kLgeSmemWords != kBigWords;
     constexpr uint32_t kBad = kErrUnsolvable | kErrCapacity | kErrLgeSize | kErrDegOverflow | kErrDupKey;
@@ -396,15 +409,24 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // states. Written for both places they may be in (the compiler then
             // uses shared-memory instructions for the usual one).
             auto eliminate_all = [&](uint32_t* const vst, uint32_t* const est) {
+            // a bit per hashed vertex triple: equations that find theirs set may repeat another
+            uint32_t* const seen = in_smem && V + C + kSeenWords <= kLgeSmemWords ? sm + V + C : nullptr;
             for (uint32_t v = tid; v < V; v += T) vst[v] = 0;
             for (uint32_t i = tid; i < 256; i += T) s_hist[i] = 0;
+            if (seen)
+                for (uint32_t i = tid; i < kSeenWords; i += T) seen[i] = 0;
             __syncthreads();
             for_core([&](uint32_t j, uint2 x) {
                 const uint32_t v0 = x.x & 0xFFFFu, v1 = x.x >> 16, v2 = x.y;
                 atomicAdd(&vst[v0], 1u);
                 atomicAdd(&vst[v1], 1u);
                 atomicAdd(&vst[v2], 1u);
-                est[j] = ((v0 + v1 + v2) << 3) | 3u;
+                uint32_t twin = kTwin;
+                if (seen) {
+                    const uint32_t h = (x.x * 0x9E3779B1u + x.y * 0x85EBCA77u) >> (32 - kLgSeen);
+                    if (!((atomicOr(&seen[h >> 5], 1u << (h & 31u)) >> (h & 31u)) & 1u)) twin = 0;
+                }
+                est[j] = ((v0 + v1 + v2) << 3) | 3u | twin;
             });
             __syncthreads();
             // activation order: core degree, heaviest first (counting sort)
@@ -480,30 +502,29 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // vertex; the copy of smallest index stays. A filter's copies carry
             // the same fingerprint, a function's copies are dropped when their
             // values agree; a key with two values has no solution at any seed
-            // and ends the build (kErrDupKey). A copy that differs from the first
-            // copy differs from the earlier copy it meets, so one comparison each
-            // finds every conflict. Copies have the same vertices, hence equation
-            // words with the same sum: only then are their signatures compared.
+            // and ends the build (kErrDupKey). Of every two copies one is a twin
+            // (it found their bit set), and copies have the same vertex sum: only
+            // such pairs' signatures are compared.
             for_core([&](uint32_t j, uint2 x) {
-                const uint32_t v = x.x & 0xFFFFu, w = est[j] >> 3;
+                const uint32_t wj = est[j];
+                if (!(wj & kTwin)) return;
+                const uint32_t v = x.x & 0xFFFFu, w = wj & kSumMask;
                 const uint32_t q1 = off_of(v + 1);
                 for (uint32_t q = off_of(v); q < q1; q++) {
                     const uint32_t j2 = ilist[q];
-                    if (j2 == j || (est[j2] >> 3) != w) continue;
+                    if (j2 == j || (est[j2] & kSumMask) != w) continue;
                     const uint32_t e = core[j], e2 = core[j2];
-                    if (e2 < e && __ldg(a.loc + e0 + e2) == __ldg(a.loc + e0 + e)) {
-                        if (task.kind == 0 && __ldg(a.val + e0 + e2) != __ldg(a.val + e0 + e)) {
-                            s_fail = 3;
-                        } else {
-                            atomicOr(&est[j], 4u);  // done: no equation of its own
-                            atomicAdd(&s_dup, 1u);
-                        }
-                        break;
+                    if (__ldg(a.loc + e0 + e2) != __ldg(a.loc + e0 + e)) continue;
+                    if (task.kind == 0 && __ldg(a.val + e0 + e2) != __ldg(a.val + e0 + e)) {
+                        s_fail = 3;
+                    } else if (!(atomicOr(&est[e < e2 ? j2 : j], 4u) & 4u)) {
+                        atomicAdd(&s_dup, 1u);  // done: no equation of its own
                     }
                 }
             });
             __syncthreads();
             if (s_fail == 3) return;
+            for (uint32_t j = tid; j < C; j += T) est[j] &= ~kTwin;
             // The rest of shared memory holds the first qcap entries of the two
             // round queues; entries beyond stay in the slab's queues.
             uint32_t qcap = 0;
@@ -548,6 +569,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             if (tid == 0) soff[0] = 0;
             const uint32_t max_rounds = m + V + 2;
             __syncthreads();
+            if (tid < kET) {
             const uint32_t open = C - s_dup;
             for (;;) {
                 const uint32_t rem = open - ns - nd;
@@ -566,7 +588,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     // 9.8K-key shard, 1%: 194 rounds, 655 active; 2.5%: 112 and 704,
                     // 4% fewer cycles)
                     const uint32_t K = max(1u, min(kMaxBatch, rem / 40u));
-                    const uint32_t wn = min(T, s_nact - apos);
+                    const uint32_t wn = min(uint32_t(kET), s_nact - apos);
                     bool elig = false;
                     uint32_t v = 0;
                     if (tid < wn) {
@@ -584,23 +606,23 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     }
                     const unsigned bal = __ballot_sync(0xFFFFFFFFu, elig);
                     if (lane == 0) s_part[warp] = __popc(bal);
-                    __syncthreads();
+                    bar_some(1, kET);
                     uint32_t rank = __popc(bal & ((1u << lane) - 1u)), tot = 0;
-                    for (uint32_t w = 0; w < kLT / 32; w++) {
+                    for (uint32_t w = 0; w < kET / 32; w++) {
                         const uint32_t x = s_part[w];
                         if (w < warp) rank += x;
                         tot += x;
                     }
                     if (elig && rank < K) s_batch[rank] = v;
                     if (elig && rank == K - 1) s_nbatch = apos + tid + 1;  // new scan position
-                    __syncthreads();
+                    bar_some(1, kET);
                     const uint32_t nb = min(K, tot);
                     apos = tot >= K ? s_nbatch : apos + wn;
                     if (na + nb > o.a_cap || (nb == 0 && apos >= s_nact)) {
                         if (tid == 0) s_fail = 2;
                         break;
                     }
-                    for (uint32_t i = tid / 4; i < nb; i += kLT / 4) {
+                    for (uint32_t i = tid / 4; i < nb; i += kET / 4) {
                         const uint32_t u = s_batch[i];
                         if ((tid & 3u) == 0) {
                             vst[u] = 1;
@@ -614,8 +636,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     // solves eight at a time. (No barrier in between: an equation of
                     // this queue has one idle variable, and whoever solves that
                     // variable elsewhere leaves the equation with none.)
-                    for (uint32_t i0 = 0; i0 < nF; i0 += kLT) {
-                        const uint32_t i = i0 + lane * (kLT / 32) + warp;
+                    for (uint32_t i0 = 0; i0 < nF; i0 += kET) {
+                        const uint32_t i = i0 + lane * (kET / 32) + warp;
                         const uint32_t j = i < nF ? qread(r & 1u, i) : 0u;
                         const uint32_t w = i < nF ? est[j] : 4u;
                         const uint32_t x = w >> 3;
@@ -640,14 +662,16 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     }
                 }
                 if (tid == 0) s_queue[(r + 2) & 3u] = s_solved[(r + 2) & 3u] = s_dense[(r + 2) & 3u] = 0;
-                __syncthreads();
+                bar_some(1, kET);
                 ns += s_solved[r & 3u];
                 nd += s_dense[r & 3u];
                 r++;
                 if (tid == 0) soff[r] = ns;
             }
+            if (tid == 0) s_batch[0] = na, s_batch[1] = ns, s_batch[2] = nd, s_batch[3] = r;
+            }
             __syncthreads();
-            A = na, S = ns, D = nd, R = r;
+            A = s_batch[0], S = s_batch[1], D = s_batch[2], R = s_batch[3];
             };
             if (kSpills || in_smem) eliminate_all(sm, sm + V);
             else eliminate_all(vstate, eqst);
@@ -732,7 +756,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
         // round is short (some 60 solves), so its latency is what counts: the next
         // round's records and the bounds of the one after are on their way while
         // this one is worked on (420 -> 160 cycles a round).
-        auto walk = [&](auto back_c, auto&& f) {
+        // Run by gt threads (this one is gtid of them) that share barrier `bar`.
+        auto walk = [&](auto back_c, uint32_t* const vx, uint32_t gt, uint32_t gtid, uint32_t bar, auto&& f) {
             constexpr bool back = decltype(back_c)::value;
             if (rec_smem) {
                 const uint32_t n = s_cnt[3];
@@ -742,7 +767,7 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     return off16[back ? n - j : j];
                 };
                 uint32_t b0 = bound(0), b1 = bound(1), b2 = bound(2);
-                auto first = [&](uint32_t x, uint32_t y) { return (back ? y : x) + tid; };
+                auto first = [&](uint32_t x, uint32_t y) { return (back ? y : x) + gtid; };
                 auto last = [&](uint32_t x, uint32_t y) { return back ? x : y; };
                 uint2 q = make_uint2(0, 0);
                 if (first(b0, b1) < last(b0, b1)) q = rec[first(b0, b1)];
@@ -754,11 +779,11 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     if (first(b1, b2) < last(b1, b2)) nq = rec[first(b1, b2)];
                     const uint32_t b3 = bound(k + 3);
                     if (on) f(q, c);
-                    for (uint32_t sj = si + T; sj < hi; sj += T) {
+                    for (uint32_t sj = si + gt; sj < hi; sj += gt) {
                         const uint2 x = rec[sj];
                         f(x, vx[x.x & 0xFFFFu]);
                     }
-                    __syncthreads();
+                    bar_some(bar, gt);
                     q = nq, b0 = b1, b1 = b2, b2 = b3;
                 }
             } else {
@@ -766,18 +791,21 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                     const uint32_t r = back ? R - 1 - k : k;
                     const uint32_t lo = __ldcg(&soff[r]), hi = __ldcg(&soff[r + 1]);
                     if (hi == lo) continue;
-                    for (uint32_t si = lo + tid; si < hi; si += T) {
+                    for (uint32_t si = lo + gtid; si < hi; si += gt) {
                         const uint2 x = rec[si];
                         f(x, vx[x.x & 0xFFFFu]);
                     }
-                    __syncthreads();
+                    bar_some(bar, gt);
                 }
             }
         };
         // Values of the solved variables: vx[x] starts as its equation's
         // right-hand side, the active variables as given.
         auto forward = [&]() {
-            walk(std::false_type{}, [&](uint2 q, uint32_t c) { vx[q.x & 0xFFFFu] = c ^ vx[q.y & 0xFFFFu] ^ vx[q.y >> 16]; });
+            if (tid < kGT)
+                walk(std::false_type{}, vx, kGT, tid, 1,
+                     [&](uint2 q, uint32_t c) { vx[q.x & 0xFFFFu] = c ^ vx[q.y & 0xFFFFu] ^ vx[q.y >> 16]; });
+            __syncthreads();
         };
         load_records();
         __syncthreads();
@@ -803,24 +831,33 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             // (Carrying the columns forward, one coefficient row per solve, takes
             // as many bits per solve as there are active variables, 2.5 times the
             // dense equations, and the rows do not fit in shared memory.)
-            for (uint32_t w = 0; w < DW; w++) {
-                __syncthreads();
-                for (uint32_t v = tid; v < V; v += T) vx[v] = 0;
-                __syncthreads();
-                if (tid < 32 && 32 * w + tid < D) {
-                    const uint2 q = __ldcg(ev + core[__ldcg(&dense[32 * w + tid])]);
-                    atomicXor(&vx[q.x & 0xFFFFu], 1u << tid);
-                    atomicXor(&vx[q.x >> 16], 1u << tid);
-                    atomicXor(&vx[q.y], 1u << tid);
-                }
-                __syncthreads();
-                walk(std::true_type{}, [&](uint2 q, uint32_t c) {
-                    if (c) {
-                        atomicXor(&vx[q.y & 0xFFFFu], c);
-                        atomicXor(&vx[q.y >> 16], c);
+            // As many groups of threads as have room for a word per variable take
+            // 32 equations each at the same time.
+            __syncthreads();
+            const uint32_t groups = rec_smem ? max(1u, min(min(DW, uint32_t(kLT / kGT)), (kLgeSmemWords - rb) / V)) : 1u;
+            const uint32_t gt = groups > 1 ? kGT : kET;  // one group alone takes the elimination's threads
+            const uint32_t grp = tid / gt, gtid = tid % gt;
+            if (grp < groups) {
+                uint32_t* const gx = vx + grp * V;
+                for (uint32_t w = grp; w < DW; w += groups) {
+                    for (uint32_t v = gtid; v < V; v += gt) gx[v] = 0;
+                    bar_some(1 + grp, gt);
+                    if (gtid < 32 && 32 * w + gtid < D) {
+                        const uint2 q = __ldcg(ev + core[__ldcg(&dense[32 * w + gtid])]);
+                        atomicXor(&gx[q.x & 0xFFFFu], 1u << gtid);
+                        atomicXor(&gx[q.x >> 16], 1u << gtid);
+                        atomicXor(&gx[q.y], 1u << gtid);
                     }
-                });
-                for (uint32_t c = tid; c < A; c += T) L[uint64_t(w) * A + c] = vx[__ldcg(&actv[c])];
+                    bar_some(1 + grp, gt);
+                    walk(std::true_type{}, gx, gt, gtid, 1 + grp, [&](uint2 q, uint32_t c) {
+                        if (c) {
+                            atomicXor(&gx[q.y & 0xFFFFu], c);
+                            atomicXor(&gx[q.y >> 16], c);
+                        }
+                    });
+                    for (uint32_t c = gtid; c < A; c += gt) L[uint64_t(w) * A + c] = gx[__ldcg(&actv[c])];
+                    bar_some(1 + grp, gt);
+                }
             }
             __syncthreads();
             uint32_t* const small = sm;
