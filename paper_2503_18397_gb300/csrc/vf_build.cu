@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kThreads) k_hist_bytes(const uint8_t* __restri
                                                          const uint64_t* __restrict__ offs, uint64_t n, Geom g,
                                                          uint32_t* __restrict__ hist, Sig* __restrict__ sig_out) {
     __shared__ uint32_t sh[kSmemBinsMax];
+    __shared__ uint4 stage[kStageBytes / 16];
     const uint32_t S = 1u << g.h;
     const bool in_smem = S <= kSmemBinsMax;
     if (in_smem)
@@ -43,9 +44,10 @@ __global__ void __launch_bounds__(kThreads) k_hist_bytes(const uint8_t* __restri
     __syncthreads();
     const uint64_t total = __ldg(offs + n);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < n; i += stride) {
-        uint64_t o0 = __ldg(offs + i), o1 = __ldg(offs + i + 1);
-        Sig s = sig_bytes(buf, total, o0, o1 - o0, g.kh, g.kl);
+    for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < n; t0 += stride) {
+        const Sig s = sig_tile(buf, offs, total, t0, n, stage, g.kh, g.kl);
+        const uint64_t i = t0 + threadIdx.x;
+        if (i >= n) continue;
         sig_out[i] = s;
         uint32_t b = uint32_t(shard_of(s, g.h));
         if (in_smem) atomicAdd(&sh[b], 1u); else atomicAdd(&hist[b], 1u);
@@ -177,11 +179,12 @@ __global__ void k_sigs_u64(const uint64_t* __restrict__ keys, uint64_t n, uint64
 
 __global__ void k_sigs_bytes(const uint8_t* __restrict__ buf, const uint64_t* __restrict__ offs, uint64_t n,
                              uint64_t kh, uint64_t kl, Sig* __restrict__ out) {
+    __shared__ uint4 stage[kStageBytes / 16];
     const uint64_t total = __ldg(offs + n);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < n; i += stride) {
-        uint64_t o0 = __ldg(offs + i), o1 = __ldg(offs + i + 1);
-        out[i] = sig_bytes(buf, total, o0, o1 - o0, kh, kl);
+    for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < n; t0 += stride) {
+        const Sig s = sig_tile(buf, offs, total, t0, n, stage, kh, kl);
+        if (t0 + threadIdx.x < n) out[t0 + threadIdx.x] = s;
     }
 }
 

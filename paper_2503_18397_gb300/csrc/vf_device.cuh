@@ -103,6 +103,78 @@ __device__ __forceinline__ Sig sig_bytes(const uint8_t* buf, uint64_t total, uin
     return Sig{mix64(a), mix64(b)};
 }
 
+// A tile of packed byte strings in shared memory. Hashing them from global
+// memory touches 32 lines with every load of a warp (one string a lane, two
+// loads a word), and the load units, not bandwidth, set the pace; staged, every
+// byte is read once, 16 at a time.
+constexpr uint32_t kStageBytes = 20 * 1024;  // 256 strings of 64 bytes, and some
+
+// Bytes [lo, hi) of the buffer to `stage` (16-byte aligned, kStageBytes), the
+// byte lo at offset `at`. false (for all threads alike) if they do not fit. The
+// caller puts a barrier behind it. 16-byte loads inside the buffer, byte loads
+// at its ends.
+__device__ __forceinline__ bool stage_bytes(const uint8_t* buf, uint64_t total, uint64_t lo, uint64_t hi, uint4* stage,
+                                            uint32_t& at) {
+    const uintptr_t first = reinterpret_cast<uintptr_t>(buf), a0 = (first + lo) & ~uintptr_t(15);
+    at = uint32_t(first + lo - a0);
+    if (hi < lo || hi > total || hi - lo > kStageBytes - 48) return false;
+    const uint32_t chunks = (at + uint32_t(hi - lo) + 15) / 16;
+    for (uint32_t c = threadIdx.x; c < chunks; c += blockDim.x) {
+        const uintptr_t a = a0 + 16 * uintptr_t(c);
+        if (a >= first && a + 16 <= first + total) {
+            stage[c] = __ldg(reinterpret_cast<const uint4*>(a));
+        } else {
+            uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (uint32_t j = 0; j < 16; j++)
+                if (a + j >= first && a + j < first + total)
+                    w[j / 4] |= uint32_t(__ldg(reinterpret_cast<const uint8_t*>(a + j))) << (8 * (j % 4));
+            stage[c] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+    return true;
+}
+
+// sig_bytes of the staged string at byte offset `p`, len bytes long.
+__device__ __forceinline__ Sig sig_staged(const uint4* stage, uint32_t p, uint32_t len, uint64_t kh, uint64_t kl) {
+    const uint64_t* w8 = reinterpret_cast<const uint64_t*>(stage) + (p >> 3);
+    const uint32_t sh = 8 * (p & 7u);
+    uint64_t a = kh ^ (uint64_t(len) * kGolden);
+    uint64_t b = kl ^ uint64_t(len);
+    uint64_t cur = len ? w8[0] : 0;
+    for (uint32_t i = 0; 8 * i < len; i++) {
+        const uint64_t nxt = w8[i + 1];  // the stage has room behind the last string
+        uint64_t w = sh ? (cur >> sh) | (nxt << (64 - sh)) : cur;
+        const uint32_t left = len - 8 * i;
+        if (left < 8) w &= (uint64_t(1) << (8 * left)) - 1;
+        a = mix64(a ^ w);
+        b = mix64(b + w);
+        cur = nxt;
+    }
+    return Sig{mix64(a), mix64(b)};
+}
+
+// Signature of string i of the tile [t0, t0 + blockDim.x) of m packed strings
+// (i = t0 + threadIdx.x), through `stage`; every thread of the block calls it.
+__device__ __forceinline__ Sig sig_tile(const uint8_t* buf, const uint64_t* __restrict__ offs, uint64_t total,
+                                        uint64_t t0, uint64_t m, uint4* stage, uint64_t kh, uint64_t kl) {
+    const uint64_t i = t0 + threadIdx.x, t1 = t0 + blockDim.x < m ? t0 + blockDim.x : m;
+    const uint64_t lo = __ldg(offs + t0), hi = __ldg(offs + t1);
+    const uint64_t o0 = i < m ? __ldg(offs + i) : hi, o1 = i < m ? __ldg(offs + i + 1) : hi;
+    uint32_t at;
+    __syncthreads();  // the tile before has been read
+    const bool staged = stage_bytes(buf, total, lo, hi, stage, at);
+    __syncthreads();
+    Sig s{0, 0};
+    if (i < m) {
+        if (staged && o0 >= lo && o1 >= o0 && o1 <= hi)
+            s = sig_staged(stage, at + uint32_t(o0 - lo), uint32_t(o1 - o0), kh, kl);
+        else
+            s = sig_bytes(buf, total, o0, o1 - o0, kh, kl);
+    }
+    return s;
+}
+
 // ------------------------------------------------------- shard, local, edges
 
 // Shard = top h bits of the signature (Sec. 4).

@@ -20,13 +20,23 @@ __device__ __forceinline__ uint32_t cell_q(const uint8_t* data, int b, uint64_t 
     else return cell_get_nc(data, b, i);
 }
 
+// The answer of one key from its cells' XOR.
+template <bool FILTER>
+__device__ __forceinline__ void put_answer(void* out, uint64_t i, uint32_t r, uint64_t local, int b) {
+    if constexpr (FILTER) {
+        static_cast<uint8_t*>(out)[i] = uint8_t(r == fingerprint(local, b));
+    } else {
+        if (b <= 8) static_cast<uint8_t*>(out)[i] = uint8_t(r);
+        else if (b <= 16) static_cast<uint16_t*>(out)[i] = uint16_t(r);
+        else static_cast<uint32_t*>(out)[i] = r;
+    }
+}
+
 // K: vertices per edge (3, or 4 for a 4-uniform fuse graph).
-template <int WIDTH, bool FILTER, bool BYTES, int K>
-__global__ void __launch_bounds__(kQThreads) k_query(const void* __restrict__ keys, const uint64_t* __restrict__ offs,
-                                                     uint64_t m, Geom g, const uint8_t* __restrict__ data,
-                                                     void* __restrict__ out) {
+template <int WIDTH, bool FILTER, int K>
+__global__ void __launch_bounds__(kQThreads) k_query(const uint64_t* __restrict__ keys, uint64_t m, Geom g,
+                                                     const uint8_t* __restrict__ data, void* __restrict__ out) {
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    const uint64_t total = BYTES ? __ldg(offs + m) : 0;
     for (uint64_t i0 = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i0 < m; i0 += stride * kQ) {
         uint64_t idx[kQ], loc[kQ], cell[kQ][K];
         bool ok[kQ];
@@ -34,16 +44,8 @@ __global__ void __launch_bounds__(kQThreads) k_query(const void* __restrict__ ke
         for (int k = 0; k < kQ; k++) {
             idx[k] = i0 + uint64_t(k) * stride;
             ok[k] = idx[k] < m;
-            Sig s{0, 0};
-            if (ok[k]) {
-                if constexpr (BYTES) {
-                    uint64_t o0 = __ldg(offs + idx[k]), o1 = __ldg(offs + idx[k] + 1);
-                    s = sig_bytes(static_cast<const uint8_t*>(keys), total, o0, o1 - o0, g.kh, g.kl);
-                } else {
-                    // keys are read once: evict-first, so the cells they probe stay in L2
-                    s = sig_u64(__ldcs(static_cast<const uint64_t*>(keys) + idx[k]), g.kh, g.kl);
-                }
-            }
+            // keys are read once: evict-first, so the cells they probe stay in L2
+            const Sig s = ok[k] ? sig_u64(__ldcs(keys + idx[k]), g.kh, g.kl) : Sig{0, 0};
             uint64_t base = shard_of(s, g.h) * g.cells;
             loc[k] = local_of(s, g.h);
             uint64_t v[4];
@@ -61,33 +63,53 @@ __global__ void __launch_bounds__(kQThreads) k_query(const void* __restrict__ ke
             if (!ok[k]) continue;
             uint32_t r = x[k][0] ^ x[k][1] ^ x[k][2];
             if constexpr (K == 4) r ^= x[k][3];
-            if constexpr (FILTER) {
-                static_cast<uint8_t*>(out)[idx[k]] = uint8_t(r == fingerprint(loc[k], g.b));
-            } else {
-                if (g.b <= 8) static_cast<uint8_t*>(out)[idx[k]] = uint8_t(r);
-                else if (g.b <= 16) static_cast<uint16_t*>(out)[idx[k]] = uint16_t(r);
-                else static_cast<uint32_t*>(out)[idx[k]] = r;
-            }
+            put_answer<FILTER>(out, idx[k], r, loc[k], g.b);
         }
+    }
+}
+
+// Byte strings: a block takes tiles of consecutive strings through shared
+// memory (sig_tile) and probes one key a thread; the resident blocks keep
+// enough probes in flight.
+template <int WIDTH, bool FILTER, int K>
+__global__ void __launch_bounds__(kQThreads) k_query_bytes(const uint8_t* __restrict__ buf,
+                                                           const uint64_t* __restrict__ offs, uint64_t m, Geom g,
+                                                           const uint8_t* __restrict__ data, void* __restrict__ out) {
+    __shared__ uint4 stage[kStageBytes / 16];
+    const uint64_t total = __ldg(offs + m);
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < m; t0 += stride) {
+        const Sig s = sig_tile(buf, offs, total, t0, m, stage, g.kh, g.kl);
+        const uint64_t i = t0 + threadIdx.x;
+        if (i >= m) continue;
+        const uint64_t base = shard_of(s, g.h) * g.cells;
+        const uint64_t local = local_of(s, g.h);
+        uint64_t v[4];
+        edge_of(g, local, v);
+        uint32_t r = 0;
+#pragma unroll
+        for (int j = 0; j < K; j++) r ^= cell_q<WIDTH>(data, g.b, base + v[j]);
+        put_answer<FILTER>(out, i, r, local, g.b);
     }
 }
 
 template <int WIDTH, bool FILTER>
 static void launch_q(bool bytes, const void* keys, const uint64_t* offs, uint64_t m, const Geom& g,
                      const uint8_t* data, void* out, cudaStream_t st) {
-    uint64_t blocks = (m + uint64_t(kQThreads) * kQ - 1) / (uint64_t(kQThreads) * kQ);
+    const uint64_t per = uint64_t(kQThreads) * (bytes ? 1 : kQ);
+    uint64_t blocks = (m + per - 1) / per;
     uint64_t cap = uint64_t(num_sms()) * 16;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
+    const uint64_t* k64 = static_cast<const uint64_t*>(keys);
+    const uint8_t* k8 = static_cast<const uint8_t*>(keys);
     if (g.k == 4) {
-        if (bytes)
-            k_query<WIDTH, FILTER, true, 4><<<unsigned(blocks), kQThreads, 0, st>>>(keys, offs, m, g, data, out);
-        else
-            k_query<WIDTH, FILTER, false, 4><<<unsigned(blocks), kQThreads, 0, st>>>(keys, offs, m, g, data, out);
+        if (bytes) k_query_bytes<WIDTH, FILTER, 4><<<unsigned(blocks), kQThreads, 0, st>>>(k8, offs, m, g, data, out);
+        else k_query<WIDTH, FILTER, 4><<<unsigned(blocks), kQThreads, 0, st>>>(k64, m, g, data, out);
     } else if (bytes) {
-        k_query<WIDTH, FILTER, true, 3><<<unsigned(blocks), kQThreads, 0, st>>>(keys, offs, m, g, data, out);
+        k_query_bytes<WIDTH, FILTER, 3><<<unsigned(blocks), kQThreads, 0, st>>>(k8, offs, m, g, data, out);
     } else {
-        k_query<WIDTH, FILTER, false, 3><<<unsigned(blocks), kQThreads, 0, st>>>(keys, offs, m, g, data, out);
+        k_query<WIDTH, FILTER, 3><<<unsigned(blocks), kQThreads, 0, st>>>(k64, m, g, data, out);
     }
 }
 
