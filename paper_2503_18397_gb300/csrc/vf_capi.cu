@@ -414,35 +414,26 @@ vf_status solve_rounds(const vf_info& in, const vf::Geom& g, const uint64_t* loc
     return VF_OK;
 }
 
-// One attempt of the asynchronous fuse-regime solver. Returns VF_OK, VF_EBUILD
-// (peel failed: retry), or an error.
+// One attempt of the default fuse-regime solver: peeling by clusters of CTAs (with
+// enough shards) or by the worklist, then the dataflow assignment. Returns VF_OK, VF_EBUILD (peel failed: retry), or an error.
 vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, const uint32_t* val,
                      const unsigned long long* start, uint8_t* data, cudaStream_t st, uint64_t* peeled,
                      uint64_t cell_base, const uint32_t* drop, uint64_t ndrop, DevBuf* claimed_out,
                      const unsigned long long* seg_ends = nullptr) {
     const uint64_t n = in.n_eff;
     const uint64_t V = in.total_cells;
-    DevBuf W, queue, claimed, pv, rec, rec3, ctr;
+    DevBuf W, queue, claimed, rec, rec3, ctr;
     const bool own_incidence = seg_ends && vf::incidence_seg_fits(g);  // writes every vertex word
+    const uint64_t ewords = std::max<uint64_t>((n + 31) / 32, 1);
     VF_CK(W.alloc(V * 4, st));
-    if (!own_incidence) VF_CK(cudaMemsetAsync(W.p, 0, V * 4, st));
     VF_CK(queue.alloc(V * 8, st));
-    VF_CK(cudaMemsetAsync(queue.p, 0xFF, V * 8, st));
-    const uint64_t ewords = std::max<uint64_t>((n + 31) / 32, 1), vwords = std::max<uint64_t>((V + 31) / 32, 1);
     VF_CK(claimed.alloc(ewords * 4, st));
-    if (drop)  // dropped duplicates count as claimed: they are never peeled
-        VF_CK(cudaMemcpyAsync(claimed.p, drop, ewords * 4, cudaMemcpyDeviceToDevice, st));
-    else
-        VF_CK(cudaMemsetAsync(claimed.p, 0, ewords * 4, st));
-    VF_CK(pv.alloc(vwords * 4, st));
-    VF_CK(cudaMemsetAsync(pv.p, 0, vwords * 4, st));
     VF_CK(rec.alloc(std::max<uint64_t>(V, 1) * 16, st));  // one slot per item, at most one item per vertex
     if (g.k == 4) VF_CK(rec3.alloc(std::max<uint64_t>(V, 1) * 4, st));  // the third other vertex
     VF_CK(ctr.alloc(vf::kFlowWords * 4, st));
-    VF_CK(cudaMemsetAsync(ctr.p, 0, vf::kFlowWords * 4, st));
     DevBuf rc;  // record slots per shard, one 128-byte line each
-    VF_CK(rc.alloc(std::max<uint64_t>(in.shards, 1) * vf::kRcStride * 4, st));
-    VF_CK(cudaMemsetAsync(rc.p, 0, std::max<uint64_t>(in.shards, 1) * vf::kRcStride * 4, st));
+    const uint64_t rc_words = std::max<uint64_t>(in.shards, 1) * vf::kRcStride;
+    VF_CK(rc.alloc(rc_words * 4, st));
     vf::FlowArgs a;
     std::memset(&a, 0, sizeof a);
     a.loc = loc;
@@ -456,7 +447,6 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
     a.queue_cap = V;
     a.claimed = claimed.as<uint32_t>();
     a.claimed_bits = n;
-    a.pv = pv.as<uint32_t>();
     a.rec = rec.as<uint4>();
     a.rec3 = g.k == 4 ? rec3.as<uint32_t>() : nullptr;
     a.rc = rc.as<uint32_t>();
@@ -470,24 +460,68 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
     a.cell_base = cell_base;
     a.assign_limit = g_debug_assign_limit.load();
     a.stall = g_debug_stall_assign.load() ? 1u : 0u;
-    {
-        PhaseTimer t(kPhAccum, st);
-        if (own_incidence)
-            VF_CK(vf::launch_incidence_seg(loc, n, start, a.S, g, seg_ends, a.W, a.err, drop, false, st));
-        else
-            VF_CK(vf::launch_incidence32(loc, n, start, a.S, g, a.W, a.err, drop, st));
-    }
-    {
-        // per batch: (head rebase), initial items, worklist peel; then the peeled count
-        PhaseTimer t(kPhPeel, st, int(3 * vf::flow_batches(a)));
-        VF_CK(vf::launch_flow_peel(a, st));
-    }
     std::vector<uint32_t> h(vf::kFlowWords);
-    std::vector<uint32_t> hrc(std::max<uint64_t>(in.shards, 1) * vf::kRcStride);
-    VF_CK(cudaMemcpyAsync(h.data(), a.ctr, vf::kFlowWords * 4, cudaMemcpyDeviceToHost, st));
-    VF_CK(cudaMemcpyAsync(hrc.data(), rc.p, hrc.size() * 4, cudaMemcpyDeviceToHost, st));
-    VF_CK(cudaStreamSynchronize(st));
-    const uint32_t count = h[vf::kFlowPeeled], err = h[vf::kFlowErr];
+    std::vector<uint32_t> hrc(rc_words);
+    vf::FrontConfig fc;
+    DevBuf heads;
+    for (bool waves = vf::front_config(g, a.S, fc);; waves = false) {
+        if (!own_incidence) VF_CK(cudaMemsetAsync(W.p, 0, V * 4, st));
+        if (drop)  // dropped duplicates count as claimed: they are never peeled
+            VF_CK(cudaMemcpyAsync(claimed.p, drop, ewords * 4, cudaMemcpyDeviceToDevice, st));
+        else
+            VF_CK(cudaMemsetAsync(claimed.p, 0, ewords * 4, st));
+        VF_CK(cudaMemsetAsync(ctr.p, 0, vf::kFlowWords * 4, st));
+        VF_CK(cudaMemsetAsync(rc.p, 0, rc_words * 4, st));
+        {
+            PhaseTimer t(kPhAccum, st);
+            if (own_incidence)
+                VF_CK(vf::launch_incidence_seg(loc, n, start, a.S, g, seg_ends, a.W, a.err, drop, false, st));
+            else
+                VF_CK(vf::launch_incidence32(loc, n, start, a.S, g, a.W, a.err, drop, st));
+        }
+        if (waves) {
+            vf::FrontArgs f;
+            std::memset(&f, 0, sizeof f);
+            f.loc = loc;
+            f.val = val;
+            f.start = start;
+            f.S = a.S;
+            f.g = g;
+            f.W = a.W;
+            f.claimed = a.claimed;
+            f.rec = a.rec;
+            f.rec3 = a.rec3;
+            f.rc = a.rc;
+            f.lg_cta = uint32_t(31 - __builtin_clz(fc.cta));
+            f.lists = queue.as<uint2>();
+            f.list_cap = uint32_t(in.cells >> (f.lg_cta + 1));  // two buffers a CTA, half its share of the cells each
+            const uint64_t nl = (vf::kFrontHead + 1) * (in.shards << f.lg_cta), nr = (vf::kFrontHead + 1) * in.shards;
+            VF_CK(heads.alloc((nl + nr) * 4, st));
+            f.list_n = heads.as<uint32_t>();
+            f.rcv = f.list_n + nl;
+            VF_CK(cudaMemsetAsync(heads.p, 0, (nl + nr) * 4, st));
+            f.epsg = a.epsg;
+            f.ahead = 5;  // (none: +5% at 10^8 keys; 12: +3%)
+            f.err = a.ctr + vf::kFrontErr;
+            f.err_before = a.err;
+            PhaseTimer t(kPhPeel, st, int(vf::kFrontHead) + 3);  // scan, head rounds, waves; peeled count
+            VF_CK(vf::launch_front_peel(f, fc, st));
+            VF_CK(vf::launch_count_claims(a.claimed, n, a.ctr + vf::kFlowPeeled, st));
+        } else {
+            VF_CK(cudaMemsetAsync(queue.p, 0xFF, V * 8, st));
+            // per batch: (head rebase), initial items, worklist peel; then the peeled count
+            PhaseTimer t(kPhPeel, st, int(3 * vf::flow_batches(a)));
+            VF_CK(vf::launch_flow_peel(a, st));
+            VF_CK(vf::launch_count_claims(a.claimed, n, a.ctr + vf::kFlowPeeled, st));
+        }
+        VF_CK(cudaMemcpyAsync(h.data(), a.ctr, vf::kFlowWords * 4, cudaMemcpyDeviceToHost, st));
+        VF_CK(cudaMemcpyAsync(hrc.data(), rc.p, hrc.size() * 4, cudaMemcpyDeviceToHost, st));
+        VF_CK(cudaStreamSynchronize(st));
+        // a list beyond its room: the worklist takes the attempt alone, from the start
+        if (waves && ((h[vf::kFlowErr] | h[vf::kFrontErr]) & (vf::kErrFrontier | vf::kErrCapacity))) continue;
+        break;
+    }
+    const uint32_t count = h[vf::kFlowPeeled], err = h[vf::kFlowErr] | h[vf::kFrontErr];
     uint64_t slots = 0, rmax = 0;
     for (uint64_t s = 0; s < in.shards; s++) {
         slots += hrc[s * vf::kRcStride];

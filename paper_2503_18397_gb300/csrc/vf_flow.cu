@@ -315,13 +315,14 @@ __global__ void k_rebase_head(FlowArgs a) {
 }
 
 // Peeled edges = set claim bits.
-__global__ void __launch_bounds__(kFT) k_count_claims(FlowArgs a, uint64_t words) {
+__global__ void __launch_bounds__(kFT) k_count_claims(const uint32_t* __restrict__ claimed, uint64_t words,
+                                                      uint32_t* __restrict__ count) {
     uint32_t c = 0;
     for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < words; i += uint64_t(gridDim.x) * blockDim.x)
-        c += __popc(__ldg(a.claimed + i));
+        c += __popc(__ldg(claimed + i));
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, d);
-    if (lane32() == 0 && c) atomicAdd(a.ctr + kFlowPeeled, c);
+    if (lane32() == 0 && c) atomicAdd(count, c);
 }
 
 // Worklist peeling; one chain per lane at a time. An iteration has two memory
@@ -351,6 +352,9 @@ __global__ void __launch_bounds__(kFT) k_flow_peel(FlowArgs a) {
     uint32_t idle = 0;
     uint32_t dacc = 0;  // lane 0: ended chains not yet added to done
     unsigned nap = 32;
+    // A wrapped degree (only the incidence kernel reports it) makes every word
+    // worthless as an index: the attempt fails unpeeled.
+    if (dev_atomic32(*a.err).load(cuda::memory_order_relaxed) & kErrDegOverflow) return;
     for (;;) {
         const unsigned mhave = __ballot_sync(0xFFFFFFFFu, have);
         const bool need = !have && slot == ~0ull && mhave == 0;  // only an idle warp takes queue slots
@@ -410,7 +414,6 @@ __global__ void __launch_bounds__(kFT) k_flow_peel(FlowArgs a) {
             if (have) {
                 const uint64_t rs = uint64_t(rsh) * cells + rbase;
                 if (peeled) {
-                    atomicOr(a.pv + (v >> 5), 1u << (v & 31u));
                     const uint32_t s = rsh;  // v / cells, taken in phase 1
                     const uint32_t base = s * cells;
                     const unsigned long long st0 = __ldg(a.start + s);
@@ -580,10 +583,13 @@ __global__ void __launch_bounds__(kFT) k_flow_peel(FlowArgs a) {
 // -------------------------------------------------------------- assignment
 
 // Vertices no edge was peeled from are final with value 0; the others wait.
+// After a complete peel those are the vertices whose word is left at degree one
+// (an edge is removed from the other vertices, not from the one it was peeled
+// from); every other vertex has degree zero.
 __global__ void __launch_bounds__(kFT) k_final_init(FlowArgs a) {
     const uint64_t V = uint64_t(a.S) * a.g.cells;
     for (uint64_t v = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; v < V; v += uint64_t(gridDim.x) * blockDim.x)
-        a.fv[v] = (a.stall || ((__ldg(a.pv + (v >> 5)) >> (v & 31u)) & 1u)) ? 0ull : kFinal;
+        a.fv[v] = (a.stall || (__ldg(a.W + v) & 31u) == 1u) ? 0ull : kFinal;
 }
 
 // Dataflow assignment over the record slots, largest slot first within each
@@ -929,10 +935,12 @@ cudaError_t launch_flow_peel(const FlowArgs& a, cudaStream_t st) {
         if (a.g.k == 4) k_flow_peel<4><<<worker_grid(), kFT, 0, st>>>(a);
         else k_flow_peel<3><<<worker_grid(), kFT, 0, st>>>(a);
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const uint64_t words = (uint64_t(a.claimed_bits) + 31) / 32;
-    k_count_claims<<<grid_for(words), kFT, 0, st>>>(a, words);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_claims(const uint32_t* claimed, uint64_t edges, uint32_t* count, cudaStream_t st) {
+    const uint64_t words = (edges + 31) / 32;
+    k_count_claims<<<grid_for(words), kFT, 0, st>>>(claimed, words, count);
     return cudaGetLastError();
 }
 

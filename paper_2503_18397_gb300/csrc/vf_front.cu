@@ -1,0 +1,550 @@
+// Fuse-regime peeling of libvfunc (sm_103a), the waves: one cluster of CTAs per
+// shard in synchronous rounds over vertex words in L2, with one cluster-wide
+// exchange per round and no counter that more than one CTA takes.
+//
+// A fuse shard peels as two waves that move inward from its ends (Sec. 4.5):
+// about 8000 dependent rounds of ~1000 edges at 12.5M keys. The first
+// kFrontHead rounds, in which every degree-one vertex's short cascade is peeled
+// (a third of the edges), are launches of their own over all shards' lists. From
+// there on a round's latency counts, not bandwidth, and k_front_peel is built
+// around the round's dependent chain:
+//   claim bit and signature of the frontier's edges (one L2 trip, both in
+//   flight together, sent before the round's exchange is waited for)
+//   -> the edge's other vertices -> their fetch-and-adds (one L2 trip, whose
+//   results are the next frontier) -> the CTA's list in shared memory.
+// The exchange: every CTA sends its frontier's size to every CTA of the
+// cluster with st.async, which also completes that CTA's mbarrier: one one-way
+// message per pair orders the rounds, tells every CTA the round's total (the
+// exit test, equal in all CTAs) and where its records start (the sum of the
+// sizes before its own). No fence is needed: what a round hands to the next in
+// global memory is fetch-and-adds whose results have come back. (A
+// barrier.cluster with release and acquire costs ~650 cycles.)
+//
+// Vertex words, claims and records are the worklist solver's. An edge claimed
+// for a vertex at the end of round r is removed in round r+1. A round's
+// entries take the shard's record slots behind those of the rounds before, in
+// list order, empty where the claim failed. A vertex that an edge of round r
+// frees is peeled in a later round, so decreasing slot order is a reverse
+// peeling order, as the assignment needs it.
+//
+// The CTA whose fetch-and-add frees a vertex keeps it, so sizes drift apart
+// as the waves branch and die out; when one CTA holds more than twice the mean
+// (every CTA sees the same sizes), the round's pushes are dealt out over the
+// cluster through distributed shared memory, behind a full cluster barrier.
+//
+// Measured (one GB300, b = 8; peel per attempt, worklist -> this): 2^20 keys 4.37 ->
+// 3.55 ms, 10^8 (8 shards) 31.8 -> 26.0, 3*10^8 (16) 50.3 -> 30.9, 10^9 (64) 201 -> 88;
+// 4-uniform 10^8 15.2 -> 16.8, 3*10^8 56.9 -> 28.0. A round takes ~4300 cycles at 10^8:
+// ~1100 to the claims and signatures, ~1400 to the removals, ~450 waiting for
+// the slowest CTA, the rest between them (a remote fetch-and-add also costs an
+// SM ~3.3 cycles a lane, L2 or distributed shared memory alike, and a CTA has
+// ~64 entries a round). With many shards random DRAM sectors bound it: more
+// than 16 clusters at once gain little at 10^9 keys.
+#include <algorithm>
+#include <mutex>
+
+#include "vf_internal.h"
+
+namespace vf {
+
+constexpr int kFrWork = 256;            // threads that hold frontier entries
+constexpr int kFrT = kFrWork + 32;      // and the warp that exchanges the sizes
+constexpr uint32_t kFrList = 2048;      // frontier entries a CTA holds in shared memory, per buffer
+constexpr uint32_t kFrMaxC = 16;        // CTAs per cluster
+constexpr uint32_t kFrPolls = 1u << 26; // tests of an exchange's wait (some 20 ns each): then it gives up
+constexpr uint32_t kFrHole = 0xFFFFFFFFu;
+constexpr int kFrHeadT = 1024;          // threads of a head round's block (one block per list)
+constexpr uint32_t kFrHeadPer = 2;      // entries a thread has in flight there
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
+
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Stores v in a peer's shared memory and counts 4 bytes on the peer's mbarrier.
+__device__ __forceinline__ void post_u32(uint32_t remote, uint32_t v, uint32_t remote_mbar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(remote), "r"(v),
+                 "r"(remote_mbar)
+                 : "memory");
+}
+
+__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// A frontier entry on its way: vertex and edge (shard-local), the edge's
+// signature, value and claim word as it was, then its other vertices in edge order.
+template <int K>
+struct FrontItem {
+    uint64_t local;
+    uint32_t v, e, value, cold;
+    uint32_t o[K - 1];
+    bool on;  // holds an entry; after front_others: holds an edge to remove
+};
+
+// Claims the entry's edge and loads its signature (and value).
+template <int K, bool VAL>
+__device__ __forceinline__ void front_fetch(FrontItem<K>& x, const FrontArgs& a, uint2 ve, unsigned long long st0, uint32_t ns) {
+    x.v = ve.x;
+    x.e = ve.y;
+    x.on = ve.y < ns;
+    if (!x.on) {  // impossible for exact words: touch nothing
+        atomicOr(a.err, kErrCapacity);
+        return;
+    }
+    const uint32_t e = uint32_t(st0) + ve.y;  // a group holds fewer than 2^32 edges
+    x.cold = atomicOr(a.claimed + (e >> 5), 1u << (e & 31u));
+    x.local = __ldg(a.loc + e);
+    if (VAL) x.value = __ldg(a.val + e);
+}
+
+template <int K>
+__device__ __forceinline__ void front_others(FrontItem<K>& x, const Geom& g, unsigned long long st0) {
+    const uint32_t lgs = uint32_t(g.lg_seg), smask = (1u << lgs) - 1u;
+    const uint32_t v0 = uint32_t(mulhi(x.local, g.span));
+    const uint32_t s1 = (v0 >> lgs) + 1u;
+    const uint64_t rm = mix64(x.local ^ kEdgeSalt);
+    uint32_t vv[K];
+    vv[0] = v0;
+    vv[1] = (s1 << lgs) + (uint32_t(rm) & smask);
+    vv[2] = ((s1 + 1u) << lgs) + (uint32_t(rm >> 32) & smask);
+    if constexpr (K == 4) vv[3] = ((s1 + 2u) << lgs) + (uint32_t(mix64(x.local ^ kEdgeSalt2)) & smask);
+    bool past = false;
+#pragma unroll
+    for (int k = 0; k < K - 1; k++) {
+        past = past || vv[k] == x.v;
+        x.o[k] = past ? vv[k + 1] : vv[k];
+    }
+    x.on = !((x.cold >> ((uint32_t(st0) + x.e) & 31u)) & 1u);
+}
+
+// The entry's record, in shard slot `slot`.
+template <int K, bool VAL>
+__device__ __forceinline__ void front_record(const FrontItem<K>& x, const FrontArgs& a, uint32_t base, uint32_t cells, uint32_t slot) {
+    if (slot >= cells) return;  // at most one entry per vertex: impossible, and reported by the caller
+    uint4* const rec = a.rec + base + slot;
+    if (x.on) {
+        *rec = make_uint4(base + x.v, base + x.o[0], base + x.o[1],
+                          VAL ? x.value : fingerprint_slice(x.local, a.g.b, a.g.fpb, a.g.fps));
+        if constexpr (K == 4) a.rec3[uint64_t(base) + slot] = base + x.o[2];
+    } else {
+        rec->x = kFrHole;
+    }
+}
+
+// ------------------------------------------------------------------ head
+
+// List `list` (shard s, rank k of lg_cta: list s * C + k), buffer buf.
+__device__ __forceinline__ uint2* front_list(const FrontArgs& a, uint32_t list, uint32_t buf) {
+    return a.lists + (uint64_t(list) * 2 + buf) * a.list_cap;
+}
+
+// Round 0: the vertices of degree one, each list those of its share of the cells.
+__global__ void __launch_bounds__(kFrHeadT) k_front_scan(FrontArgs a) {
+    __shared__ uint32_t s_cnt;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    const uint32_t C = 1u << a.lg_cta, list = blockIdx.x, s = list >> a.lg_cta, rank = list & (C - 1u);
+    const uint32_t cells = uint32_t(a.g.cells), quads = cells / 4;
+    if (tid == 0) s_cnt = 0;
+    __syncthreads();
+    const uint4* const W4 = reinterpret_cast<const uint4*>(a.W + uint64_t(s) * cells);
+    const uint32_t per = (quads + C - 1) / C, q0 = min(quads, rank * per), q1 = min(quads, q0 + per);
+    uint2* const out = front_list(a, list, 0);
+    for (uint32_t c = q0 + (tid & ~31u); c < q1; c += kFrHeadT) {
+        const uint32_t q = c + lane;
+        const uint4 w = q < q1 ? __ldcg(W4 + q) : make_uint4(0, 0, 0, 0);
+        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+        uint32_t mine = 0;
+#pragma unroll
+        for (int j = 0; j < 4; j++) mine += (ws[j] & 31u) == 1u;
+        uint32_t incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if (lane >= uint32_t(d)) incl += y;
+        }
+        uint32_t at = 0;
+        if (lane == 31 && incl) at = atomicAdd(&s_cnt, incl);
+        at = __shfl_sync(0xFFFFFFFFu, at, 31) + incl - mine;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if ((ws[j] & 31u) == 1u) {
+                if (at < a.list_cap) out[at] = make_uint2(4u * q + j, ws[j] >> 5);
+                else atomicOr(a.err, kErrFrontier);
+                at++;
+            }
+    }
+    __syncthreads();
+    if (tid == 0) a.list_n[list] = min(s_cnt, a.list_cap);
+}
+
+// Round r of every list: entries in buffer r & 1, list_n[r], records behind rcv[r].
+template <int K, bool VAL>
+__global__ void __launch_bounds__(kFrHeadT) k_front_head(FrontArgs a, uint32_t r) {
+    __shared__ uint32_t s_cnt;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, below = (1u << lane) - 1u;
+    const uint32_t C = 1u << a.lg_cta, list = blockIdx.x, s = list >> a.lg_cta, rank = list & (C - 1u);
+    const uint32_t lists = a.S << a.lg_cta;
+    // Degrees that wrapped in the incidence make every word worthless as an index.
+    if (*reinterpret_cast<const volatile uint32_t*>(a.err_before) != 0) return;
+    if (tid == 0) s_cnt = 0;
+    __syncthreads();
+    const uint32_t cells = uint32_t(a.g.cells), base = s * cells;
+    const uint32_t* const cnt = a.list_n + uint64_t(r) * lists;
+    const uint32_t sz = lane < C ? __ldcg(cnt + (s << a.lg_cta) + lane) : 0u;
+    const uint32_t before = __ldcg(a.rcv + uint64_t(r) * a.S + s);
+    const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz);
+    const uint32_t at = before + __reduce_add_sync(0xFFFFFFFFu, lane < rank ? sz : 0u);
+    const uint32_t n = __shfl_sync(0xFFFFFFFFu, sz, rank);
+    const unsigned long long st0 = __ldg(a.start + s);
+    const uint32_t ns = uint32_t(__ldg(a.start + s + 1) - st0);
+    uint32_t* const W = a.W + base;
+    const uint2* const in = front_list(a, list, r & 1u);
+    uint2* const out = front_list(a, list, (r + 1) & 1u);
+    if (rank == 0 && tid == 0) {
+        a.rcv[uint64_t(r + 1) * a.S + s] = before + total;
+        if (before + total > cells) atomicOr(a.err, kErrFrontier);
+    }
+    for (uint32_t i0 = tid & ~31u; i0 < n; i0 += kFrHeadT * kFrHeadPer) {
+        FrontItem<K> x[kFrHeadPer];
+        uint32_t w[kFrHeadPer][K - 1];
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++) {
+            const uint32_t i = i0 + j * kFrHeadT + lane;
+            x[j].on = false;
+            if (i < n) front_fetch<K, VAL>(x[j], a, __ldcg(in + i), st0, ns);
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++) {
+            if (x[j].on) front_others(x[j], a.g, st0);
+#pragma unroll
+            for (int k = 0; k < K - 1; k++)
+                w[j][k] = x[j].on ? atomicAdd(W + x[j].o[k], 0u - (1u + (x[j].e << 5))) : 0u;
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++) {
+            const uint32_t i = i0 + j * kFrHeadT + lane;
+            if (i < n) front_record<K, VAL>(x[j], a, base, cells, at + i);
+#pragma unroll
+            for (int k = 0; k < K - 1; k++) {
+                const uint32_t nw = w[j][k] - (1u + (x[j].e << 5));
+                const bool free_v = x[j].on && (nw & 31u) == 1u;
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, free_v);
+                if (!m) continue;
+                uint32_t to = 0;
+                if (lane == 0) to = atomicAdd(&s_cnt, uint32_t(__popc(m)));
+                to = __shfl_sync(0xFFFFFFFFu, to, 0) + __popc(m & below);
+                if (free_v) {
+                    if (to < a.list_cap) out[to] = make_uint2(x[j].o[k], nw >> 5);
+                    else atomicOr(a.err, kErrFrontier);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) a.list_n[uint64_t(r + 1) * lists + list] = min(s_cnt, a.list_cap);
+}
+
+// ------------------------------------------------------------------ waves
+
+// An entry for CTA `peer` of the cluster: its next list is list[] here, cnt its counter (rare: kept out of line).
+__device__ __noinline__ void front_deal(const FrontArgs& a, uint32_t cnt, uint32_t list, uint2* beyond, uint32_t peer, uint2 ve) {
+    uint32_t ps;
+    asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], 1;"
+                 : "=r"(ps)
+                 : "r"(map_to_cta(cnt, peer))
+                 : "memory");
+    if (ps < kFrList) {
+        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(map_to_cta(list + 8u * ps, peer)), "r"(ve.x), "r"(ve.y)
+                     : "memory");
+    } else if (ps < a.list_cap) {
+        beyond[ps] = ve;
+    } else {
+        atomicOr(a.err, kErrFrontier);
+    }
+}
+
+struct FrontShared {
+    uint2 list[2][kFrList];                    // (vertex, edge), both shard-local
+    __align__(16) uint32_t size[2][kFrMaxC];   // frontier sizes of the round, one per CTA
+    __align__(8) unsigned long long mbar[2];   // exchange of even and of odd rounds
+    uint32_t cnt[3];                           // frontier counts; round r counts its next one in cnt[(r + 1) % 3]
+    uint32_t deal;                             // entries dealt out by this CTA so far
+    uint32_t total[2], most[2];                // of the exchange of even and odd rounds: all entries, the largest CTA's
+    uint32_t fail;                             // a wait gave up
+};
+
+// K: vertices per edge (3, or 4 for a 4-uniform fuse graph). VAL: a function.
+template <int K, bool VAL>
+__global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
+    __shared__ FrontShared sh;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, below = (1u << lane) - 1u;
+    uint32_t rank, C, cid, ncl;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(cid));
+    asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(ncl));
+    // What earlier launches reported (the same in all CTAs) voids the attempt.
+    if (*reinterpret_cast<const volatile uint32_t*>(a.err_before) != 0) return;
+    const uint32_t cells = uint32_t(a.g.cells);
+    const uint32_t lgs = uint32_t(a.g.lg_seg);
+    const bool exchanger = warp == kFrWork / 32;
+    const uint32_t mbar_addr = smem_u32(&sh.mbar[0]);
+    // where this CTA's size goes in the CTA of this lane's number, and that CTA's mbarrier
+    const uint32_t to_size = map_to_cta(smem_u32(&sh.size[0][rank]), lane < C ? lane : 0u);
+    const uint32_t to_mbar = map_to_cta(mbar_addr, lane < C ? lane : 0u);
+    if (tid == 0) {
+        for (int j = 0; j < 2; j++)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_addr + 8u * j) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        sh.deal = sh.fail = 0;
+    }
+    uint32_t xr = 0;  // exchanges so far: mbar[xr & 1], whose phase parity is (xr >> 1) & 1
+    bool failed = false;
+    for (uint32_t s = cid; s < a.S && !failed; s += ncl) {
+        const uint32_t base = s * cells;
+        const unsigned long long st0 = __ldg(a.start + s);
+        const uint32_t ns = uint32_t(__ldg(a.start + s + 1) - st0);
+        uint32_t* const W = a.W + base;
+        // a list beyond shared memory goes on at the same index of this CTA's list of the head
+        uint2* const list0 = front_list(a, s * C + rank, 0);
+        auto put = [&](uint32_t buf, uint32_t i, uint2 x) {
+            if (i < kFrList) sh.list[buf][i] = x;
+            else if (i < a.list_cap) list0[buf * a.list_cap + i] = x;
+            else atomicOr(a.err, kErrFrontier);
+        };
+        // kFrontHead is even: the head left its entries in buffer 0
+        const uint32_t left = __ldcg(a.list_n + uint64_t(kFrontHead) * (a.S << a.lg_cta) + s * C + rank);
+        for (uint32_t i = tid; i < left && i < kFrList; i += kFrT) sh.list[0][i] = __ldcg(list0 + i);
+        if (tid < 3) sh.cnt[tid] = tid == 0 ? left : 0u;
+        __syncthreads();
+        cluster_barrier();  // every CTA's counters (and at first its mbarriers) are ready
+        uint32_t before = __ldcg(a.rcv + uint64_t(kFrontHead) * a.S + s);  // record slots taken so far
+        // segments whose words and signatures have been asked for: [0, pf_lo) and (pf_hi, T)
+        int pf_lo = 0, pf_hi = int(cells >> lgs) - 1;
+        uint32_t c0 = 0, c1 = 1, c2 = 2;  // r % 3, (r + 1) % 3, (r + 2) % 3
+        for (uint32_t cur = 0;; cur ^= 1u) {
+            uint32_t n = sh.cnt[c0];
+            n = min(n, max(a.list_cap, kFrList));
+            const uint32_t p = xr & 1u, parity = (xr >> 1) & 1u, mb = mbar_addr + 8u * p;
+            xr++;
+            if (exchanger) {
+                if (lane < C) post_u32(to_size + 4u * kFrMaxC * p, n, to_mbar + 8u * p);
+                if (lane == 0) {
+                    sh.cnt[c2] = 0;  // last read a round ago; pushed to from the next round on
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(4u * C)
+                                 : "memory");
+                }
+                if (n > 0) {
+                    // while the sizes are on their way: what the waves reach next comes to L2
+                    const bool have = lane < n;
+                    const uint32_t sg = have ? sh.list[cur][lane].x >> lgs : 0u;
+                    const uint32_t T = cells >> lgs;
+                    const unsigned ml = __ballot_sync(0xFFFFFFFFu, have && sg < T / 2);
+                    const unsigned mr = __ballot_sync(0xFFFFFFFFu, have && sg >= T / 2);
+                    const int suml = int(__reduce_add_sync(0xFFFFFFFFu, have && sg < T / 2 ? sg : 0u));
+                    const int sumr = int(__reduce_add_sync(0xFFFFFFFFu, have && sg >= T / 2 ? sg : 0u));
+                    int t = -1;
+                    if (ml && pf_lo < int(T) && (pf_lo - int(a.ahead)) * __popc(ml) <= suml) t = pf_lo++;
+                    else if (mr && pf_hi >= 0 && (pf_hi + int(a.ahead)) * __popc(mr) >= sumr) t = pf_hi--;
+                    if (t >= 0 && lane == 0) {
+                        const uint32_t part = (1u << lgs) >> a.lg_cta;  // words of this CTA's share
+                        if (part >= 32)
+                            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(W + (uint32_t(t) << lgs) + rank * part),
+                                         "r"(part * 4u)
+                                         : "memory");
+                        const uint32_t pe = a.epsg >> a.lg_cta;  // of ~epsg edges that start in a segment
+                        const uint64_t e0 = (st0 + uint64_t(t) * a.epsg + rank * pe) & ~uint64_t(1);
+                        const uint32_t bytes = (pe * 8u) & ~15u;
+                        if (bytes && e0 + bytes / 8 <= st0 + ns)
+                            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.loc + e0), "r"(bytes) : "memory");
+                    }
+                }
+                uint32_t polls = 0;
+                while (!mbar_try(mb, parity)) {
+                    if (++polls > kFrPolls) {
+                        sh.fail = 1;
+                        break;
+                    }
+                }
+                const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
+                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz), most = __reduce_max_sync(0xFFFFFFFFu, sz);
+                if (lane == 0) sh.total[p] = total, sh.most[p] = most;
+            } else {
+                uint32_t i = tid;
+                FrontItem<K> x;
+                x.on = false;
+                auto entry = [&]() { return i < kFrList ? sh.list[cur][i] : __ldcg(list0 + cur * a.list_cap + i); };
+                if (i < n) front_fetch<K, VAL>(x, a, entry(), st0, ns);
+                if (x.on) front_others(x, a.g, st0);
+                uint32_t polls = 0;
+                while (!mbar_try(mb, parity)) {
+                    if (++polls > kFrPolls) {
+                        sh.fail = 1;
+                        break;
+                    }
+                }
+                uint32_t at = 0;
+                bool deal = false;
+                for (uint32_t i0 = 32u * warp; i0 < n; i0 += kFrWork) {
+                    uint32_t w[K - 1];
+                    const uint32_t dec = 1u + (x.e << 5);
+#pragma unroll
+                    for (int k = 0; k < K - 1; k++) w[k] = x.on ? atomicAdd(W + x.o[k], 0u - dec) : 0u;
+                    if (i0 == 32u * warp) {  // while the removals are on their way: where the round's records go
+                        const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
+                        const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz);
+                        at = before + __reduce_add_sync(0xFFFFFFFFu, lane < rank ? sz : 0u);
+                        deal = __reduce_max_sync(0xFFFFFFFFu, sz) > 2u * (total >> a.lg_cta) + 64u;
+                    }
+                    if (i < n) front_record<K, VAL>(x, a, base, cells, at + i);
+                    // the vertices left at degree one join the next list
+                    unsigned m[K - 1];
+                    uint32_t all = 0;
+#pragma unroll
+                    for (int k = 0; k < K - 1; k++) {
+                        w[k] -= dec;
+                        m[k] = __ballot_sync(0xFFFFFFFFu, x.on && (w[k] & 31u) == 1u);
+                        all += __popc(m[k]);
+                    }
+                    if (all) {
+                        uint32_t to = 0;
+                        if (lane == 0) to = atomicAdd(deal ? &sh.deal : &sh.cnt[c1], all);
+                        to = __shfl_sync(0xFFFFFFFFu, to, 0);
+#pragma unroll
+                        for (int k = 0; k < K - 1; k++) {
+                            if ((m[k] >> lane) & 1u) {
+                                const uint32_t slot = to + __popc(m[k] & below);
+                                const uint2 ve = make_uint2(x.o[k], w[k] >> 5);
+                                if (!deal) {
+                                    put(cur ^ 1u, slot, ve);
+                                } else {  // to the CTAs of the cluster in turn
+                                    const uint32_t peer = (slot + rank) & (C - 1u);
+                                    front_deal(a, smem_u32(&sh.cnt[c1]), smem_u32(&sh.list[cur ^ 1u][0]),
+                                               front_list(a, s * C + peer, cur ^ 1u), peer, ve);
+                                }
+                            }
+                            to += __popc(m[k]);
+                        }
+                    }
+                    i += kFrWork;
+                    x.on = false;
+                    if (i < n) {
+                        front_fetch<K, VAL>(x, a, entry(), st0, ns);
+                        if (x.on) front_others(x, a.g, st0);
+                    }
+                }
+            }
+            __syncthreads();
+            // equal in every CTA of the cluster, and so are the ways out below
+            const uint32_t total = sh.total[p];
+            if (sh.fail) {
+                failed = true;
+                if (tid == 0) atomicOr(a.err, kErrTimeout);
+                break;
+            }
+            if (total == 0) {
+                if (rank == 0 && tid == 0) a.rc[s * kRcStride] = before;
+                break;
+            }
+            before += total;
+            if (before > cells) {
+                if (tid == 0) atomicOr(a.err, kErrFrontier);
+                break;
+            }
+            if (sh.most[p] > 2u * (total >> a.lg_cta) + 64u) cluster_barrier();  // this round's pushes were dealt out
+            const uint32_t t = c0;
+            c0 = c1, c1 = c2, c2 = t;
+        }
+        cluster_barrier();  // no CTA starts the next shard (or leaves) while a peer still works on this one
+    }
+}
+
+// ------------------------------------------------------------------ launches
+
+static const void* front_kernel(const Geom& g) {
+    const bool val = g.kind == 0;
+    if (g.k == 4)
+        return val ? reinterpret_cast<const void*>(k_front_peel<4, true>) : reinterpret_cast<const void*>(k_front_peel<4, false>);
+    return val ? reinterpret_cast<const void*>(k_front_peel<3, true>) : reinterpret_cast<const void*>(k_front_peel<3, false>);
+}
+
+static cudaLaunchConfig_t front_launch(unsigned cta, unsigned clusters, cudaStream_t st, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(cta * clusters);
+    lc.blockDim = dim3(kFrT);
+    lc.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cta;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
+    at[1].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
+    lc.attrs = at;
+    lc.numAttrs = 2;
+    return lc;
+}
+
+bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg) {
+    if (g.regime != kRegimeFuse || (g.k != 3 && g.k != 4) || g.lg_seg < 5 || g.lg_seg > 26) return false;
+    static std::mutex mu;
+    static FrontConfig known[4][64];  // per kernel and device: cta = 0 unknown, ~0u not able
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    const void* fn = front_kernel(g);
+    std::lock_guard<std::mutex> lock(mu);
+    FrontConfig& k = known[(g.k == 4 ? 2 : 0) + (g.kind == 0 ? 1 : 0)][dev];
+    if (k.cta == 0) {
+        k.cta = ~0u;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+        for (unsigned c : {kFrMaxC, 8u}) {
+            cudaLaunchAttribute at[2]{};
+            const cudaLaunchConfig_t lc = front_launch(c, 1, nullptr, at);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, fn, &lc) == cudaSuccess && n > 0) {
+                k.cta = c;
+                k.clusters = unsigned(n);
+                break;
+            }
+            cudaGetLastError();
+        }
+    }
+    if (k.cta == ~0u) return false;
+    cfg.cta = k.cta;
+    cfg.clusters = std::max(1u, std::min(S, k.clusters));
+    return true;
+}
+
+cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaStream_t st) {
+    const unsigned lists = a.S << a.lg_cta;
+    k_front_scan<<<lists, kFrHeadT, 0, st>>>(a);
+    for (uint32_t r = 0; r < kFrontHead; r++) {
+        if (a.g.k == 4) {
+            if (a.g.kind == 0) k_front_head<4, true><<<lists, kFrHeadT, 0, st>>>(a, r);
+            else k_front_head<4, false><<<lists, kFrHeadT, 0, st>>>(a, r);
+        } else {
+            if (a.g.kind == 0) k_front_head<3, true><<<lists, kFrHeadT, 0, st>>>(a, r);
+            else k_front_head<3, false><<<lists, kFrHeadT, 0, st>>>(a, r);
+        }
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[2]{};
+    const cudaLaunchConfig_t lc = front_launch(cfg.cta, cfg.clusters, st, at);
+    void* args[] = {const_cast<FrontArgs*>(&a)};
+    return cudaLaunchKernelExC(&lc, front_kernel(a.g), args);
+}
+
+}  // namespace vf

@@ -110,6 +110,7 @@ enum : uint32_t {
     kFlowNext = 128,    // u64: assignment: next record position to take
     kFlowPeeled = 160,  // edges peeled
     kFlowErr = 192,     // error bits
+    kFrontErr = 193,    // error bits of the cluster kernel
     kFlowWords = 224
 };
 constexpr uint32_t kRcStride = 32;  // per-shard record counters, one 128-byte line each
@@ -126,7 +127,6 @@ struct FlowArgs {
     uint64_t queue_cap;
     uint32_t* claimed;                // one bit per edge
     uint64_t claimed_bits;            // edges
-    uint32_t* pv;                     // one bit per vertex: an edge was peeled from it
     uint4* rec;                       // per slot {peeled vertex, other, other, value}; x = ~0: empty;
                                       // shard s owns slots [s*cells, (s+1)*cells)
     uint32_t* rec3;                   // k = 4: per slot the third other vertex (else NULL)
@@ -166,6 +166,8 @@ cudaError_t launch_find_dups(const uint64_t* loc, const uint32_t* val, uint64_t 
 // Peels the shards in batches whose waves fit in L2 (flow_batches launches
 // of initial items + worklist peel), then counts the peeled edges.
 cudaError_t launch_flow_peel(const FlowArgs& a, cudaStream_t st);
+// Edges whose claim bit is set, added to *count.
+cudaError_t launch_count_claims(const uint32_t* claimed, uint64_t edges, uint32_t* count, cudaStream_t st);
 uint32_t flow_batches(const FlowArgs& a);
 cudaError_t launch_flow_assign(const FlowArgs& a, cudaStream_t st);
 // Counting sort of each shard's edges by the segment of their first vertex
@@ -175,6 +177,38 @@ cudaError_t launch_segment_order(const uint64_t* loc, const uint32_t* val, uint6
                                  const unsigned long long* start, uint32_t S, const Geom& g, unsigned long long* counts,
                                  uint64_t* loc_out, uint32_t* val_out, cudaStream_t st);
 uint64_t segment_order_bins(const Geom& g, uint32_t S);
+
+// Peeling of fuse shards in synchronous rounds, the waves by a cluster of CTAs
+// per shard (csrc/vf_front.cu); words, claims and records as the worklist solver's.
+constexpr uint32_t kFrontHead = 8;    // rounds before the waves (even), a launch each
+struct FrontConfig {
+    unsigned cta = 0, clusters = 0;   // CTAs per cluster, clusters of the launch
+};
+struct FrontArgs {
+    const uint64_t* loc;              // as FlowArgs
+    const uint32_t* val;
+    const unsigned long long* start;
+    uint32_t S;
+    Geom g;
+    uint32_t* W;
+    uint32_t* claimed;
+    uint4* rec;
+    uint32_t* rec3;
+    uint32_t* rc;
+    uint2* lists;                     // frontier entries (vertex, edge), shard-local: two buffers of list_cap for
+    uint32_t list_cap;                //   each CTA of each shard's cluster
+    uint32_t* list_n;                 // their numbers, by head round ((kFrontHead + 1) * S * CTAs)
+    uint32_t* rcv;                    // record slots taken per shard, by head round ((kFrontHead + 1) * S; first row zero)
+    uint32_t epsg;                    // edges per start segment
+    uint32_t ahead;                   // segments ahead of a wave's middle that are brought to L2
+    uint32_t lg_cta;                  // lg of the cluster size
+    uint32_t* err;                    // error bits
+    const uint32_t* err_before;       // error bits of the incidence
+};
+// The launch's shape for S shards; false where the kernel does not apply (other
+// regimes, few shards, or a device without such clusters).
+bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg);
+cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaStream_t st);
 
 // Fuse-regime wave solver (csrc/vf_wave.cu): 64-bit vertex words that hold the
 // degree, the other two vertices and the value of the edges' sum; phase I in
