@@ -37,8 +37,8 @@
 // shuffle.
 //
 // Assignment is a dataflow in decreasing slot order per shard: once final, a
-// vertex's value word (64 bits, in the queue's memory) holds its value with bit
-// 32 set (vertices no edge was peeled from are final from the start, value 0);
+// vertex's value word (16 to 64 bits, in the queue's memory) holds its value with
+// its final bit set (vertices no edge was peeled from are final from the start, value 0);
 // an edge waits (bounded) until its two other vertices are final. An edge only
 // waits on edges of its shard with larger slots, which were handed out before
 // it, so the earliest unfinished edge can always proceed.
@@ -52,7 +52,9 @@ namespace vf {
 
 constexpr int kFT = 256;
 constexpr unsigned long long kEmpty = ~0ull;
-constexpr unsigned long long kFinal = 1ull << 32;
+// Value words of the assignment: the value below one bit that says it is final,
+// in the narrowest word that holds both.
+template <class FV> constexpr FV kFinal = FV(1) << (sizeof(FV) == 8 ? 32 : 8 * sizeof(FV) - 1);
 constexpr uint32_t kHole = 0xFFFFFFFFu;     // record of an item whose claim failed
 constexpr uint32_t kIdleLimit = 1u << 23;  // polls of ~1 us: a wait gives up after ~8 s
 constexpr unsigned kNapMax = 512;          // ns, peeling (idle lanes; 256 -> 512 ns: -0.7%)
@@ -586,10 +588,12 @@ __global__ void __launch_bounds__(kFT) k_flow_peel(FlowArgs a) {
 // After a complete peel those are the vertices whose word is left at degree one
 // (an edge is removed from the other vertices, not from the one it was peeled
 // from); every other vertex has degree zero.
+template <class FV>
 __global__ void __launch_bounds__(kFT) k_final_init(FlowArgs a) {
     const uint64_t V = uint64_t(a.S) * a.g.cells;
+    FV* const fv = static_cast<FV*>(a.fv);
     for (uint64_t v = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; v < V; v += uint64_t(gridDim.x) * blockDim.x)
-        a.fv[v] = (a.stall || (__ldg(a.W + v) & 31u) == 1u) ? 0ull : kFinal;
+        fv[v] = (a.stall || (__ldg(a.W + v) & 31u) == 1u) ? FV(0) : kFinal<FV>;
 }
 
 // Dataflow assignment over the record slots, largest slot first within each
@@ -598,8 +602,10 @@ __global__ void __launch_bounds__(kFT) k_final_init(FlowArgs a) {
 // together; 2.5% faster than interleaving single records), so every shard's
 // dataflow advances at once; a record waits only on larger slots of its own
 // shard, which come at smaller positions.
-template <int K>
+template <int K, class FV>
 __global__ void __launch_bounds__(kFT) k_flow_assign(FlowArgs a) {
+    using word = cuda::atomic_ref<FV, cuda::thread_scope_device>;
+    FV* const fv = static_cast<FV*>(a.fv);
     const int b = a.g.b;
     const uint64_t count = ((a.rmax + 31) & ~uint64_t(31)) * a.S;
     const uint64_t cells = a.g.cells;
@@ -631,13 +637,12 @@ __global__ void __launch_bounds__(kFT) k_flow_assign(FlowArgs a) {
         bool fail = false;
         for (;;) {
             if (!done) {
-                const unsigned long long wy = dev_atomic64(a.fv[r.y]).load(cuda::memory_order_relaxed);
-                const unsigned long long wz = dev_atomic64(a.fv[r.z]).load(cuda::memory_order_relaxed);
-                const unsigned long long w3 =
-                    K == 4 && r3 != kHole ? dev_atomic64(a.fv[r3]).load(cuda::memory_order_relaxed) : kFinal;
-                if (wy & wz & w3 & kFinal) {
+                const FV wy = word(fv[r.y]).load(cuda::memory_order_relaxed);
+                const FV wz = word(fv[r.z]).load(cuda::memory_order_relaxed);
+                const FV w3 = K == 4 && r3 != kHole ? word(fv[r3]).load(cuda::memory_order_relaxed) : kFinal<FV>;
+                if (wy & wz & w3 & kFinal<FV>) {
                     const uint32_t x = (r.w ^ uint32_t(wy) ^ uint32_t(wz) ^ uint32_t(w3)) & vmask;
-                    dev_atomic64(a.fv[r.x]).store(kFinal | x, cuda::memory_order_relaxed);
+                    word(fv[r.x]).store(FV(kFinal<FV> | x), cuda::memory_order_relaxed);
                     cell_put_zero(a.data, b, a.cell_base + r.x, x);
                     done = true;
                 }
@@ -944,13 +949,29 @@ cudaError_t launch_count_claims(const uint32_t* claimed, uint64_t edges, uint32_
     return cudaGetLastError();
 }
 
-cudaError_t launch_flow_assign(const FlowArgs& a, cudaStream_t st) {
-    k_final_init<<<grid_for(uint64_t(a.S) * a.g.cells), kFT, 0, st>>>(a);
+template <class FV>
+static cudaError_t launch_assign_words(const FlowArgs& a, cudaStream_t st) {
+    k_final_init<FV><<<grid_for(uint64_t(a.S) * a.g.cells), kFT, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || a.nrec == 0 || a.rmax == 0) return e;
-    if (a.g.k == 4) k_flow_assign<4><<<assign_grid(a.g), kFT, 0, st>>>(a);
-    else k_flow_assign<3><<<assign_grid(a.g), kFT, 0, st>>>(a);
+    if (a.g.k == 4) k_flow_assign<4, FV><<<assign_grid(a.g), kFT, 0, st>>>(a);
+    else k_flow_assign<3, FV><<<assign_grid(a.g), kFT, 0, st>>>(a);
     return cudaGetLastError();
+}
+
+// While the 64-bit words of the ~12 segments that each of a shard's two waves is in
+// stay in L2, they are taken (16-bit words put more waiting vertices on a
+// sector: 2^20 keys 1.08 -> 1.18 ms, 4-uniform 10^8 7.3 -> 8.3 ms). Beyond that
+// the narrowest word that holds b bits and the final bit is (10^9 keys, b = 8,
+// 0.8 GB of such 64-bit words: 90 -> 62 ms; 10^8, 50 MB: 10.1 -> 9.9 ms).
+constexpr uint64_t kWideWordsMB = 48;
+
+cudaError_t launch_flow_assign(const FlowArgs& a, cudaStream_t st) {
+    const uint64_t hot = a.g.regime == kRegimeFuse ? (uint64_t(a.S) * 24 * 8) << a.g.lg_seg : uint64_t(a.S) * a.g.cells * 8;
+    if (hot <= kWideWordsMB << 20) return launch_assign_words<unsigned long long>(a, st);
+    if (a.g.b < 16) return launch_assign_words<unsigned short>(a, st);
+    if (a.g.b < 32) return launch_assign_words<unsigned int>(a, st);
+    return launch_assign_words<unsigned long long>(a, st);
 }
 
 cudaError_t launch_segment_order(const uint64_t* loc, const uint32_t* val, uint64_t n,

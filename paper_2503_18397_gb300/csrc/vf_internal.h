@@ -122,8 +122,7 @@ struct FlowArgs {
     Geom g;
     uint32_t* W;                      // S*cells vertex words (degree, sum of edge indices)
     unsigned long long* queue;        // work items (vertex << 32 | edge); all ones = empty
-    unsigned long long* fv;           // assignment: S*cells value words, value | 1 << 32 once final
-                                      // (the queue's memory, reused)
+    void* fv;                         // assignment: S*cells value words with a final bit (the queue's memory, reused)
     uint64_t queue_cap;
     uint32_t* claimed;                // one bit per edge
     uint64_t claimed_bits;            // edges
