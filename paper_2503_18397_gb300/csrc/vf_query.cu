@@ -128,52 +128,113 @@ static void launch_w(bool bytes, const void* keys, const uint64_t* offs, uint64_
 
 constexpr int kReqCache = 4096;
 
+// The cells' XOR of key i of request r and its answer.
+__device__ __forceinline__ void query_one(const QueryReq& r, uint64_t i) {
+    const Sig s = sig_u64(__ldcs(r.keys + i), r.g.kh, r.g.kl);
+    const uint64_t base = shard_of(s, r.g.h) * r.g.cells;
+    const uint64_t local = local_of(s, r.g.h);
+    uint64_t v[4];
+    edge_of(r.g, local, v);
+    if (r.g.b > 32) {  // values wider than 32 bits
+        uint64_t y = cell_get64(r.data, r.g.b, base + v[0]) ^ cell_get64(r.data, r.g.b, base + v[1]) ^
+                     cell_get64(r.data, r.g.b, base + v[2]);
+        if (r.g.k == 4) y ^= cell_get64(r.data, r.g.b, base + v[3]);
+        if (r.g.kind == 1) static_cast<uint8_t*>(r.out)[i] = uint8_t(y == fingerprint64(local, r.g.b));
+        else static_cast<uint64_t*>(r.out)[i] = y;
+        return;
+    }
+    uint32_t x = cell_get_nc(r.data, r.g.b, base + v[0]) ^ cell_get_nc(r.data, r.g.b, base + v[1]) ^
+                 cell_get_nc(r.data, r.g.b, base + v[2]);
+    if (r.g.k == 4) x ^= cell_get_nc(r.data, r.g.b, base + v[3]);
+    if (r.g.kind == 1) put_answer<true>(r.out, i, x, local, r.g.b);
+    else put_answer<false>(r.out, i, x, local, r.g.b);
+}
+
+// kQ keys of one request per thread, spaced a block apart, with all their
+// cell loads in flight before any is used (as k_query).
+template <int WIDTH, bool FILTER, int K>
+__device__ __forceinline__ void query_tile(const QueryReq& r, uint64_t i0, uint32_t m) {
+    const Geom g = r.g;
+    const uint64_t* const keys = r.keys + i0;
+    uint64_t loc[kQ], cell[kQ][K];
+#pragma unroll
+    for (int k = 0; k < kQ; k++) {
+        const uint32_t i = threadIdx.x + k * kQThreads;
+        const Sig s = i < m ? sig_u64(__ldcs(keys + i), g.kh, g.kl) : Sig{0, 0};
+        const uint64_t base = shard_of(s, g.h) * g.cells;
+        loc[k] = local_of(s, g.h);
+        uint64_t v[4];
+        edge_of(g, loc[k], v);
+#pragma unroll
+        for (int j = 0; j < K; j++) cell[k][j] = base + v[j];
+    }
+    uint32_t x[kQ];
+#pragma unroll
+    for (int k = 0; k < kQ; k++) {
+        uint32_t c[K];
+#pragma unroll
+        for (int j = 0; j < K; j++) c[j] = threadIdx.x + k * kQThreads < m ? cell_q<WIDTH>(r.data, g.b, cell[k][j]) : 0u;
+        x[k] = c[0] ^ c[1] ^ c[2];
+        if constexpr (K == 4) x[k] ^= c[3];
+    }
+#pragma unroll
+    for (int k = 0; k < kQ; k++) {
+        const uint32_t i = threadIdx.x + k * kQThreads;
+        if (i < m) put_answer<FILTER>(r.out, i0 + i, x[k], loc[k], g.b);
+    }
+}
+
 // Requests against many resident structures in one launch: request r owns
-// keys [key_off, key_off + m) of the launch's key space. Neighbouring keys of a
-// warp mostly share a request, so descriptor reads are broadcasts.
-__global__ void __launch_bounds__(kQThreads) k_query_batch(const QueryReq* __restrict__ reqs, uint32_t count,
+// keys [key_off, key_off + m) of the launch's key space. A block takes tiles of
+// consecutive keys; a tile almost always lies within one request, whose
+// descriptor is then looked up once for the block and whose keys go four a
+// thread (96 requests of 3*10^5 to 1.5*10^6 keys: 1.80 ms with a search and one key
+// a thread, 1.07 this way). A tile with a boundary in it is taken key by key.
+__global__ void __launch_bounds__(kQThreads, 4) k_query_batch(const QueryReq* __restrict__ reqs, uint32_t count,
                                                            uint64_t total) {
+    constexpr uint32_t kTileKeys = kQThreads * kQ;
     __shared__ uint64_t s_off[kReqCache];
     const bool cached = count <= kReqCache;
     if (cached)
         for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) s_off[i] = reqs[i].key_off;
     __syncthreads();
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    for (uint64_t g = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; g < total; g += stride) {
+    auto request_of = [&](uint64_t g) {
         uint32_t lo = 0, hi = count;
         while (hi - lo > 1) {
             const uint32_t mid = (lo + hi) >> 1;
             const uint64_t o = cached ? s_off[mid] : reqs[mid].key_off;
             if (o <= g) lo = mid; else hi = mid;
         }
-        const QueryReq& r = reqs[lo];
-        const uint64_t i = g - r.key_off;
-        const Sig s = sig_u64(__ldg(r.keys + i), r.g.kh, r.g.kl);
-        const uint64_t base = shard_of(s, r.g.h) * r.g.cells;
-        const uint64_t local = local_of(s, r.g.h);
-        uint64_t v[4];
-        edge_of(r.g, local, v);
-        if (r.g.b > 32) {  // values wider than 32 bits
-            uint64_t y = cell_get64(r.data, r.g.b, base + v[0]) ^ cell_get64(r.data, r.g.b, base + v[1]) ^
-                         cell_get64(r.data, r.g.b, base + v[2]);
-            if (r.g.k == 4) y ^= cell_get64(r.data, r.g.b, base + v[3]);
-            if (r.g.kind == 1) static_cast<uint8_t*>(r.out)[i] = uint8_t(y == fingerprint64(local, r.g.b));
-            else static_cast<uint64_t*>(r.out)[i] = y;
-            continue;
+        return lo;
+    };
+    for (uint64_t t0 = uint64_t(blockIdx.x) * kTileKeys; t0 < total; t0 += uint64_t(gridDim.x) * kTileKeys) {
+        const uint32_t m = total - t0 < kTileKeys ? uint32_t(total - t0) : kTileKeys;
+        const uint32_t first = request_of(t0);
+        const QueryReq& r = reqs[first];
+        const uint64_t i0 = t0 - r.key_off;
+        if (i0 + m <= r.m && r.g.k != 4 && (r.g.b == 8 || r.g.b == 16)) {
+            if (r.g.kind == 1) {
+                if (r.g.b == 8) query_tile<8, true, 3>(r, i0, m);
+                else query_tile<16, true, 3>(r, i0, m);
+            } else {
+                if (r.g.b == 8) query_tile<8, false, 3>(r, i0, m);
+                else query_tile<16, false, 3>(r, i0, m);
+            }
+        } else if (i0 + m <= r.m && r.g.k != 4 && r.g.b <= 32) {
+            if (r.g.kind == 1) query_tile<0, true, 3>(r, i0, m);
+            else query_tile<0, false, 3>(r, i0, m);
+        } else {
+            for (uint32_t i = threadIdx.x; i < m; i += kQThreads) {
+                const QueryReq& q = reqs[request_of(t0 + i)];
+                query_one(q, t0 + i - q.key_off);
+            }
         }
-        uint32_t x = cell_get_nc(r.data, r.g.b, base + v[0]) ^ cell_get_nc(r.data, r.g.b, base + v[1]) ^
-                     cell_get_nc(r.data, r.g.b, base + v[2]);
-        if (r.g.k == 4) x ^= cell_get_nc(r.data, r.g.b, base + v[3]);
-        if (r.g.kind == 1) static_cast<uint8_t*>(r.out)[i] = uint8_t(x == fingerprint(local, r.g.b));
-        else if (r.g.b <= 8) static_cast<uint8_t*>(r.out)[i] = uint8_t(x);
-        else if (r.g.b <= 16) static_cast<uint16_t*>(r.out)[i] = uint16_t(x);
-        else static_cast<uint32_t*>(r.out)[i] = x;
     }
 }
 
 cudaError_t launch_query_batch(const QueryReq* reqs, uint32_t count, uint64_t total, cudaStream_t st) {
     if (total == 0 || count == 0) return cudaSuccess;
-    uint64_t blocks = (total + kQThreads - 1) / kQThreads;
+    uint64_t blocks = (total + kQThreads * kQ - 1) / (kQThreads * kQ);
     const uint64_t cap = uint64_t(num_sms()) * 16;
     if (blocks > cap) blocks = cap;
     k_query_batch<<<unsigned(blocks < 1 ? 1 : blocks), kQThreads, 0, st>>>(reqs, count, total);
