@@ -149,7 +149,7 @@ def _ptr(x):
     if _is_tensor(x):
         if not x.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        return C.c_void_p(x.data_ptr())
+        return x.data_ptr()
     if isinstance(x, np.ndarray):
         if not x.flags["C_CONTIGUOUS"]:
             raise ValueError("array must be C-contiguous")
@@ -160,9 +160,20 @@ def _ptr(x):
 def _stream(stream, *bufs):
     if stream is not None:
         return C.c_void_p(stream if isinstance(stream, int) else stream.cuda_stream)
-    if torch is not None and any(_is_tensor(b) and b.is_cuda for b in bufs if b is not None):
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if torch is not None:
+        for b in bufs:
+            if isinstance(b, torch.Tensor) and b.is_cuda:
+                return _current_stream()
     return None
+
+
+def _current_stream():
+    """The current device's current stream (without the Stream object that
+    torch.cuda.current_stream() makes, where torch has the plain handle)."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(raw(torch.cuda.current_device()))
 
 
 def _len(keys, offsets):
@@ -182,6 +193,7 @@ class Structure:
 
     def __init__(self, handle):
         self._h = handle
+        self._out = None  # element type of this structure's answers, once asked for
 
     @property
     def handle(self):
@@ -278,19 +290,25 @@ def _out_dtype(info: VfInfo):
     return np.uint16 if info.b <= 16 else np.uint32 if info.b <= 32 else np.uint64
 
 
-def _torch_dtype(dt):
-    # 64-bit results come back as int64 tensors holding the bit patterns
-    return {np.uint8: torch.uint8, np.uint16: torch.uint16, np.uint32: torch.uint32, np.uint64: torch.int64}[dt]
+def _answers(s: Structure):
+    """_out_dtype of a structure, whose kind and width never change."""
+    if s._out is None:
+        s._out = _out_dtype(vf_get_info(s))
+    return s._out
+
+
+# 64-bit results come back as int64 tensors holding the bit patterns
+_TORCH_DTYPE = {} if torch is None else {np.uint8: torch.uint8, np.uint16: torch.uint16, np.uint32: torch.uint32,
+                                         np.uint64: torch.int64}
 
 
 def vf_query(s: Structure, keys, offsets=None, out=None, stream=None):
     """Query keys; returns `out` (allocated like `keys`: CUDA tensor or numpy)."""
     m = _len(keys, offsets)
     if out is None:
-        dt = _out_dtype(vf_get_info(s))
+        dt = _answers(s)
         if _is_tensor(keys):
-            tdt = _torch_dtype(dt)
-            out = torch.empty(m, dtype=tdt, device=keys.device)
+            out = torch.empty(m, dtype=_TORCH_DTYPE[dt], device=keys.device)
         else:
             out = np.empty(m, dtype=dt)
     _check(lib().vf_query(s.handle, _ptr(keys), _ptr(offsets), m, _ptr(out), _stream(stream, keys, out)))
@@ -304,9 +322,7 @@ def vf_query_batch(requests, stream=None):
     outs = []
     for i, (s, keys, out) in enumerate(requests):
         if out is None:
-            dt = _out_dtype(vf_get_info(s))
-            tdt = _torch_dtype(dt)
-            out = torch.empty(len(keys), dtype=tdt, device=keys.device)
+            out = torch.empty(len(keys), dtype=_TORCH_DTYPE[_answers(s)], device=keys.device)
         outs.append(out)
         arr[i].s = s.handle
         arr[i].keys = _ptr(keys)

@@ -277,24 +277,27 @@ struct Staged {
     const void* keys = nullptr;
     const uint64_t* offs = nullptr;
     const void* values = nullptr;
-    uint64_t key_bytes = 0;
     DevBuf kbuf, obuf, vbuf;
 };
 
 vf_status stage_keys(int key_kind, const void* keys, const uint64_t* offsets, uint64_t n, cudaStream_t st,
                      Staged& s) {
     if (key_kind == VF_KEYS_U64) {
-        s.key_bytes = n * 8;
         if (on_device(keys) || n == 0) {
             s.keys = keys;
         } else {
-            VF_CK(s.kbuf.alloc(s.key_bytes, st));
-            VF_CK(cudaMemcpyAsync(s.kbuf.p, keys, s.key_bytes, cudaMemcpyHostToDevice, st));
+            VF_CK(s.kbuf.alloc(n * 8, st));
+            VF_CK(cudaMemcpyAsync(s.kbuf.p, keys, n * 8, cudaMemcpyHostToDevice, st));
             s.keys = s.kbuf.p;
         }
         return VF_OK;
     }
-    const bool offs_dev = on_device(offsets);
+    const bool offs_dev = on_device(offsets), keys_dev = on_device(keys);
+    if (offs_dev && keys_dev) {  // nothing to copy: the kernels read the total from the offsets
+        s.offs = offsets;
+        s.keys = keys;
+        return VF_OK;
+    }
     uint64_t total = 0;
     if (offs_dev) {
         VF_CK(cudaMemcpyAsync(&total, offsets + n, 8, cudaMemcpyDeviceToHost, st));
@@ -306,8 +309,7 @@ vf_status stage_keys(int key_kind, const void* keys, const uint64_t* offsets, ui
         VF_CK(cudaMemcpyAsync(s.obuf.p, offsets, (n + 1) * 8, cudaMemcpyHostToDevice, st));
         s.offs = s.obuf.as<uint64_t>();
     }
-    s.key_bytes = total;
-    if (on_device(keys) || total == 0) {
+    if (keys_dev || total == 0) {
         s.keys = keys;
         if (total == 0) {
             VF_CK(s.kbuf.alloc(16, st));
@@ -1707,18 +1709,24 @@ vf_status vf_query(const vf_struct* s, const void* keys, const uint64_t* offsets
     if (m == 0) return VF_OK;
     if (!keys || !out) return fail(VF_EINVAL, "vf_query: NULL keys or out");
     const int key_kind = offsets ? VF_KEYS_BYTES : VF_KEYS_U64;
-    for (const auto& pw : {std::make_pair(keys, "keys"), std::make_pair(static_cast<const void*>(offsets), "offsets"),
-                           std::make_pair(static_cast<const void*>(out), "out")}) {
-        const vf_status cs = vf::check_here(pw.first, pw.second);
+    // (each look at a pointer is a driver call, and a small query is nothing else)
+    const vf::MemWhere kw = vf::mem_where(keys), ow = vf::mem_where(out);
+    if (kw == vf::MemWhere::kElsewhere) return vf::check_here(keys, "keys");
+    if (offsets) {
+        const vf_status cs = vf::check_here(offsets, "offsets");
         if (cs != VF_OK) return cs;
     }
+    if (ow == vf::MemWhere::kElsewhere) return vf::check_here(out, "out");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t ob = s->info.kind == VF_FILTER ? 1 : value_bytes(s->info.b);
-    const bool out_dev = on_device(out);
+    const bool out_dev = ow == vf::MemWhere::kHere;
     if (key_kind == VF_KEYS_U64) {
-        const bool keys_dev = on_device(keys);
+        const bool keys_dev = kw == vf::MemWhere::kHere;
         if (!keys_dev || !out_dev)
             return query_pipelined(s, static_cast<const uint64_t*>(keys), keys_dev, m, out, out_dev, ob, st);
+        PhaseTimer t(kPhQuery, st);
+        VF_CK(vf::launch_query(key_kind, keys, nullptr, m, s->geom, s->data, out, st));
+        return VF_OK;
     }
     Staged in_keys;
     vf_status rs = stage_keys(key_kind, keys, offsets, m, st, in_keys);
