@@ -3,6 +3,9 @@
 //   k_scatter_*   bucket (local signature, value) by shard (radix scatter)
 //   k_accumulate  fuse regime: degree and XOR-of-edge incidence per vertex (Sec. 4.3)
 //   k_sigs_*      signatures only (inspection entry point)
+#include <algorithm>
+#include <atomic>
+
 #include "vf_internal.h"
 
 namespace vf {
@@ -149,6 +152,89 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const uint64_t* __restrict
     }
 }
 
+// The same for 32 to 256 shards, where a warp's stores to its keys' shards would
+// touch as many sectors as it has lanes: a tile of 4096 keys is put in shard
+// order in shared memory first, and consecutive lanes then store consecutive
+// keys of a shard (10^9 keys, 64 shards: SCAT_A -> SCAT_B ms).
+constexpr int kStageItems = 16;
+constexpr uint32_t kStageShards = 256;
+constexpr uint32_t kStageTile = kThreads * kStageItems;
+
+template <bool SIG, bool VAL>
+__global__ void __launch_bounds__(kThreads) k_scatter_staged(const uint64_t* __restrict__ keys, const Sig* __restrict__ sig_in,
+                                                             const void* __restrict__ values, uint64_t n, Geom g,
+                                                             unsigned long long* __restrict__ cursor,
+                                                             uint64_t* __restrict__ loc_out,
+                                                             uint32_t* __restrict__ val_out, uint32_t s_lo, uint32_t s_hi) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t* s_x = reinterpret_cast<uint64_t*>(smem);                              // kStageTile
+    uint32_t* s_v = reinterpret_cast<uint32_t*>(s_x + kStageTile);                  // kStageTile (VAL)
+    uint8_t* s_sh = reinterpret_cast<uint8_t*>(s_v + (VAL ? kStageTile : 0));       // kStageTile
+    __shared__ uint32_t s_cnt[kStageShards], s_warp[kThreads / 32];
+    __shared__ unsigned long long s_base[kStageShards];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t S = 1u << g.h;
+    for (uint64_t t0 = uint64_t(blockIdx.x) * kStageTile; t0 < n; t0 += uint64_t(gridDim.x) * kStageTile) {
+        const uint32_t m = n - t0 < uint64_t(kStageTile) ? uint32_t(n - t0) : kStageTile;
+        s_cnt[tid] = 0;  // kThreads == kStageShards
+        uint64_t loc[kStageItems];
+        uint32_t rk[kStageItems];  // the shard, then its rank in the tile above it
+#pragma unroll
+        for (int j = 0; j < kStageItems; j++) {
+            const uint32_t i = tid + uint32_t(j) * kThreads;
+            Sig s{0, 0};
+            if (i < m) {
+                if constexpr (SIG) s = sig_in[t0 + i];
+                else s = sig_u64(__ldg(keys + t0 + i), g.kh, g.kl);
+            }
+            loc[j] = local_of(s, g.h);
+            rk[j] = uint32_t(shard_of(s, g.h));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kStageItems; j++) {
+            const uint32_t i = tid + uint32_t(j) * kThreads, s = rk[j];
+            if (i < m && s >= s_lo && s < s_hi) rk[j] |= atomicAdd(&s_cnt[s], 1u) << 8;  // only the shard group being built
+            else rk[j] = 0xFFFFFFFFu;
+        }
+        __syncthreads();
+        const uint32_t c = tid < S ? s_cnt[tid] : 0u;
+        uint32_t incl = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if (lane >= uint32_t(d)) incl += y;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        uint32_t first = incl - c, all = 0;
+        for (uint32_t w = 0; w < kThreads / 32; w++) {
+            if (w < warp) first += s_warp[w];
+            all += s_warp[w];
+        }
+        if (tid < S) {
+            s_cnt[tid] = first;
+            if (c) s_base[tid] = atomicAdd(&cursor[tid], (unsigned long long)c) - first;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kStageItems; j++) {
+            if (rk[j] == 0xFFFFFFFFu) continue;
+            const uint32_t s = rk[j] & 255u, at = s_cnt[s] + (rk[j] >> 8);
+            s_x[at] = loc[j];
+            s_sh[at] = uint8_t(s);
+            if (VAL) s_v[at] = load_value(values, g.b, t0 + tid + uint32_t(j) * kThreads);
+        }
+        __syncthreads();
+        for (uint32_t at = tid; at < all; at += kThreads) {
+            const unsigned long long pos = s_base[s_sh[at]] + at;
+            loc_out[pos] = s_x[at];
+            if (VAL) val_out[pos] = s_v[at];
+        }
+        __syncthreads();
+    }
+}
+
 // Many shards (h > 12): one global atomic per key.
 __global__ void __launch_bounds__(kThreads) k_scatter_wide(const uint64_t* __restrict__ keys,
                                                            const Sig* __restrict__ sig_in,
@@ -261,7 +347,28 @@ cudaError_t launch_scatter(const uint64_t* keys_u64, const Sig* sig_in, const vo
                            const Geom& g, unsigned long long* cursor, uint64_t* loc_out, uint32_t* val_out,
                            uint32_t s_lo, uint32_t s_hi, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    if ((1u << g.h) <= uint32_t(kSmemBinsMax))
+    if (g.h >= 5 && (1u << g.h) <= kStageShards) {
+        const size_t smem = size_t(kStageTile) * (values ? 13 : 9);
+        static std::atomic<uint64_t> attr_done{0};
+        int dev = 0;
+        cudaGetDevice(&dev);
+        const uint64_t bit = uint64_t(1) << (dev & 63);
+        if (!(attr_done.load() & bit)) {
+            const int most = int(size_t(kStageTile) * 13);
+            for (const void* f : {reinterpret_cast<const void*>(k_scatter_staged<true, true>),
+                                  reinterpret_cast<const void*>(k_scatter_staged<true, false>),
+                                  reinterpret_cast<const void*>(k_scatter_staged<false, true>),
+                                  reinterpret_cast<const void*>(k_scatter_staged<false, false>)}) {
+                const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+                if (e != cudaSuccess) return e;
+            }
+            attr_done.fetch_or(bit);
+        }
+        const unsigned grid = unsigned(std::min<uint64_t>((n + kStageTile - 1) / kStageTile, uint64_t(num_sms()) * 4));
+        auto go = [&](auto* k) { k<<<grid, kThreads, smem, st>>>(keys_u64, sig_in, values, n, g, cursor, loc_out, val_out, s_lo, s_hi); };
+        if (sig_in) values ? go(k_scatter_staged<true, true>) : go(k_scatter_staged<true, false>);
+        else values ? go(k_scatter_staged<false, true>) : go(k_scatter_staged<false, false>);
+    } else if ((1u << g.h) <= uint32_t(kSmemBinsMax))
         if (sig_in)
             k_scatter<true><<<stream_grid(n, kItems), kThreads, 0, st>>>(keys_u64, sig_in, values, n, g, cursor,
                                                                          loc_out, val_out, s_lo, s_hi);
