@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const uint64_t* __restrict
 // touch as many sectors as it has lanes: a tile of 4096 keys is put in shard
 // order in shared memory first, and consecutive lanes then store consecutive
 // keys of a shard (10^9 keys, 64 shards: SCAT_A -> SCAT_B ms).
-constexpr int kStageItems = 16;
+constexpr int kStageItems = 8;
 constexpr uint32_t kStageShards = 256;
 constexpr uint32_t kStageTile = kThreads * kStageItems;
 
@@ -174,6 +174,17 @@ __global__ void __launch_bounds__(kThreads) k_scatter_staged(const uint64_t* __r
     __shared__ unsigned long long s_base[kStageShards];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t S = 1u << g.h;
+    uint64_t nk[SIG ? 1 : kStageItems];
+    auto ahead = [&](uint64_t t) {
+        if constexpr (!SIG) {
+#pragma unroll
+            for (int j = 0; j < kStageItems; j++) {
+                const uint64_t i = t + tid + uint32_t(j) * kThreads;
+                nk[j] = i < n ? __ldg(keys + i) : 0ull;
+            }
+        }
+    };
+    ahead(uint64_t(blockIdx.x) * kStageTile);
     for (uint64_t t0 = uint64_t(blockIdx.x) * kStageTile; t0 < n; t0 += uint64_t(gridDim.x) * kStageTile) {
         const uint32_t m = n - t0 < uint64_t(kStageTile) ? uint32_t(n - t0) : kStageTile;
         s_cnt[tid] = 0;  // kThreads == kStageShards
@@ -185,11 +196,12 @@ __global__ void __launch_bounds__(kThreads) k_scatter_staged(const uint64_t* __r
             Sig s{0, 0};
             if (i < m) {
                 if constexpr (SIG) s = sig_in[t0 + i];
-                else s = sig_u64(__ldg(keys + t0 + i), g.kh, g.kl);
+                else s = sig_u64(nk[j], g.kh, g.kl);
             }
             loc[j] = local_of(s, g.h);
             rk[j] = uint32_t(shard_of(s, g.h));
         }
+        ahead(t0 + uint64_t(gridDim.x) * kStageTile);
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < kStageItems; j++) {

@@ -163,6 +163,8 @@ __global__ void __launch_bounds__(kIncSegThreads) k_incidence_seg(const uint64_t
                                                                   uint32_t* __restrict__ W, uint32_t* err,
                                                                   const uint32_t* __restrict__ drop) {
     extern __shared__ uint32_t sw[];
+    __shared__ uint32_t s_lost;
+    if (threadIdx.x == 0) s_lost = 0;
     const uint32_t lgc = g.lg_seg < kIncSegLgChunk ? g.lg_seg : kIncSegLgChunk;
     const uint32_t chunk = 1u << lgc, nch = 1u << (g.lg_seg - lgc);
     const uint32_t K = g.k == 4 ? 4u : 3u;
@@ -176,6 +178,7 @@ __global__ void __launch_bounds__(kIncSegThreads) k_incidence_seg(const uint64_t
         for (uint32_t i = threadIdx.x; i < chunk; i += blockDim.x) sw[i] = 0;
         __syncthreads();
         bool wrap = false;
+        uint32_t put = 0;  // contributions of this thread to the chunk
 #pragma unroll 1
         for (uint32_t k = 0; k < K; k++) {  // vertex k of the edges of bin t - k
             if (t < k || t - k >= nb) continue;
@@ -211,7 +214,8 @@ __global__ void __launch_bounds__(kIncSegThreads) k_incidence_seg(const uint64_t
                         wrap |= (atomicAdd(sw + r, 1u) & 31u) == 31u;
                         atomicXor(sw + r, el << 5);
                     } else {
-                        wrap |= (atomicAdd(sw + r, 1u + (el << 5)) & 31u) == 31u;
+                        atomicAdd(sw + r, 1u + (el << 5));
+                        put++;
                     }
                 }
             }
@@ -219,8 +223,23 @@ __global__ void __launch_bounds__(kIncSegThreads) k_incidence_seg(const uint64_t
         if (wrap) atomicOr(err, kErrDegOverflow);
         __syncthreads();
         uint32_t* out = W + uint64_t(sh) * g.cells + (uint64_t(t) << g.lg_seg) + (uint64_t(ch) << lgc);
-        for (uint32_t i = threadIdx.x; i < chunk; i += blockDim.x) out[i] = sw[i];
+        uint32_t got = 0;
+        for (uint32_t i = threadIdx.x; i < chunk; i += blockDim.x) {
+            const uint32_t w = sw[i];
+            out[i] = w;
+            got += w & 31u;
+        }
+        if (!XOR) {
+            // a degree that went past 31 has lost 32 of the contributions (no
+            // fetch-and-add has to return its word for that to be seen)
+            const uint32_t lost = __reduce_add_sync(0xFFFFFFFFu, put - got);
+            if ((threadIdx.x & 31u) == 0 && lost) atomicAdd(&s_lost, lost);
+        }
         __syncthreads();
+        if (!XOR && threadIdx.x == 0 && s_lost) {
+            atomicOr(err, kErrDegOverflow);
+            s_lost = 0;
+        }
     }
 }
 

@@ -28,8 +28,8 @@
 // peeling order, as the assignment needs it.
 //
 // The CTA whose fetch-and-add frees a vertex keeps it, so sizes drift apart
-// as the waves branch and die out; when one CTA holds more than twice the mean
-// (every CTA sees the same sizes), the round's pushes are dealt out over the
+// as the waves branch and die out; when one CTA holds well more than the mean
+// (front_uneven; every CTA sees the same sizes), the round's pushes are dealt out over the
 // cluster through distributed shared memory, behind a full cluster barrier.
 //
 // Measured (one GB300, b = 8; peel per attempt, worklist -> this): 2^20 keys 4.37 ->
@@ -54,7 +54,7 @@ constexpr uint32_t kFrMaxC = 16;        // CTAs per cluster
 constexpr uint32_t kFrPolls = 1u << 26; // tests of an exchange's wait (some 20 ns each): then it gives up
 constexpr uint32_t kFrHole = 0xFFFFFFFFu;
 constexpr int kFrHeadT = 1024;          // threads of a head round's block (one block per list)
-constexpr uint32_t kFrHeadPer = 2;      // entries a thread has in flight there
+constexpr uint32_t kFrHeadPer = 4;      // entries a thread has in flight there (2: +0.15 ms at 10^8 keys)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
 
@@ -238,21 +238,33 @@ __global__ void __launch_bounds__(kFrHeadT) k_front_head(FrontArgs a, uint32_t r
         for (uint32_t j = 0; j < kFrHeadPer; j++) {
             const uint32_t i = i0 + j * kFrHeadT + lane;
             if (i < n) front_record<K, VAL>(x[j], a, base, cells, at + i);
+        }
+        // one reservation per warp for all the pass frees
+        unsigned m[kFrHeadPer][K - 1];
+        uint32_t all = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++)
 #pragma unroll
             for (int k = 0; k < K - 1; k++) {
-                const uint32_t nw = w[j][k] - (1u + (x[j].e << 5));
-                const bool free_v = x[j].on && (nw & 31u) == 1u;
-                const unsigned m = __ballot_sync(0xFFFFFFFFu, free_v);
-                if (!m) continue;
-                uint32_t to = 0;
-                if (lane == 0) to = atomicAdd(&s_cnt, uint32_t(__popc(m)));
-                to = __shfl_sync(0xFFFFFFFFu, to, 0) + __popc(m & below);
-                if (free_v) {
-                    if (to < a.list_cap) out[to] = make_uint2(x[j].o[k], nw >> 5);
+                w[j][k] -= 1u + (x[j].e << 5);
+                m[j][k] = __ballot_sync(0xFFFFFFFFu, x[j].on && (w[j][k] & 31u) == 1u);
+                all += __popc(m[j][k]);
+            }
+        if (!all) continue;
+        uint32_t to = 0;
+        if (lane == 0) to = atomicAdd(&s_cnt, all);
+        to = __shfl_sync(0xFFFFFFFFu, to, 0);
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++)
+#pragma unroll
+            for (int k = 0; k < K - 1; k++) {
+                if ((m[j][k] >> lane) & 1u) {
+                    const uint32_t q = to + __popc(m[j][k] & below);
+                    if (q < a.list_cap) out[q] = make_uint2(x[j].o[k], w[j][k] >> 5);
                     else atomicOr(a.err, kErrFrontier);
                 }
+                to += __popc(m[j][k]);
             }
-        }
     }
     __syncthreads();
     if (tid == 0) a.list_n[uint64_t(r + 1) * lists + list] = min(s_cnt, a.list_cap);
@@ -275,6 +287,14 @@ __device__ __noinline__ void front_deal(const FrontArgs& a, uint32_t cnt, uint32
     } else {
         atomicOr(a.err, kErrFrontier);
     }
+}
+
+// Whether a round whose largest CTA holds `most` of `total` entries deals out what
+// it frees: beyond 1.25 times the mean and 48 more (4-uniform 10^8, ~150 entries a
+// CTA: 16.9 ms at twice the mean + 64, 12.2 at 1.25 times + 16; 3-uniform, ~64 a
+// CTA: 26.1 and 27.1, so the constant keeps small rounds from dealing often).
+__device__ __forceinline__ bool front_uneven(uint32_t most, uint32_t total, uint32_t lg_cta) {
+    return 4u * most > 5u * (total >> lg_cta) + 4u * 48u;
 }
 
 struct FrontShared {
@@ -408,7 +428,7 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                         const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
                         const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz);
                         at = before + __reduce_add_sync(0xFFFFFFFFu, lane < rank ? sz : 0u);
-                        deal = __reduce_max_sync(0xFFFFFFFFu, sz) > 2u * (total >> a.lg_cta) + 64u;
+                        deal = front_uneven(__reduce_max_sync(0xFFFFFFFFu, sz), total, a.lg_cta);
                     }
                     if (i < n) front_record<K, VAL>(x, a, base, cells, at + i);
                     // the vertices left at degree one join the next list
@@ -465,7 +485,7 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 if (tid == 0) atomicOr(a.err, kErrFrontier);
                 break;
             }
-            if (sh.most[p] > 2u * (total >> a.lg_cta) + 64u) cluster_barrier();  // this round's pushes were dealt out
+            if (front_uneven(sh.most[p], total, a.lg_cta)) cluster_barrier();  // this round's pushes were dealt out
             const uint32_t t = c0;
             c0 = c1, c1 = c2, c2 = t;
         }
