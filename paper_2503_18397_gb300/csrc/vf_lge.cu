@@ -1,7 +1,7 @@
 // LGE-regime solver of libvfunc (sm_103a): one CTA per shard, shards taken
 // from a global counter so uneven shards balance across SMs.
 //
-// Per shard, all synchronisation is __syncthreads (no spin-waits):
+// Per shard, all synchronisation is block barriers (no spin-waits):
 //  1. incidence: degree (8-bit lanes) and XOR of shard-local edge indices
 //     (16-bit lanes) per vertex, in shared memory (Sec. 4.3, XOR trick);
 //  2. peeling in synchronous rounds; each round first reads every frontier
@@ -13,25 +13,32 @@
 //     heaviest idle variables are made active (a batch of ~2.5% of the open
 //     equations at a time); equations left with no idle variable form the
 //     dense system over the active variables;
-//  4. every solved variable is an affine function of the active ones; the
-//     bit-packed coefficient rows (32 active variables per word) are built
-//     round by round (from one record per solve gathered after step 3), the
-//     dense rows are reduced by Gauss-Jordan elimination in shared memory, or
-//     in the CTA's slab when they do not fit (free variables = 0), solved
-//     variables are evaluated forward, and peeled edges are assigned in
-//     reverse peel order.
+//  4. the dense equations are carried back through the solves, 32 at a time
+//     with one word per variable in shared memory, until only active variables
+//     are left in them; the dense rows are reduced a word of columns at a time
+//     (free variables = 0); the solved variables are then evaluated forward
+//     and the peeled edges' vertices in reverse peel order, all in shared
+//     memory, and the cells stored once.
 //
-// Three configurations of the kernel share this code. Each round of steps 2-3
-// ends in a CTA barrier, so one CTA per SM leaves the SM idle at every
-// barrier; several CTAs per SM overlap several shards instead. Shards of at
-// most kLgeSmallTaskKeys keys run in the small configuration (192 threads,
-// 72 KB of shared memory, three CTAs per SM), larger ones in the medium one
-// (256 threads, 108 KB, two per SM). A shard whose peel arrays do not fit is
-// handed, unchanged, to the spill list, which the large configuration (512
-// threads, 200 KB, one CTA per SM) then solves from the start: all solve the
-// same system, so which one ran changes neither the outcome nor the retry count. A shard beyond the solver's pool
-// (active variables, coefficient rows) fails with kErrLgeSize, a capacity
-// error that ends the build rather than a retry.
+// What bounds it: the latency of a shard's dependent steps (a 9.8K-key shard has
+// ~25 peel rounds, ~112 elimination rounds, ~100 rounds of solves to walk back and
+// forth, ~11 panels), not bandwidth; several CTAs per SM overlap several shards,
+// and issue slots are 38% taken at 8192-key shards. So every step is made of
+// few barriers, on-chip words and loads sent ahead. Measured (one GB300): one
+// 10^4-key build 1836 -> 593 us; 10^7 strings in 1024 shards 9.86 -> 3.8 ms for
+// the whole build; 512 batched structures 49.9 -> 28.1 ms with this kernel alone.
+//
+// Three configurations of the kernel share this code. Shards of at most
+// kLgeSmallTaskKeys keys run in the small configuration (192 threads, 72 KB of
+// shared memory, three CTAs per SM), larger ones in the medium one (256
+// threads, 108 KB, two per SM). A shard whose arrays do not fit is handed,
+// unchanged, to the spill list, which the large configuration (512 threads, 200
+// KB, one CTA per SM) then solves from the start: all solve the same system, so
+// which one ran changes neither the outcome nor the retry count. A launch of no
+// more shards than SMs uses the large configuration alone: with an SM to itself
+// a shard is done sooner by 512 threads. A shard beyond the solver's pool (active
+// variables, dense rows) fails with kErrLgeSize, a capacity error that ends the
+// build rather than a retry.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -137,7 +144,7 @@ __device__ __forceinline__ void discard_words(const uint32_t* p, uint64_t words)
 // this, the 304 slabs resident at once (more than L2 holds) are written back
 // to DRAM line by line as they are evicted; discarding them instead keeps L2
 // for live lines. `m`, `V`: the finished shard's keys and cells; `lused`:
-// words of coefficient rows (and slab-resident dense system) it wrote.
+// words of the dense system's pool it wrote.
 __device__ void discard_slab(const uint32_t* scr, const LgeOffsets& o, uint32_t m, uint32_t V, uint64_t lused) {
     const uint64_t mm = m, vv = V;
     discard_words(scr + o.ev, 2 * mm);
@@ -966,8 +973,11 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
                         const uint32_t own = pivf[d];
                         uint32_t x = pan[d], y = 0;
                         if (own >= 2) {
-                            y = s_piv[own - 2].z ^ (1u << (own - 2));
-                            x = 0;  // its columns are done
+                            const uint4 p = s_piv[own - 2];
+                            y = p.z ^ (1u << (own - 2));
+                            // bits left stand in columns that the 64 rows had no pivot
+                            // for; a row of the next pass may, and this one takes it up
+                            x = p.y & ~(1u << p.w);
                             pivf[d] = 1;
                         } else if (k == 32) {
 #pragma unroll
