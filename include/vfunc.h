@@ -53,9 +53,10 @@ enum { VF_MODE_AUTO = 0, VF_MODE_FUSE = 1, VF_MODE_LGE = 2, VF_MODE_MWHC = 3 };
 enum { VF_REGIME_FUSE = 1, VF_REGIME_LGE = 2, VF_REGIME_MWHC = 3 };
 /* Fuse-regime solver. All peel the same hypergraph (Sec. 4.3) and give the
  * same query results; they differ in how the work is scheduled on the GPU.
- * VF_SOLVER_FLOW (default): asynchronous worklist peeling that records
- * peeled edges in an order whose reverse is a valid assignment order, then a
- * dataflow assignment. VF_SOLVER_ROUNDS: peeling in synchronous rounds with
+ * VF_SOLVER_FLOW (default): fuse graphs are peeled by a cluster of CTAs per
+ * shard in synchronous rounds, MWHC graphs (and shards whose rounds outgrow the
+ * clusters' lists) by an asynchronous worklist; both record peeled edges in an
+ * order whose reverse is a valid assignment order, then a dataflow assignment. VF_SOLVER_ROUNDS: peeling in synchronous rounds with
  * a grid barrier, assignment in reverse rounds. VF_SOLVER_WAVE: vertex words
  * that sum the degree, the other two vertices and the value of the incident
  * edges, so a peeling step is one fetch-and-add per vertex; grid-wide rounds

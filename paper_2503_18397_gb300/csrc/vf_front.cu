@@ -33,8 +33,8 @@
 // cluster through distributed shared memory, behind a full cluster barrier.
 //
 // Measured (one GB300, b = 8; peel per attempt, worklist -> this): 2^20 keys 4.37 ->
-// 3.55 ms, 10^8 (8 shards) 31.8 -> 26.0, 3*10^8 (16) 50.3 -> 30.9, 10^9 (64) 201 -> 88;
-// 4-uniform 10^8 15.2 -> 16.8, 3*10^8 56.9 -> 28.0. A round takes ~4300 cycles at 10^8:
+// 3.55 ms, 10^8 (8 shards) 31.8 -> 26.0, 3*10^8 (16) 50.3 -> 30.9, 10^9 (64) 201 -> 85;
+// 4-uniform 10^8 15.2 -> 13.3, 3*10^8 56.9 -> 28.0. A round takes ~4300 cycles at 10^8:
 // ~1100 to the claims and signatures, ~1400 to the removals, ~450 waiting for
 // the slowest CTA, the rest between them (a remote fetch-and-add also costs an
 // SM ~3.3 cycles a lane, L2 or distributed shared memory alike, and a CTA has

@@ -302,10 +302,10 @@ uint32_t lge_partition(std::vector<LgeTask>& tasks, uint64_t small_keys = kLgeSm
 // Layout (in 32-bit words) of one CTA's LGE scratch slab for shards of at most
 // m keys and V cells.
 constexpr uint32_t kMaxActive = 4096;  // active variables per shard (up to kLgeBigShard keys)
-constexpr uint32_t kLPoolPerKey = 40;  // words of coefficient rows per shard key (up to kLgeBigShard keys)
+constexpr uint32_t kLPoolPerKey = 40;  // words of the dense system's pool per shard key (up to kLgeBigShard keys)
 // Above kLgeBigShard keys (the regime's default largest shard) both grow with
-// the shard: ~6.6% of a shard's keys become active variables, and the affine
-// rows take ~0.0011 m words per key.
+// the shard: ~6.6% of a shard's keys become active variables, ~2.6% dense
+// equations, and the dense system grows with the product of the two.
 constexpr uint32_t kLgeBigShard = 24576;
 struct LgeOffsets {
     uint64_t ev, prec, proff, lists, core, eqst, inc_off, inc_list, vstate, act, actv, solves, soff, srec, dense, lc,
