@@ -35,11 +35,12 @@ __global__ void __launch_bounds__(kThreads) k_hist_u64(const uint64_t* __restric
 }
 
 // Byte-string keys: hash once, keep the signature for the scatter pass.
-__global__ void __launch_bounds__(kThreads) k_hist_bytes(const uint8_t* __restrict__ buf,
+__global__ void __launch_bounds__(kThreads, 5) k_hist_bytes(const uint8_t* __restrict__ buf,
                                                          const uint64_t* __restrict__ offs, uint64_t n, Geom g,
                                                          uint32_t* __restrict__ hist, Sig* __restrict__ sig_out) {
+    static_assert(kThreads == kTileStrings, "a string a thread");
     __shared__ uint32_t sh[kSmemBinsMax];
-    __shared__ uint4 stage[kStageBytes / 16];
+    __shared__ StringTile tile;
     const uint32_t S = 1u << g.h;
     const bool in_smem = S <= kSmemBinsMax;
     if (in_smem)
@@ -48,8 +49,8 @@ __global__ void __launch_bounds__(kThreads) k_hist_bytes(const uint8_t* __restri
     const uint64_t total = __ldg(offs + n);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < n; t0 += stride) {
-        const Sig s = sig_tile(buf, offs, total, t0, n, stage, g.kh, g.kl);
-        const uint64_t i = t0 + threadIdx.x;
+        uint64_t i;
+        const Sig s = sig_tile(buf, offs, total, t0, n, tile, g.kh, g.kl, i);
         if (i >= n) continue;
         sig_out[i] = s;
         uint32_t b = uint32_t(shard_of(s, g.h));
@@ -277,12 +278,13 @@ __global__ void k_sigs_u64(const uint64_t* __restrict__ keys, uint64_t n, uint64
 
 __global__ void k_sigs_bytes(const uint8_t* __restrict__ buf, const uint64_t* __restrict__ offs, uint64_t n,
                              uint64_t kh, uint64_t kl, Sig* __restrict__ out) {
-    __shared__ uint4 stage[kStageBytes / 16];
+    __shared__ StringTile tile;
     const uint64_t total = __ldg(offs + n);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < n; t0 += stride) {
-        const Sig s = sig_tile(buf, offs, total, t0, n, stage, kh, kl);
-        if (t0 + threadIdx.x < n) out[t0 + threadIdx.x] = s;
+        uint64_t i;
+        const Sig s = sig_tile(buf, offs, total, t0, n, tile, kh, kl, i);
+        if (i < n) out[i] = s;
     }
 }
 

@@ -70,17 +70,21 @@ __global__ void __launch_bounds__(kQThreads) k_query(const uint64_t* __restrict_
 
 // Byte strings: a block takes tiles of consecutive strings through shared
 // memory (sig_tile) and probes one key a thread; the resident blocks keep
-// enough probes in flight.
+// enough probes in flight. A tile alternates between loads and remixes, with
+// barriers between, so blocks on an SM count (six of 40 registers a thread, not
+// five of 48), and blocks of few tiles, which start as others end (3*10^6
+// strings: 101 -> 92 us with both; six resident blocks a SM that stay: 102).
 template <int WIDTH, bool FILTER, int K>
-__global__ void __launch_bounds__(kQThreads) k_query_bytes(const uint8_t* __restrict__ buf,
+__global__ void __launch_bounds__(kQThreads, 6) k_query_bytes(const uint8_t* __restrict__ buf,
                                                            const uint64_t* __restrict__ offs, uint64_t m, Geom g,
                                                            const uint8_t* __restrict__ data, void* __restrict__ out) {
-    __shared__ uint4 stage[kStageBytes / 16];
+    static_assert(kQThreads == kTileStrings, "a string a thread");
+    __shared__ StringTile tile;
     const uint64_t total = __ldg(offs + m);
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < m; t0 += stride) {
-        const Sig s = sig_tile(buf, offs, total, t0, m, stage, g.kh, g.kl);
-        const uint64_t i = t0 + threadIdx.x;
+        uint64_t i;
+        const Sig s = sig_tile(buf, offs, total, t0, m, tile, g.kh, g.kl, i);
         if (i >= m) continue;
         const uint64_t base = shard_of(s, g.h) * g.cells;
         const uint64_t local = local_of(s, g.h);
@@ -98,7 +102,7 @@ static void launch_q(bool bytes, const void* keys, const uint64_t* offs, uint64_
                      const uint8_t* data, void* out, cudaStream_t st) {
     const uint64_t per = uint64_t(kQThreads) * (bytes ? 1 : kQ);
     uint64_t blocks = (m + per - 1) / per;
-    uint64_t cap = uint64_t(num_sms()) * 16;
+    uint64_t cap = uint64_t(num_sms()) * (bytes ? 24 : 16);  // bytes: four times what is resident
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const uint64_t* k64 = static_cast<const uint64_t*>(keys);
