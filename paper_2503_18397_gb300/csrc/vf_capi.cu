@@ -465,7 +465,9 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
     std::vector<uint32_t> h(vf::kFlowWords);
     std::vector<uint32_t> hrc(rc_words);
     vf::FrontConfig fc;
-    DevBuf heads;
+    vf::FrontArgs f;
+    DevBuf heads, rounds;
+    bool by_round = false;  // the records are assigned round by round
     for (bool waves = vf::front_config(g, a.S, fc);; waves = false) {
         if (!own_incidence) VF_CK(cudaMemsetAsync(W.p, 0, V * 4, st));
         if (drop)  // dropped duplicates count as claimed: they are never peeled
@@ -482,7 +484,6 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
                 VF_CK(vf::launch_incidence32(loc, n, start, a.S, g, a.W, a.err, drop, st));
         }
         if (waves) {
-            vf::FrontArgs f;
             std::memset(&f, 0, sizeof f);
             f.loc = loc;
             f.val = val;
@@ -502,6 +503,12 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
             f.list_n = heads.as<uint32_t>();
             f.rcv = f.list_n + nl;
             VF_CK(cudaMemsetAsync(heads.p, 0, (nl + nr) * 4, st));
+            // (the waits that the fault hooks shorten are the dataflow's)
+            by_round = vf::front_assign_fits(g, a.S) && !a.stall && !a.assign_limit;
+            if (by_round) {
+                VF_CK(rounds.alloc(in.shards * vf::kFrontRounds * 4, st));
+                f.round = rounds.as<uint32_t>();
+            }
             f.epsg = a.epsg;
             f.ahead = 5;  // (none: +5% at 10^8 keys; 12: +3%)
             f.err = a.ctr + vf::kFrontErr;
@@ -521,6 +528,7 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         VF_CK(cudaStreamSynchronize(st));
         // a list beyond its room: the worklist takes the attempt alone, from the start
         if (waves && ((h[vf::kFlowErr] | h[vf::kFrontErr]) & (vf::kErrFrontier | vf::kErrCapacity))) continue;
+        by_round = by_round && waves;
         break;
     }
     const uint32_t count = h[vf::kFlowPeeled], err = h[vf::kFlowErr] | h[vf::kFrontErr];
@@ -528,6 +536,7 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
     for (uint64_t s = 0; s < in.shards; s++) {
         slots += hrc[s * vf::kRcStride];
         rmax = std::max<uint64_t>(rmax, hrc[s * vf::kRcStride]);
+        by_round = by_round && hrc[s * vf::kRcStride + 1] <= vf::kFrontRounds;
     }
     *peeled = count - ndrop;  // claim bits include the dropped duplicates
     if (err & vf::kErrTimeout) return fail(VF_ETIMEOUT, "asynchronous peeling wait timed out");
@@ -537,6 +546,14 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         return VF_EBUILD;
     }
     if (rmax > in.cells) return fail(VF_ECUDA, "asynchronous peeling took more record slots than items");
+    if (by_round) {  // no bounded waits: no error word to look at
+        {
+            PhaseTimer t(kPhAssign, st, int(vf::kFrontHead) + 1);
+            VF_CK(vf::launch_front_assign(f, fc, data, cell_base, st));
+        }
+        VF_CK(cudaStreamSynchronize(st));
+        return VF_OK;
+    }
     a.nrec = slots;
     a.rmax = rmax;
     {

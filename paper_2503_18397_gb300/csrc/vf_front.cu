@@ -308,7 +308,8 @@ struct FrontShared {
 };
 
 // K: vertices per edge (3, or 4 for a 4-uniform fuse graph). VAL: a function.
-template <int K, bool VAL>
+// ROUNDS: notes where each round's records start (0.5% of the peel at 10^8 keys).
+template <int K, bool VAL, bool ROUNDS>
 __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
     __shared__ FrontShared sh;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, below = (1u << lane) - 1u;
@@ -356,6 +357,7 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
         // segments whose words and signatures have been asked for: [0, pf_lo) and (pf_hi, T)
         int pf_lo = 0, pf_hi = int(cells >> lgs) - 1;
         uint32_t c0 = 0, c1 = 1, c2 = 2;  // r % 3, (r + 1) % 3, (r + 2) % 3
+        uint32_t rounds = 0;  // (the exchanger's)
         for (uint32_t cur = 0;; cur ^= 1u) {
             uint32_t n = sh.cnt[c0];
             n = min(n, max(a.list_cap, kFrList));
@@ -403,6 +405,11 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
                 const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz), most = __reduce_max_sync(0xFFFFFFFFu, sz);
                 if (lane == 0) sh.total[p] = total, sh.most[p] = most;
+                if (ROUNDS && rank == 0 && lane == 0) {  // where the round's records start, for the assignment
+                    if (total == 0) a.rc[s * kRcStride + 1] = rounds;
+                    else if (rounds < kFrontRounds) a.round[uint64_t(s) * kFrontRounds + rounds] = before;
+                    rounds++;
+                }
             } else {
                 uint32_t i = tid;
                 FrontItem<K> x;
@@ -493,19 +500,122 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
     }
 }
 
-// ------------------------------------------------------------------ launches
+// ------------------------------------------------------------ assignment
 
-static const void* front_kernel(const Geom& g) {
-    const bool val = g.kind == 0;
-    if (g.k == 4)
-        return val ? reinterpret_cast<const void*>(k_front_peel<4, true>) : reinterpret_cast<const void*>(k_front_peel<4, false>);
-    return val ? reinterpret_cast<const void*>(k_front_peel<3, true>) : reinterpret_cast<const void*>(k_front_peel<3, false>);
+// The records of one round depend on no other of the round: an edge's other
+// vertices are freed by its removal, so what is peeled from them comes in a later
+// round. So the rounds go back one by one, the waves' by the shard's cluster with a
+// cluster barrier behind each, the head's in a launch each; the cells themselves
+// hold the values.
+// A round of the waves is one trip to L2 for the two values, whose records were
+// loaded two rounds ahead, and one barrier; the worklist's dataflow polls a value
+// word written by another SM. Measured (b = 8, dataflow -> this): 10^9 keys 62 -> 27
+// ms, 4-uniform 8*10^8 38 -> 24. Asking L2 for the next round's cells a round ahead
+// was slower (27 -> 34): a CTA's requests, some 200 a round, already count.
+constexpr int kFrAssignT = 128;
+
+// The answer of a record: its value and the cells of the edge's other vertices.
+template <int K, class T>
+__device__ __forceinline__ void front_put(T* cells, uint4 q, uint32_t q3) {
+    if (q.x == kFrHole) return;
+    uint32_t x = q.w ^ __ldcg(cells + q.y) ^ __ldcg(cells + q.z);
+    if constexpr (K == 4) x ^= __ldcg(cells + q3);
+    cells[q.x] = T(x);
 }
 
-static cudaLaunchConfig_t front_launch(unsigned cta, unsigned clusters, cudaStream_t st, cudaLaunchAttribute* at) {
+template <int K, class T>
+__global__ void __launch_bounds__(kFrAssignT) k_front_assign(FrontArgs a, T* cells) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    uint32_t rank, C, s;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(s));
+    const uint32_t end = __ldg(a.rc + s * kRcStride), R = __ldg(a.rc + s * kRcStride + 1);
+    const uint32_t* const off = a.round + uint64_t(s) * kFrontRounds;
+    const uint4* const rec = a.rec + uint64_t(s) * a.g.cells;
+    const uint32_t* const rec3 = K == 4 ? a.rec3 + uint64_t(s) * a.g.cells : nullptr;
+    // bound(0), bound(1): the ends of the last round, and so on back
+    auto bound = [&](uint32_t k) { return k == 0 ? end : __ldg(off + R - min(k, R)); };
+    const uint32_t me = ((warp * C + rank) << 5) + lane, step = C * kFrAssignT;
+    auto load = [&](uint32_t i, uint32_t hi, uint4& q, uint32_t& q3) {
+        q.x = kFrHole;
+        if (i >= hi) return;
+        q = __ldcg(rec + i);
+        if constexpr (K == 4) q3 = __ldcg(rec3 + i);
+    };
+    if (R == 0) return;
+    uint32_t b0 = bound(0), b1 = bound(1), b2 = bound(2), b3 = bound(3);
+    uint4 q, q1, q2;
+    uint32_t t = 0, t1 = 0, t2 = 0;
+    load(b1 + me, b0, q, t);
+    load(b2 + me, b1, q1, t1);
+    for (uint32_t k = 0; k < R; k++) {
+        const uint32_t b4 = bound(k + 4);
+        load(b3 + me, b2, q2, t2);
+        front_put<K, T>(cells, q, t);
+        for (uint32_t i = b1 + me + step; i < b0; i += step) {
+            uint4 x;
+            uint32_t x3 = 0;
+            load(i, b0, x, x3);
+            front_put<K, T>(cells, x, x3);
+        }
+        cluster_barrier();
+        q = q1, q1 = q2, t = t1, t1 = t2;
+        b0 = b1, b1 = b2, b2 = b3, b3 = b4;
+    }
+}
+
+// Round r of the head, every shard's records over gridDim.x / S blocks.
+template <int K, class T>
+__global__ void __launch_bounds__(kFrWork) k_front_head_assign(FrontArgs a, T* cells, uint32_t r) {
+    const uint32_t per = gridDim.x / a.S, s = blockIdx.x / per;
+    const uint32_t lo = __ldg(a.rcv + uint64_t(r) * a.S + s), hi = __ldg(a.rcv + uint64_t(r + 1) * a.S + s);
+    const uint64_t base = uint64_t(s) * a.g.cells;
+    const uint32_t step = per * kFrWork;
+    for (uint64_t i = uint64_t(lo) + (blockIdx.x % per) * kFrWork + threadIdx.x; i < hi; i += kFrHeadPer * step) {
+        uint4 q[kFrHeadPer];
+        uint32_t q3[kFrHeadPer], x[kFrHeadPer];
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++) {
+            const uint64_t at = i + uint64_t(j) * step;
+            q[j] = make_uint4(kFrHole, 0, 0, 0);
+            q3[j] = 0;
+            if (at < hi) {
+                q[j] = __ldcs(a.rec + base + at);
+                if constexpr (K == 4) q3[j] = __ldcs(a.rec3 + base + at);
+            }
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++) {
+            x[j] = q[j].w;
+            if (q[j].x == kFrHole) continue;
+            x[j] ^= __ldcg(cells + q[j].y) ^ __ldcg(cells + q[j].z);
+            if constexpr (K == 4) x[j] ^= __ldcg(cells + q3[j]);
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < kFrHeadPer; j++)
+            if (q[j].x != kFrHole) cells[q[j].x] = T(x[j]);
+    }
+}
+
+// ------------------------------------------------------------------ launches
+
+template <int K, bool VAL>
+static const void* front_kernel(bool rounds) {
+    return rounds ? reinterpret_cast<const void*>(k_front_peel<K, VAL, true>)
+                  : reinterpret_cast<const void*>(k_front_peel<K, VAL, false>);
+}
+static const void* front_kernel(const Geom& g, bool rounds) {
+    const bool val = g.kind == 0;
+    if (g.k == 4) return val ? front_kernel<4, true>(rounds) : front_kernel<4, false>(rounds);
+    return val ? front_kernel<3, true>(rounds) : front_kernel<3, false>(rounds);
+}
+
+static cudaLaunchConfig_t front_launch(unsigned cta, unsigned clusters, cudaStream_t st, cudaLaunchAttribute* at,
+                                       unsigned threads = kFrT) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(cta * clusters);
-    lc.blockDim = dim3(kFrT);
+    lc.blockDim = dim3(threads);
     lc.stream = st;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cta;
@@ -520,15 +630,18 @@ static cudaLaunchConfig_t front_launch(unsigned cta, unsigned clusters, cudaStre
 bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg) {
     if (g.regime != kRegimeFuse || (g.k != 3 && g.k != 4) || g.lg_seg < 5 || g.lg_seg > 26) return false;
     static std::mutex mu;
-    static FrontConfig known[4][64];  // per kernel and device: cta = 0 unknown, ~0u not able
+    static FrontConfig known[8][64];  // per kernel and device: cta = 0 unknown, ~0u not able
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-    const void* fn = front_kernel(g);
+    const bool rounds = front_assign_fits(g, S);
+    const void* fn = front_kernel(g, rounds);
     std::lock_guard<std::mutex> lock(mu);
-    FrontConfig& k = known[(g.k == 4 ? 2 : 0) + (g.kind == 0 ? 1 : 0)][dev];
+    FrontConfig& k = known[(rounds ? 4 : 0) + (g.k == 4 ? 2 : 0) + (g.kind == 0 ? 1 : 0)][dev];
     if (k.cta == 0) {
         k.cta = ~0u;
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+        for (bool r : {false, true})  // (the fault hooks take the one without rounds)
+            if (cudaFuncSetAttribute(front_kernel(g, r), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+                cudaGetLastError();
         for (unsigned c : {kFrMaxC, 8u}) {
             cudaLaunchAttribute at[2]{};
             const cudaLaunchConfig_t lc = front_launch(c, 1, nullptr, at);
@@ -564,7 +677,47 @@ cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaSt
     cudaLaunchAttribute at[2]{};
     const cudaLaunchConfig_t lc = front_launch(cfg.cta, cfg.clusters, st, at);
     void* args[] = {const_cast<FrontArgs*>(&a)};
-    return cudaLaunchKernelExC(&lc, front_kernel(a.g), args);
+    return cudaLaunchKernelExC(&lc, front_kernel(a.g, a.round != nullptr), args);
+}
+
+// A round here costs more than a level of the dataflow (~1.6 against ~1.1 us: a
+// barrier behind every store), whatever it holds; the dataflow's polls cost more
+// the more records are under way at once. The line lies where the shards' segments
+// hold 2^20 cells together (4-uniform graphs, whose rounds are some four times as
+// wide: 2^18), ms, dataflow and rounds: 10^8 8.9, 12.7; 3*10^8 (2^20) 14.7, 14.8;
+// 4*10^8 (2^20) 21.1, 23.6; 6*10^8 (2^21) 30.1, 18.5; 10^9 (2^22) 62, 27; 4-uniform
+// 2*10^8 (2^18) 11.3, 11.8; 4*10^8 (2^19) 19.7, 14.6.
+constexpr uint64_t kRoundCells = 1u << 20;
+
+bool front_assign_fits(const Geom& g, uint32_t S) {
+    if ((g.b != 8 && g.b != 16 && g.b != 32) || S > kFrontRoundShards) return false;
+    return (uint64_t(S) << g.lg_seg) << (g.k == 4 ? 2 : 0) > kRoundCells;
+}
+
+template <int K, class T>
+static cudaError_t assign_rounds(const FrontArgs& a, const FrontConfig& cfg, T* cells, cudaStream_t st) {
+    const auto waves = k_front_assign<K, T>;
+    cudaError_t e = cudaFuncSetAttribute(waves, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    // a cluster per shard: none waits for another, so they need not all be resident
+    cudaLaunchAttribute at[2]{};
+    const cudaLaunchConfig_t lc = front_launch(cfg.cta, a.S, st, at, kFrAssignT);
+    e = cudaLaunchKernelEx(&lc, waves, a, cells);
+    if (e != cudaSuccess) return e;
+    const unsigned per = std::max(8u, (num_sms() * 8u + a.S - 1) / a.S);
+    for (uint32_t r = kFrontHead; r-- > 0;) k_front_head_assign<K, T><<<a.S * per, kFrWork, 0, st>>>(a, cells, r);
+    return cudaGetLastError();
+}
+
+template <class T>
+static cudaError_t assign_cells(const FrontArgs& a, const FrontConfig& cfg, T* cells, cudaStream_t st) {
+    return a.g.k == 4 ? assign_rounds<4>(a, cfg, cells, st) : assign_rounds<3>(a, cfg, cells, st);
+}
+
+cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig& cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st) {
+    if (a.g.b == 8) return assign_cells(a, cfg, data + cell_base, st);
+    if (a.g.b == 16) return assign_cells(a, cfg, reinterpret_cast<uint16_t*>(data) + cell_base, st);
+    return assign_cells(a, cfg, reinterpret_cast<uint32_t*>(data) + cell_base, st);
 }
 
 }  // namespace vf

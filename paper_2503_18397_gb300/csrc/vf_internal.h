@@ -198,6 +198,7 @@ struct FrontArgs {
     uint32_t list_cap;                //   each CTA of each shard's cluster
     uint32_t* list_n;                 // their numbers, by head round ((kFrontHead + 1) * S * CTAs)
     uint32_t* rcv;                    // record slots taken per shard, by head round ((kFrontHead + 1) * S; first row zero)
+    uint32_t* round;                  // record slots taken before each round of a shard's waves (kFrontRounds a shard)
     uint32_t epsg;                    // edges per start segment
     uint32_t ahead;                   // segments ahead of a wave's middle that are brought to L2
     uint32_t lg_cta;                  // lg of the cluster size
@@ -208,6 +209,14 @@ struct FrontArgs {
 // regimes, few shards, or a device without such clusters).
 bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg);
 cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaStream_t st);
+// Assignment of the attempt's records round by round, last to first, straight in the
+// (zeroed) data array: for cells of 8, 16 or 32 bits and many shards, where no shard's
+// waves took more than kFrontRounds rounds (their number: the second word of the
+// shard's line of rc).
+constexpr uint32_t kFrontRounds = 1u << 15;
+constexpr uint32_t kFrontRoundShards = 1024;  // at most 128 MB of round starts
+bool front_assign_fits(const Geom& g, uint32_t S);
+cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig& cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st);
 
 // Fuse-regime wave solver (csrc/vf_wave.cu): 64-bit vertex words that hold the
 // degree, the other two vertices and the value of the edges' sum; phase I in

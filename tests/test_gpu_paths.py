@@ -105,6 +105,39 @@ def test_cluster_peel(vf, orc, arity, n, eps):  # noqa: F811
                 n_other=10_000)
 
 
+@pytest.mark.parametrize("n,b,kw", [
+    (600_000_000, 8, dict(kind="filter")), (600_000_000, 16, dict(kind="func")),   # 32 shards, 2^16-cell segments
+    (400_000_000, 8, dict(kind="filter", arity=4)),                               # 32 shards, 2^14-cell segments
+    (40_000_000, 32, dict(kind="func", arity=4, eps=0.03)),                        # 1024 shards of few short rounds
+    (40_000_000, 13, dict(kind="func", arity=4, eps=0.03)),                        # a bit array: the dataflow's
+])
+def test_assignment_by_rounds_and_by_dataflow(vf, n, b, kw):  # noqa: F811
+    kw = dict(kw)
+    kind = vf.FILTER if kw.pop("kind") == "filter" else vf.FUNC
+    keys = synth.u64_keys_torch(0, n, 12)
+    vals = None
+    if kind == vf.FUNC:
+        vals = (keys & ((1 << b) - 1)).to(torch.uint16 if b <= 16 else torch.uint32)
+    p = vf.vf_params_default(kind=kind, b=b, mode=vf.MODE_FUSE, seed=3, **kw)
+    seeds = []
+    for limit in (0, 1 << 23):  # a limit on the dataflow's waits keeps the dataflow
+        vf.vf_debug_faults(assign_poll_limit=limit)
+        try:
+            s = vf.vf_build(keys, vals, params=p)
+        finally:
+            vf.vf_debug_faults()
+        out = s.query(keys)
+        if vals is None:
+            assert bool(out.all())
+        else:
+            signed = torch.int16 if b <= 16 else torch.int32
+            assert bool((out.view(signed) == vals.view(signed)).all())
+        seeds.append(s.info.seed)
+        s.free()
+        del out
+    assert seeds[0] == seeds[1]
+
+
 def test_a_key_given_forty_times(vf, orc):  # noqa: F811
     # its vertices' degrees wrap (more than 31 edges): the attempt fails unpeeled, for
     # functions and filters alike, and no index is read off a wrapped word
