@@ -95,7 +95,7 @@ ALGO_BYTES = {
 }
 
 # The same phases counted by what the kernels here move (the segment sort's
-# counting and scatter passes, the asynchronous peel's 16-byte records and queue items, the polled
+# counting and scatter passes, the peel's 16-byte records and list entries, the polled
 # value words of the dataflow assignment): a second figure, for comparison.
 def _seg_sort_bytes(kind):
     return 24.0 + (0 if kind == "filter" else 8.0)
@@ -490,9 +490,9 @@ def phase_table(phases, n, steps, b, kind, hbm, peak_kind, workload, fuse, k=3):
 # Per-launch DRAM traffic (bytes) from ncu captures of the same kernels, scaled
 # from the captured case by units processed; absent until a capture of the
 # current kernel exists (profiles/ holds the summaries).
-TRAFFIC = {("c2", "peel"): round(1120.07e6 / 2e7 * 1e8),   # k_flow_peel, one launch per attempt at 1e8
-           ("c2", "query"): round(189.42e6 / 2e7 * 1e8),  # k_query, one launch per 1e8 queries
-           ("c3", "lge"): round(788.86e6 + 806.24e6)}     # k_lge medium configuration, full-size capture
+TRAFFIC = {("c2", "peel"): round(1120.07e6 / 2e7 * 1e8),   # k_flow_peel, one launch per attempt at 1e8 (the clusters'
+                                                           # eight head rounds and waves: 92 B an edge, not 56)
+           ("c2", "query"): round(189.42e6 / 2e7 * 1e8)}  # k_query, one launch per 1e8 queries
 
 
 # ---------------------------------------------------------------- reference arm
