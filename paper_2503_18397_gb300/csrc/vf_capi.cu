@@ -463,11 +463,12 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
     a.assign_limit = g_debug_assign_limit.load();
     a.stall = g_debug_stall_assign.load() ? 1u : 0u;
     std::vector<uint32_t> h(vf::kFlowWords);
-    std::vector<uint32_t> hrc(rc_words);
+    std::vector<uint32_t> hrc(rc_words), hhead(in.shards);
     vf::FrontConfig fc;
     vf::FrontArgs f;
     DevBuf heads, rounds;
     bool by_round = false;  // the records are assigned round by round
+    bool by_head = false;   // those of the head rounds are, the others by the dataflow
     for (bool waves = vf::front_config(g, a.S, fc);; waves = false) {
         if (!own_incidence) VF_CK(cudaMemsetAsync(W.p, 0, V * 4, st));
         if (drop)  // dropped duplicates count as claimed: they are never peeled
@@ -504,7 +505,9 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
             f.rcv = f.list_n + nl;
             VF_CK(cudaMemsetAsync(heads.p, 0, (nl + nr) * 4, st));
             // (the waits that the fault hooks shorten are the dataflow's)
-            by_round = vf::front_assign_fits(g, a.S) && !a.stall && !a.assign_limit;
+            const bool native = (g.b == 8 || g.b == 16 || g.b == 32) && !a.stall && !a.assign_limit;
+            by_round = native && vf::front_assign_fits(g, a.S);
+            by_head = native && V >= vf::kFrontHeadCells;
             if (by_round) {
                 VF_CK(rounds.alloc(in.shards * vf::kFrontRounds * 4, st));
                 f.round = rounds.as<uint32_t>();
@@ -525,6 +528,9 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         }
         VF_CK(cudaMemcpyAsync(h.data(), a.ctr, vf::kFlowWords * 4, cudaMemcpyDeviceToHost, st));
         VF_CK(cudaMemcpyAsync(hrc.data(), rc.p, hrc.size() * 4, cudaMemcpyDeviceToHost, st));
+        by_head = by_head && waves;
+        if (by_head)
+            VF_CK(cudaMemcpyAsync(hhead.data(), f.rcv + vf::kFrontHead * in.shards, hhead.size() * 4, cudaMemcpyDeviceToHost, st));
         VF_CK(cudaStreamSynchronize(st));
         // a list beyond its room: the worklist takes the attempt alone, from the start
         if (waves && ((h[vf::kFlowErr] | h[vf::kFrontErr]) & (vf::kErrFrontier | vf::kErrCapacity))) continue;
@@ -532,10 +538,13 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         break;
     }
     const uint32_t count = h[vf::kFlowPeeled], err = h[vf::kFlowErr] | h[vf::kFrontErr];
+    if (!by_head) std::fill(hhead.begin(), hhead.end(), 0u);
     uint64_t slots = 0, rmax = 0;
+    bool overrun = false;
     for (uint64_t s = 0; s < in.shards; s++) {
         slots += hrc[s * vf::kRcStride];
-        rmax = std::max<uint64_t>(rmax, hrc[s * vf::kRcStride]);
+        overrun = overrun || hrc[s * vf::kRcStride] > in.cells || hhead[s] > hrc[s * vf::kRcStride];
+        rmax = std::max<uint64_t>(rmax, hrc[s * vf::kRcStride] - hhead[s]);  // (zero without a head of its own)
         by_round = by_round && hrc[s * vf::kRcStride + 1] <= vf::kFrontRounds;
     }
     *peeled = count - ndrop;  // claim bits include the dropped duplicates
@@ -545,20 +554,22 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         if (claimed_out) claimed_out->adopt(claimed);
         return VF_EBUILD;
     }
-    if (rmax > in.cells) return fail(VF_ECUDA, "asynchronous peeling took more record slots than items");
+    if (overrun) return fail(VF_ECUDA, "peeling took more record slots than items");
     if (by_round) {  // no bounded waits: no error word to look at
         {
             PhaseTimer t(kPhAssign, st, int(vf::kFrontHead) + 1);
-            VF_CK(vf::launch_front_assign(f, fc, data, cell_base, st));
+            VF_CK(vf::launch_front_assign(f, &fc, data, cell_base, st));
         }
         VF_CK(cudaStreamSynchronize(st));
         return VF_OK;
     }
     a.nrec = slots;
     a.rmax = rmax;
+    if (by_head) a.head_end = f.rcv + vf::kFrontHead * in.shards;
     {
-        PhaseTimer t(kPhAssign, st, slots ? 2 : 1);  // final flags, dataflow assignment
+        PhaseTimer t(kPhAssign, st, (slots ? 2 : 1) + (by_head ? int(vf::kFrontHead) : 0));  // final flags, dataflow, head rounds
         VF_CK(vf::launch_flow_assign(a, st));
+        if (by_head) VF_CK(vf::launch_front_assign(f, nullptr, data, cell_base, st));
     }
     uint32_t e2 = 0;
     VF_CK(cudaMemcpyAsync(&e2, a.err, 4, cudaMemcpyDeviceToHost, st));

@@ -643,8 +643,8 @@ __global__ void __launch_bounds__(kFT) k_flow_assign(FlowArgs a) {
             const uint64_t c = k >> 5;  // a warp's 32 positions: consecutive records of one shard
             const uint32_t s = uint32_t(c % a.S);
             const uint64_t j = ((c / a.S) << 5) + (k & 31u);
-            const uint32_t taken = __ldg(a.rc + s * kRcStride);
-            if (j < taken) {
+            const uint32_t taken = __ldg(a.rc + s * kRcStride), first = a.head_end ? __ldg(a.head_end + s) : 0u;
+            if (j < taken - first) {
                 const uint64_t rs = s * cells + (taken - 1 - j);
                 r = __ldg(a.rec + rs);
                 if (K == 4 && r.x != kHole) r3 = __ldg(a.rec3 + rs);  // third other vertex

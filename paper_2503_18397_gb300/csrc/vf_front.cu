@@ -686,12 +686,20 @@ cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaSt
 // hold 2^20 cells together (4-uniform graphs, whose rounds are some four times as
 // wide: 2^18), ms, dataflow and rounds: 10^8 8.9, 12.7; 3*10^8 (2^20) 14.7, 14.8;
 // 4*10^8 (2^20) 21.1, 23.6; 6*10^8 (2^21) 30.1, 18.5; 10^9 (2^22) 62, 27; 4-uniform
-// 2*10^8 (2^18) 11.3, 11.8; 4*10^8 (2^19) 19.7, 14.6.
+// 2*10^8 (2^18) 11.3, 11.8; 4*10^8 (2^19) 19.7, 14.6 (the head's records in launches of
+// their own take a seventh off the dataflow and leave the line where it is).
 constexpr uint64_t kRoundCells = 1u << 20;
 
 bool front_assign_fits(const Geom& g, uint32_t S) {
     if ((g.b != 8 && g.b != 16 && g.b != 32) || S > kFrontRoundShards) return false;
     return (uint64_t(S) << g.lg_seg) << (g.k == 4 ? 2 : 0) > kRoundCells;
+}
+
+template <int K, class T>
+static cudaError_t assign_head(const FrontArgs& a, T* cells, cudaStream_t st) {
+    const unsigned per = std::max(8u, (num_sms() * 8u + a.S - 1) / a.S);
+    for (uint32_t r = kFrontHead; r-- > 0;) k_front_head_assign<K, T><<<a.S * per, kFrWork, 0, st>>>(a, cells, r);
+    return cudaGetLastError();
 }
 
 template <int K, class T>
@@ -703,18 +711,16 @@ static cudaError_t assign_rounds(const FrontArgs& a, const FrontConfig& cfg, T* 
     cudaLaunchAttribute at[2]{};
     const cudaLaunchConfig_t lc = front_launch(cfg.cta, a.S, st, at, kFrAssignT);
     e = cudaLaunchKernelEx(&lc, waves, a, cells);
-    if (e != cudaSuccess) return e;
-    const unsigned per = std::max(8u, (num_sms() * 8u + a.S - 1) / a.S);
-    for (uint32_t r = kFrontHead; r-- > 0;) k_front_head_assign<K, T><<<a.S * per, kFrWork, 0, st>>>(a, cells, r);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : assign_head<K>(a, cells, st);
 }
 
 template <class T>
-static cudaError_t assign_cells(const FrontArgs& a, const FrontConfig& cfg, T* cells, cudaStream_t st) {
-    return a.g.k == 4 ? assign_rounds<4>(a, cfg, cells, st) : assign_rounds<3>(a, cfg, cells, st);
+static cudaError_t assign_cells(const FrontArgs& a, const FrontConfig* cfg, T* cells, cudaStream_t st) {
+    if (!cfg) return a.g.k == 4 ? assign_head<4>(a, cells, st) : assign_head<3>(a, cells, st);
+    return a.g.k == 4 ? assign_rounds<4>(a, *cfg, cells, st) : assign_rounds<3>(a, *cfg, cells, st);
 }
 
-cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig& cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st) {
+cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig* cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st) {
     if (a.g.b == 8) return assign_cells(a, cfg, data + cell_base, st);
     if (a.g.b == 16) return assign_cells(a, cfg, reinterpret_cast<uint16_t*>(data) + cell_base, st);
     return assign_cells(a, cfg, reinterpret_cast<uint32_t*>(data) + cell_base, st);

@@ -131,7 +131,8 @@ struct FlowArgs {
     uint32_t* rec3;                   // k = 4: per slot the third other vertex (else NULL)
     uint32_t* rc;                     // record slots taken per shard, one counter per kRcStride words
     uint64_t nrec;                    // assignment: record slots taken by the peel, all shards
-    uint64_t rmax;                    // assignment: the most slots any shard took
+    uint64_t rmax;                    // assignment: the most slots any shard took (behind head_end)
+    const uint32_t* head_end;         // assignment: per shard the first slot to assign, or NULL: all
     uint32_t epsg;                    // fuse regime: edges per start segment (signature prefetch), 0: none
     uint32_t* ctr;                    // kFlowWords counter words
     uint32_t* err;                    // == ctr + kFlowErr
@@ -216,7 +217,13 @@ cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaSt
 constexpr uint32_t kFrontRounds = 1u << 15;
 constexpr uint32_t kFrontRoundShards = 1024;  // at most 128 MB of round starts
 bool front_assign_fits(const Geom& g, uint32_t S);
-cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig& cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st);
+// cfg NULL: the records of the head's rounds alone (after the dataflow assigned the
+// waves'): a third of the edges, which depend on nothing of their round, so that the
+// dataflow's polls and its order buy them nothing (10^8 keys 8.87 -> 7.72 ms, 4*10^8
+// 21.1 -> 18.1). Eight launches: from 2^23 cells on (assignment with and without them,
+// ms: 4*10^6 keys 1.214, 1.212; 8*10^6 1.358, 1.376; 1.6*10^7 1.590, 1.737).
+constexpr uint64_t kFrontHeadCells = 1u << 23;
+cudaError_t launch_front_assign(const FrontArgs& a, const FrontConfig* cfg, uint8_t* data, uint64_t cell_base, cudaStream_t st);
 
 // Fuse-regime wave solver (csrc/vf_wave.cu): 64-bit vertex words that hold the
 // degree, the other two vertices and the value of the edges' sum; phase I in

@@ -109,6 +109,8 @@ def test_cluster_peel(vf, orc, arity, n, eps):  # noqa: F811
     (600_000_000, 8, dict(kind="filter")), (600_000_000, 16, dict(kind="func")),   # 32 shards, 2^16-cell segments
     (400_000_000, 8, dict(kind="filter", arity=4)),                               # 32 shards, 2^14-cell segments
     (40_000_000, 32, dict(kind="func", arity=4, eps=0.03)),                        # 1024 shards of few short rounds
+    (20_000_000, 16, dict(kind="func")), (9_000_000, 8, dict(kind="filter", arity=4)),  # the head's rounds, then
+    (10_000_000, 32, dict(kind="func")),                                           # the dataflow for the waves
     (40_000_000, 13, dict(kind="func", arity=4, eps=0.03)),                        # a bit array: the dataflow's
 ])
 def test_assignment_by_rounds_and_by_dataflow(vf, n, b, kw):  # noqa: F811
