@@ -620,7 +620,8 @@ __global__ void __launch_bounds__(kFT) k_final_init(FlowArgs a) {
 // grab: 32 consecutive records of one shard, whose vertices were peeled close
 // together; 2.5% faster than interleaving single records), so every shard's
 // dataflow advances at once; a record waits only on larger slots of its own
-// shard, which come at smaller positions.
+// shard, which come at smaller positions. Slots below a shard's head_end are left
+// out: the head rounds' records, assigned by launches of their own.
 template <int K, class FV>
 __global__ void __launch_bounds__(kFT) k_flow_assign(FlowArgs a) {
     using word = cuda::atomic_ref<FV, cuda::thread_scope_device>;
