@@ -332,6 +332,12 @@ vf_status vf_build_static(const uint64_t *keys, const void *values, uint64_t n, 
  * Errors: VF_EINVAL (fail_attempts < 0). */
 vf_status vf_debug_faults(int fail_attempts, uint32_t assign_poll_limit, int stall_assign);
 
+/* The same for the clusters that peel fuse graphs (VF_SOLVER_FLOW); off by default.
+ *   poll_limit: tests of its mbarrier after which a CTA's wait for the sizes of a
+ *     round gives up (0: the default, over a second). The clusters then leave the
+ *     peel, the build returns VF_ETIMEOUT and the CUDA context stays usable. */
+vf_status vf_debug_front(uint32_t poll_limit);
+
 /* Random 32-byte sector reads per second that this device delivers from a
  * table of table_bytes bytes (the paper has no counterpart; a measurement
  * aid for the query's roofline). A query reads three cells at random

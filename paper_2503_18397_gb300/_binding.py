@@ -127,8 +127,9 @@ def lib():
         L.vf_last_error.argtypes = []
         L.vf_last_error.restype = C.c_char_p
         L.vf_debug_faults.argtypes = [i32, C.c_uint32, i32]
+        L.vf_debug_front.argtypes = [C.c_uint32]
         for name in ("vf_build", "vf_query", "vf_get_info", "vf_plan", "vf_data", "vf_export", "vf_signatures",
-                     "vf_free", "vf_timing_enable", "vf_timing_read", "vf_debug_faults"):
+                     "vf_free", "vf_timing_enable", "vf_timing_read", "vf_debug_faults", "vf_debug_front"):
             getattr(L, name).restype = C.c_int
         _lib = L
     return _lib
@@ -442,6 +443,11 @@ def vf_timing_enable(on: bool = True):
 def vf_debug_faults(fail_attempts: int = 0, assign_poll_limit: int = 0, stall_assign: bool = False):
     """Fault injection for tests (process-wide; all zero = off)."""
     _check(lib().vf_debug_faults(int(fail_attempts), int(assign_poll_limit), 1 if stall_assign else 0))
+
+
+def vf_debug_front(poll_limit: int = 0):
+    """Limits of the cluster peel for tests (process-wide; zero = off)."""
+    _check(lib().vf_debug_front(int(poll_limit)))
 
 
 def vf_sector_rate(table_bytes: int, stream=None) -> float:

@@ -25,6 +25,7 @@ thread_local std::string g_last_error;
 std::atomic<int> g_debug_fail_attempts{0};
 std::atomic<uint32_t> g_debug_assign_limit{0};
 std::atomic<int> g_debug_stall_assign{0};
+std::atomic<uint32_t> g_debug_front_limit{0};  // vf_debug_front
 
 vf_status fail(vf_status st, const std::string& msg) {
     g_last_error = msg;
@@ -514,6 +515,8 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
             }
             f.epsg = a.epsg;
             f.ahead = 5;  // (none: +5% at 10^8 keys; 12: +3%)
+            f.polls = g_debug_front_limit.load();
+            if (f.polls == 0) f.polls = vf::kFrontPolls;
             f.err = a.ctr + vf::kFrontErr;
             f.err_before = a.err;
             PhaseTimer t(kPhPeel, st, int(vf::kFrontHead) + 3);  // scan, head rounds, waves; peeled count
@@ -533,7 +536,8 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
             VF_CK(cudaMemcpyAsync(hhead.data(), f.rcv + vf::kFrontHead * in.shards, hhead.size() * 4, cudaMemcpyDeviceToHost, st));
         VF_CK(cudaStreamSynchronize(st));
         // a list beyond its room: the worklist takes the attempt alone, from the start
-        if (waves && ((h[vf::kFlowErr] | h[vf::kFrontErr]) & (vf::kErrFrontier | vf::kErrCapacity))) continue;
+        const uint32_t we = h[vf::kFlowErr] | h[vf::kFrontErr];
+        if (waves && !(we & vf::kErrTimeout) && (we & (vf::kErrFrontier | vf::kErrCapacity))) continue;
         by_round = by_round && waves;
         break;
     }
@@ -1869,6 +1873,11 @@ vf_status vf_debug_faults(int fail_attempts, uint32_t assign_poll_limit, int sta
     g_debug_fail_attempts = fail_attempts;
     g_debug_assign_limit = assign_poll_limit;
     g_debug_stall_assign = stall_assign != 0;
+    return VF_OK;
+}
+
+vf_status vf_debug_front(uint32_t poll_limit) {
+    g_debug_front_limit = poll_limit;
     return VF_OK;
 }
 

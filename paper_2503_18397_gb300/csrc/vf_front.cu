@@ -19,6 +19,10 @@
 // sizes before its own). No fence is needed: what a round hands to the next in
 // global memory is fetch-and-adds whose results have come back. (A
 // barrier.cluster with release and acquire costs ~650 cycles.)
+// The wait for it is bounded. A CTA whose wait runs out leaves a mark with every CTA
+// of the cluster before it comes to its next cluster barrier, and all of them leave
+// the peel behind that barrier, whichever of theirs it meets: the marks that name
+// a barrier are the same for all behind it.
 //
 // Vertex words, claims and records are the worklist solver's. An edge claimed
 // for a vertex at the end of round r is removed in round r+1. A round's
@@ -51,7 +55,6 @@ constexpr int kFrWork = 256;            // threads that hold frontier entries
 constexpr int kFrT = kFrWork + 32;      // and the warp that exchanges the sizes
 constexpr uint32_t kFrList = 2048;      // frontier entries a CTA holds in shared memory, per buffer
 constexpr uint32_t kFrMaxC = 16;        // CTAs per cluster
-constexpr uint32_t kFrPolls = 1u << 26; // tests of an exchange's wait (some 20 ns each): then it gives up
 constexpr uint32_t kFrHole = 0xFFFFFFFFu;
 constexpr int kFrHeadT = 1024;          // threads of a head round's block (one block per list)
 constexpr uint32_t kFrHeadPer = 4;      // entries a thread has in flight there (2: +0.15 ms at 10^8 keys)
@@ -304,7 +307,9 @@ struct FrontShared {
     uint32_t cnt[3];                           // frontier counts; round r counts its next one in cnt[(r + 1) % 3]
     uint32_t deal;                             // entries dealt out by this CTA so far
     uint32_t total[2], most[2];                // of the exchange of even and odd rounds: all entries, the largest CTA's
-    uint32_t fail;                             // a wait gave up
+    uint32_t fail[2];                          // a wait of that exchange gave up
+    uint2 mark[kFrMaxC];                       // by a CTA whose wait did: the cluster barrier it comes to next (they
+                                               // are counted from 1), its exchanges so far
 };
 
 // K: vertices per edge (3, or 4 for a 4-uniform fuse graph). VAL: a function.
@@ -331,11 +336,40 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
         for (int j = 0; j < 2; j++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_addr + 8u * j) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        sh.deal = sh.fail = 0;
+        sh.deal = sh.fail[0] = sh.fail[1] = 0;
+        for (uint32_t j = 0; j < kFrMaxC; j++) sh.mark[j] = make_uint2(0, 0);
     }
     uint32_t xr = 0;  // exchanges so far: mbar[xr & 1], whose phase parity is (xr >> 1) & 1
-    bool failed = false;
-    for (uint32_t s = cid; s < a.S && !failed; s += ncl) {
+    // This CTA's size for exchange x to every CTA (the exchanger's).
+    auto post = [&](uint32_t x, uint32_t n) {
+        const uint32_t p = x & 1u;
+        if (lane < C) post_u32(to_size + 4u * kFrMaxC * p, n, to_mbar + 8u * p);
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar_addr + 8u * p), "r"(4u * C)
+                         : "memory");
+    };
+    // Waits for exchange x; false, for the warp alike: not after `most` tests.
+    auto arrived = [&](uint32_t x, uint32_t most) {
+        uint32_t polls = 0;
+        bool in = true;
+        while (!mbar_try(mbar_addr + 8u * (x & 1u), (x >> 1) & 1u)) {
+            if (++polls > most) {
+                in = false;
+                break;
+            }
+        }
+        return __all_sync(0xFFFFFFFFu, in) != 0;
+    };
+    uint32_t bars = 0, gone = 0;  // cluster barriers so far; the most exchanges a CTA that gave up had posted
+    // A cluster barrier; true, for all CTAs alike: a wait ran out, leave.
+    auto meet = [&]() {
+        cluster_barrier();
+        bars++;
+        const volatile uint2& m = sh.mark[lane & (kFrMaxC - 1u)];
+        gone = __reduce_max_sync(0xFFFFFFFFu, m.x == bars ? m.y : 0u);
+        return gone != 0;
+    };
+    for (uint32_t s = cid; s < a.S; s += ncl) {
         const uint32_t base = s * cells;
         const unsigned long long st0 = __ldg(a.start + s);
         const uint32_t ns = uint32_t(__ldg(a.start + s + 1) - st0);
@@ -352,24 +386,20 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
         for (uint32_t i = tid; i < left && i < kFrList; i += kFrT) sh.list[0][i] = __ldcg(list0 + i);
         if (tid < 3) sh.cnt[tid] = tid == 0 ? left : 0u;
         __syncthreads();
-        cluster_barrier();  // every CTA's counters (and at first its mbarriers) are ready
+        if (meet()) break;  // every CTA's counters (and at first its mbarriers) are ready
         uint32_t before = __ldcg(a.rcv + uint64_t(kFrontHead) * a.S + s);  // record slots taken so far
         // segments whose words and signatures have been asked for: [0, pf_lo) and (pf_hi, T)
         int pf_lo = 0, pf_hi = int(cells >> lgs) - 1;
         uint32_t c0 = 0, c1 = 1, c2 = 2;  // r % 3, (r + 1) % 3, (r + 2) % 3
         uint32_t rounds = 0;  // (the exchanger's)
+        bool gave_up = false;
         for (uint32_t cur = 0;; cur ^= 1u) {
             uint32_t n = sh.cnt[c0];
             n = min(n, max(a.list_cap, kFrList));
-            const uint32_t p = xr & 1u, parity = (xr >> 1) & 1u, mb = mbar_addr + 8u * p;
-            xr++;
+            const uint32_t x0 = xr++, p = x0 & 1u;
             if (exchanger) {
-                if (lane < C) post_u32(to_size + 4u * kFrMaxC * p, n, to_mbar + 8u * p);
-                if (lane == 0) {
-                    sh.cnt[c2] = 0;  // last read a round ago; pushed to from the next round on
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(4u * C)
-                                 : "memory");
-                }
+                post(x0, n);
+                if (lane == 0) sh.cnt[c2] = 0;  // last read a round ago; pushed to from the next round on
                 if (n > 0) {
                     // while the sizes are on their way: what the waves reach next comes to L2
                     const bool have = lane < n;
@@ -395,13 +425,7 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.loc + e0), "r"(bytes) : "memory");
                     }
                 }
-                uint32_t polls = 0;
-                while (!mbar_try(mb, parity)) {
-                    if (++polls > kFrPolls) {
-                        sh.fail = 1;
-                        break;
-                    }
-                }
+                if (!arrived(x0, a.polls)) sh.fail[p] = 1;
                 const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
                 const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz), most = __reduce_max_sync(0xFFFFFFFFu, sz);
                 if (lane == 0) sh.total[p] = total, sh.most[p] = most;
@@ -417,12 +441,9 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 auto entry = [&]() { return i < kFrList ? sh.list[cur][i] : __ldcg(list0 + cur * a.list_cap + i); };
                 if (i < n) front_fetch<K, VAL>(x, a, entry(), st0, ns);
                 if (x.on) front_others(x, a.g, st0);
-                uint32_t polls = 0;
-                while (!mbar_try(mb, parity)) {
-                    if (++polls > kFrPolls) {
-                        sh.fail = 1;
-                        break;
-                    }
+                if (!arrived(x0, a.polls)) {  // the sizes are not known: the list stays as it is
+                    sh.fail[p] = 1;
+                    n = 0;
                 }
                 uint32_t at = 0;
                 bool deal = false;
@@ -476,13 +497,16 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 }
             }
             __syncthreads();
-            // equal in every CTA of the cluster, and so are the ways out below
-            const uint32_t total = sh.total[p];
-            if (sh.fail) {
-                failed = true;
+            if (sh.fail[p]) {  // (the other exchange's flag is set behind the next barrier at the earliest)
                 if (tid == 0) atomicOr(a.err, kErrTimeout);
+                if (tid < C)
+                    asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(map_to_cta(smem_u32(&sh.mark[rank]), tid)),
+                                 "r"(bars + 1u), "r"(xr)
+                                 : "memory");
                 break;
             }
+            // equal in every CTA that knows the round's sizes, and so are the ways out below
+            const uint32_t total = sh.total[p];
             if (total == 0) {
                 if (rank == 0 && tid == 0) a.rc[s * kRcStride] = before;
                 break;
@@ -492,11 +516,22 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 if (tid == 0) atomicOr(a.err, kErrFrontier);
                 break;
             }
-            if (front_uneven(sh.most[p], total, a.lg_cta)) cluster_barrier();  // this round's pushes were dealt out
+            if (front_uneven(sh.most[p], total, a.lg_cta)) {  // this round's pushes were dealt out
+                gave_up = meet();
+                if (gave_up) break;
+            }
             const uint32_t t = c0;
             c0 = c1, c1 = c2, c2 = t;
         }
-        cluster_barrier();  // no CTA starts the next shard (or leaves) while a peer still works on this one
+        if (gave_up || meet()) break;  // no CTA starts the next shard (or leaves) while a peer still works on this one
+    }
+    // After a wait ran out: sizes may be on their way still. The CTAs are at most one
+    // exchange apart (the next one takes a size of all), so those behind post it too,
+    // and no CTA ends before all of both exchanges' sizes have come to it.
+    if (gone && exchanger) {
+        if (xr < gone) post(xr, 0);
+        if (gone > 1) arrived(gone - 2, kFrontPolls);
+        arrived(gone - 1, kFrontPolls);
     }
 }
 

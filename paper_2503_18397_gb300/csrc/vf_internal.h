@@ -181,6 +181,7 @@ uint64_t segment_order_bins(const Geom& g, uint32_t S);
 // Peeling of fuse shards in synchronous rounds, the waves by a cluster of CTAs
 // per shard (csrc/vf_front.cu); words, claims and records as the worklist solver's.
 constexpr uint32_t kFrontHead = 8;    // rounds before the waves (even), a launch each
+constexpr uint32_t kFrontPolls = 1u << 26;  // some 20 ns each
 struct FrontConfig {
     unsigned cta = 0, clusters = 0;   // CTAs per cluster, clusters of the launch
 };
@@ -202,6 +203,7 @@ struct FrontArgs {
     uint32_t* round;                  // record slots taken before each round of a shard's waves (kFrontRounds a shard)
     uint32_t epsg;                    // edges per start segment
     uint32_t ahead;                   // segments ahead of a wave's middle that are brought to L2
+    uint32_t polls;                   // tests of an exchange's wait, then it gives up
     uint32_t lg_cta;                  // lg of the cluster size
     uint32_t* err;                    // error bits
     const uint32_t* err_before;       // error bits of the incidence

@@ -79,3 +79,24 @@ def test_assignment_wait_runs_out_and_the_context_stays_usable(vf):
     assert (s.query(_dev(keys)).cpu().numpy() == vals).all()
     s.free()
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n,arity,eps", [(1 << 20, 3, 0.001), (5_000_000, 4, 0.01)])
+@pytest.mark.parametrize("limit", [1, 10])
+def test_exchange_wait_runs_out_and_the_context_stays_usable(vf, limit, n, arity, eps):
+    # one shard and several; 4-uniform rounds deal their pushes out, with a barrier of their own
+    keys, vals = synth.u64_keys(0, n, 63), synth.values(n, 8, 63)
+    p = vf.vf_params_default(kind=vf.FUNC, b=8, seed=7, mode=vf.MODE_FUSE, arity=arity, eps=eps, max_retries=30)
+    k, v = _dev(keys), _dev(vals)
+    try:
+        vf.vf_debug_front(poll_limit=limit)
+        for _ in range(3):
+            with pytest.raises(vf.VFError) as ei:
+                vf.vf_build(k, v, params=p)
+            assert ei.value.status == 5  # VF_ETIMEOUT
+    finally:
+        vf.vf_debug_front()
+    s = vf.vf_build(k, v, params=p)
+    assert bool((s.query(k) == v).all())
+    s.free()
+    torch.cuda.synchronize()
