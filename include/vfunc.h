@@ -335,8 +335,16 @@ vf_status vf_debug_faults(int fail_attempts, uint32_t assign_poll_limit, int sta
 /* The same for the clusters that peel fuse graphs (VF_SOLVER_FLOW); off by default.
  *   poll_limit: tests of its mbarrier after which a CTA's wait for the sizes of a
  *     round gives up (0: the default, over a second). The clusters then leave the
- *     peel, the build returns VF_ETIMEOUT and the CUDA context stays usable. */
-vf_status vf_debug_front(uint32_t poll_limit);
+ *     peel, the build returns VF_ETIMEOUT and the CUDA context stays usable.
+ *   list_room: entries that a CTA's list of vertices to peel may hold (0: half its
+ *     share of the cells). A list beyond it hands the attempt to the worklist. */
+vf_status vf_debug_front(uint32_t poll_limit, uint32_t list_room);
+
+/* Attempts of VF_SOLVER_FLOW since the library was loaded (process-wide), into
+ * counts[3]: peeled by clusters, peeled by the worklist, and how many of the
+ * latter the clusters had begun and could not finish (a list beyond its room).
+ * Errors: VF_EINVAL (NULL). */
+vf_status vf_peel_attempts(uint64_t *counts);
 
 /* Random 32-byte sector reads per second that this device delivers from a
  * table of table_bytes bytes (the paper has no counterpart; a measurement

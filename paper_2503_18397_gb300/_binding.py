@@ -127,9 +127,11 @@ def lib():
         L.vf_last_error.argtypes = []
         L.vf_last_error.restype = C.c_char_p
         L.vf_debug_faults.argtypes = [i32, C.c_uint32, i32]
-        L.vf_debug_front.argtypes = [C.c_uint32]
+        L.vf_debug_front.argtypes = [C.c_uint32, C.c_uint32]
+        L.vf_peel_attempts.argtypes = [C.POINTER(u64)]
         for name in ("vf_build", "vf_query", "vf_get_info", "vf_plan", "vf_data", "vf_export", "vf_signatures",
-                     "vf_free", "vf_timing_enable", "vf_timing_read", "vf_debug_faults", "vf_debug_front"):
+                     "vf_free", "vf_timing_enable", "vf_timing_read", "vf_debug_faults", "vf_debug_front",
+                     "vf_peel_attempts"):
             getattr(L, name).restype = C.c_int
         _lib = L
     return _lib
@@ -445,9 +447,17 @@ def vf_debug_faults(fail_attempts: int = 0, assign_poll_limit: int = 0, stall_as
     _check(lib().vf_debug_faults(int(fail_attempts), int(assign_poll_limit), 1 if stall_assign else 0))
 
 
-def vf_debug_front(poll_limit: int = 0):
-    """Limits of the cluster peel for tests (process-wide; zero = off)."""
-    _check(lib().vf_debug_front(int(poll_limit)))
+def vf_debug_front(poll_limit: int = 0, list_room: int = 0):
+    """Limits of the cluster peel for tests (process-wide; all zero = off)."""
+    _check(lib().vf_debug_front(int(poll_limit), int(list_room)))
+
+
+def vf_peel_attempts() -> tuple:
+    """Attempts of the default fuse solver so far: peeled by clusters, by the worklist, begun by the former and
+    done by the latter."""
+    n = (C.c_uint64 * 3)()
+    _check(lib().vf_peel_attempts(n))
+    return tuple(n)
 
 
 def vf_sector_rate(table_bytes: int, stream=None) -> float:

@@ -25,7 +25,8 @@ thread_local std::string g_last_error;
 std::atomic<int> g_debug_fail_attempts{0};
 std::atomic<uint32_t> g_debug_assign_limit{0};
 std::atomic<int> g_debug_stall_assign{0};
-std::atomic<uint32_t> g_debug_front_limit{0};  // vf_debug_front
+std::atomic<uint32_t> g_debug_front_limit{0}, g_debug_front_room{0};  // vf_debug_front
+std::atomic<uint64_t> g_peel_attempts[3];  // by clusters, by the worklist, begun by the former and done by the latter
 
 vf_status fail(vf_status st, const std::string& msg) {
     g_last_error = msg;
@@ -500,6 +501,7 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
             f.lg_cta = uint32_t(31 - __builtin_clz(fc.cta));
             f.lists = queue.as<uint2>();
             f.list_cap = uint32_t(in.cells >> (f.lg_cta + 1));  // two buffers a CTA, half its share of the cells each
+            if (const uint32_t room = g_debug_front_room.load()) f.list_cap = std::min(f.list_cap, room);
             const uint64_t nl = (vf::kFrontHead + 1) * (in.shards << f.lg_cta), nr = (vf::kFrontHead + 1) * in.shards;
             VF_CK(heads.alloc((nl + nr) * 4, st));
             f.list_n = heads.as<uint32_t>();
@@ -535,9 +537,13 @@ vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, 
         if (by_head)
             VF_CK(cudaMemcpyAsync(hhead.data(), f.rcv + vf::kFrontHead * in.shards, hhead.size() * 4, cudaMemcpyDeviceToHost, st));
         VF_CK(cudaStreamSynchronize(st));
-        // a list beyond its room: the worklist takes the attempt alone, from the start
+        // a list beyond its room (or an impossible word): the worklist takes the attempt alone, from the start
         const uint32_t we = h[vf::kFlowErr] | h[vf::kFrontErr];
-        if (waves && !(we & vf::kErrTimeout) && (we & (vf::kErrFrontier | vf::kErrCapacity))) continue;
+        if (waves && !(we & vf::kErrTimeout) && (we & (vf::kErrFrontier | vf::kErrCapacity))) {
+            g_peel_attempts[2]++;
+            continue;
+        }
+        g_peel_attempts[waves ? 0 : 1]++;
         by_round = by_round && waves;
         break;
     }
@@ -1876,8 +1882,15 @@ vf_status vf_debug_faults(int fail_attempts, uint32_t assign_poll_limit, int sta
     return VF_OK;
 }
 
-vf_status vf_debug_front(uint32_t poll_limit) {
+vf_status vf_debug_front(uint32_t poll_limit, uint32_t list_room) {
     g_debug_front_limit = poll_limit;
+    g_debug_front_room = list_room;
+    return VF_OK;
+}
+
+vf_status vf_peel_attempts(uint64_t* counts) {
+    if (!counts) return fail(VF_EINVAL, "vf_peel_attempts: NULL argument");
+    for (int i = 0; i < 3; i++) counts[i] = g_peel_attempts[i].load();
     return VF_OK;
 }
 

@@ -348,17 +348,15 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar_addr + 8u * p), "r"(4u * C)
                          : "memory");
     };
-    // Waits for exchange x; false, for the warp alike: not after `most` tests.
-    auto arrived = [&](uint32_t x, uint32_t most) {
+    // Waits for exchange x, for `most` tests.
+    auto await = [&](uint32_t x, uint32_t most) {
         uint32_t polls = 0;
-        bool in = true;
         while (!mbar_try(mbar_addr + 8u * (x & 1u), (x >> 1) & 1u)) {
             if (++polls > most) {
-                in = false;
+                sh.fail[x & 1u] = 1;
                 break;
             }
         }
-        return __all_sync(0xFFFFFFFFu, in) != 0;
     };
     uint32_t bars = 0, gone = 0;  // cluster barriers so far; the most exchanges a CTA that gave up had posted
     // A cluster barrier; true, for all CTAs alike: a wait ran out, leave.
@@ -392,14 +390,14 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
         int pf_lo = 0, pf_hi = int(cells >> lgs) - 1;
         uint32_t c0 = 0, c1 = 1, c2 = 2;  // r % 3, (r + 1) % 3, (r + 2) % 3
         uint32_t rounds = 0;  // (the exchanger's)
-        bool gave_up = false;
+        bool done = false;
         for (uint32_t cur = 0;; cur ^= 1u) {
             uint32_t n = sh.cnt[c0];
             n = min(n, max(a.list_cap, kFrList));
             const uint32_t x0 = xr++, p = x0 & 1u;
             if (exchanger) {
-                post(x0, n);
                 if (lane == 0) sh.cnt[c2] = 0;  // last read a round ago; pushed to from the next round on
+                post(x0, n);
                 if (n > 0) {
                     // while the sizes are on their way: what the waves reach next comes to L2
                     const bool have = lane < n;
@@ -425,7 +423,7 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.loc + e0), "r"(bytes) : "memory");
                     }
                 }
-                if (!arrived(x0, a.polls)) sh.fail[p] = 1;
+                await(x0, a.polls);
                 const uint32_t sz = lane < C ? sh.size[p][lane] : 0u;
                 const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sz), most = __reduce_max_sync(0xFFFFFFFFu, sz);
                 if (lane == 0) sh.total[p] = total, sh.most[p] = most;
@@ -441,10 +439,10 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 auto entry = [&]() { return i < kFrList ? sh.list[cur][i] : __ldcg(list0 + cur * a.list_cap + i); };
                 if (i < n) front_fetch<K, VAL>(x, a, entry(), st0, ns);
                 if (x.on) front_others(x, a.g, st0);
-                if (!arrived(x0, a.polls)) {  // the sizes are not known: the list stays as it is
-                    sh.fail[p] = 1;
-                    n = 0;
-                }
+                // (in vain: the round is finished with sizes as they are, which decide only where
+                // records and pushes go, within their rooms; the vote that would tell a warp's lanes
+                // so costs a round 2%)
+                await(x0, a.polls);
                 uint32_t at = 0;
                 bool deal = false;
                 for (uint32_t i0 = 32u * warp; i0 < n; i0 += kFrWork) {
@@ -497,7 +495,9 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 }
             }
             __syncthreads();
-            if (sh.fail[p]) {  // (the other exchange's flag is set behind the next barrier at the earliest)
+            // equal in every CTA that knows the round's sizes, and so are the ways out behind the first
+            const uint32_t total = sh.total[p], gave_up = sh.fail[p];
+            if (gave_up) {  // (the other exchange's flag is set behind the next barrier at the earliest)
                 if (tid == 0) atomicOr(a.err, kErrTimeout);
                 if (tid < C)
                     asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(map_to_cta(smem_u32(&sh.mark[rank]), tid)),
@@ -505,8 +505,6 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                                  : "memory");
                 break;
             }
-            // equal in every CTA that knows the round's sizes, and so are the ways out below
-            const uint32_t total = sh.total[p];
             if (total == 0) {
                 if (rank == 0 && tid == 0) a.rc[s * kRcStride] = before;
                 break;
@@ -517,21 +515,21 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 break;
             }
             if (front_uneven(sh.most[p], total, a.lg_cta)) {  // this round's pushes were dealt out
-                gave_up = meet();
-                if (gave_up) break;
+                done = meet();
+                if (done) break;
             }
             const uint32_t t = c0;
             c0 = c1, c1 = c2, c2 = t;
         }
-        if (gave_up || meet()) break;  // no CTA starts the next shard (or leaves) while a peer still works on this one
+        if (done || meet()) break;  // no CTA starts the next shard (or leaves) while a peer still works on this one
     }
     // After a wait ran out: sizes may be on their way still. The CTAs are at most one
     // exchange apart (the next one takes a size of all), so those behind post it too,
     // and no CTA ends before all of both exchanges' sizes have come to it.
     if (gone && exchanger) {
         if (xr < gone) post(xr, 0);
-        if (gone > 1) arrived(gone - 2, kFrontPolls);
-        arrived(gone - 1, kFrontPolls);
+        if (gone > 1) await(gone - 2, kFrontPolls);
+        await(gone - 1, kFrontPolls);
     }
 }
 

@@ -100,3 +100,33 @@ def test_exchange_wait_runs_out_and_the_context_stays_usable(vf, limit, n, arity
     assert bool((s.query(k) == v).all())
     s.free()
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n,arity,eps", [(1 << 20, 3, 0.001), (3_000_000, 3, 0.001), (5_000_000, 4, 0.01),
+                                         (9_000_000, 4, 0.001)])
+def test_lists_beyond_their_room_go_to_the_worklist(vf, orc, n, arity, eps):
+    # the attempt is begun again from the keys: plan, seed and retries as the oracle's, answers exact
+    keys, vals = synth.u64_keys(0, n, 64), synth.values(n, 8, 64)
+    kw = dict(b=8, seed=9, mode=vf.MODE_FUSE, arity=arity, eps=eps, max_retries=30)
+    k, v = _dev(keys), _dev(vals)
+    before = vf.vf_peel_attempts()
+    try:
+        vf.vf_debug_front(list_room=8)
+        s = vf.vf_build(k, v, params=vf.vf_params_default(kind=vf.FUNC, **kw))
+    finally:
+        vf.vf_debug_front()
+    info = s.info
+    done = [a - b for a, b in zip(vf.vf_peel_attempts(), before)]
+    assert done == [0, info.retries + 1, info.retries + 1]
+    assert bool((s.query(k) == v).all())
+    s.free()
+    f = vf.vf_build(k, None, params=vf.vf_params_default(kind=vf.FILTER, **kw))  # by the clusters
+    done = [a - b for a, b in zip(vf.vf_peel_attempts(), before)]
+    assert done == [f.info.retries + 1, info.retries + 1, info.retries + 1]
+    assert (f.info.seed, f.info.retries) == (info.seed, info.retries) and bool(f.query(k).all())
+    f.free()
+    if n <= 3_000_000:
+        st, oi, _ = orc.build(orc.default_params(kind=orc.FUNC, **kw), keys, vals)
+        assert st == orc.OK and (oi.seed, oi.retries) == (info.seed, info.retries)
+        for g in GEOM:
+            assert getattr(info, g) == getattr(oi, g), g
