@@ -348,10 +348,13 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar_addr + 8u * p), "r"(4u * C)
                          : "memory");
     };
-    // Waits for exchange x, for `most` tests.
+    // Waits for exchange x, for `most` tests. (The first one on its own: with the limit
+    // compared in the only loop the peel takes 1.5% longer, 2^20 keys 2.63 against 2.59 ms.)
     auto await = [&](uint32_t x, uint32_t most) {
+        const uint32_t mb = mbar_addr + 8u * (x & 1u), parity = (x >> 1) & 1u;
+        if (mbar_try(mb, parity)) return;
         uint32_t polls = 0;
-        while (!mbar_try(mbar_addr + 8u * (x & 1u), (x >> 1) & 1u)) {
+        while (!mbar_try(mb, parity)) {
             if (++polls > most) {
                 sh.fail[x & 1u] = 1;
                 break;
@@ -440,8 +443,8 @@ __global__ void __launch_bounds__(kFrT) k_front_peel(FrontArgs a) {
                 if (i < n) front_fetch<K, VAL>(x, a, entry(), st0, ns);
                 if (x.on) front_others(x, a.g, st0);
                 // (in vain: the round is finished with sizes as they are, which decide only where
-                // records and pushes go, within their rooms; the vote that would tell a warp's lanes
-                // so costs a round 2%)
+                // records and pushes go, within their rooms: a vote that told a warp's lanes so
+                // would cost every round)
                 await(x0, a.polls);
                 uint32_t at = 0;
                 bool deal = false;
