@@ -418,8 +418,9 @@ vf_status solve_rounds(const vf_info& in, const vf::Geom& g, const uint64_t* loc
     return VF_OK;
 }
 
-// One attempt of the default fuse-regime solver: peeling by clusters of CTAs (with
-// enough shards) or by the worklist, then the dataflow assignment. Returns VF_OK, VF_EBUILD (peel failed: retry), or an error.
+// One attempt of the default fuse-regime solver: peeling by clusters of CTAs or, where
+// that is faster (front_config), by the worklist; then the assignment, by rounds or as
+// a dataflow. Returns VF_OK, VF_EBUILD (peel failed: retry), or an error.
 vf_status solve_flow(const vf_info& in, const vf::Geom& g, const uint64_t* loc, const uint32_t* val,
                      const unsigned long long* start, uint8_t* data, cudaStream_t st, uint64_t* peeled,
                      uint64_t cell_base, const uint32_t* drop, uint64_t ndrop, DevBuf* claimed_out,

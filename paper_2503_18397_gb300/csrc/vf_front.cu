@@ -663,6 +663,30 @@ static cudaLaunchConfig_t front_launch(unsigned cta, unsigned clusters, cudaStre
     return lc;
 }
 
+// Where the clusters are faster than the worklist. The worklist has the whole chip at
+// work on whatever is ready; a cluster has 16 SMs for its shard and a round's latency
+// for its few entries (about 2^(lg_seg - 5); 2^(lg_seg - 3) where the graph is
+// 4-uniform). Peel and assignment of an attempt, ms, worklist and clusters:
+//  * a few large shards leave most SMs idle, in the head's rounds above all. 3-uniform,
+//    one shard: 2^14 cells a segment 4.9, 4.6 (4*10^6 cells), 2^15 5.3, 5.6 (8*10^6), 2^16 9.1,
+//    13.8; two: 2^16 20.4, 19.9, 2^17 25.2, 24.9 and 25.8, 32.4 (3, 5*10^7 cells each); four:
+//    2^17 34.9, 30.1 and 40.2, 41.3, 2^18 70, 53. 4-uniform: one or two shards: 2^13 10.4, 9.4
+//    (one), 10.8, 10.0 (two), 2^14 7.7, 8.4, 8.3, 9.0; four: 2^13 11.7, 10.7, 2^14 9.6, 9.8 and 18.5,
+//    19.6, 2^15 40.8, 45.0, 2^16 (beyond L2, where the worklist's wide front costs) 57.6, 51.4; eight: 2^14
+//    27.2, 23.8, 2^15 42.6, 28.7.
+//  * shards beyond the clusters resident at once (36) wait for one another. 4-uniform,
+//    64 shards: 2^10 2.9, 3.6, 2^11 5.4, 4.9, 2^12 11.0, 7.9; 256: 2^10 11.8, 11.9, 2^11 23.0,
+//    17.7; 1024: 2^9 8.1, 14.6, 2^10 42, 48, 2^11 89, 65.
+//  * rounds of one or two entries a CTA: 16 shards of 11520 cells 0.28, 0.30, of 22272 0.56,
+//    0.52.
+static bool front_pays(const Geom& g, uint32_t S, uint32_t clusters) {
+    if (S > clusters) return g.lg_seg >= 11;
+    if (g.cells < 1u << 14) return false;
+    if (S >= 8) return true;
+    if (g.k == 4) return g.lg_seg <= 13 || (S >= 4 && g.lg_seg >= 16);
+    return S >= 4 || g.lg_seg <= (S == 1 ? 14 : 16);
+}
+
 bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg) {
     if (g.regime != kRegimeFuse || (g.k != 3 && g.k != 4) || g.lg_seg < 5 || g.lg_seg > 26) return false;
     static std::mutex mu;
@@ -690,7 +714,7 @@ bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg) {
             cudaGetLastError();
         }
     }
-    if (k.cta == ~0u) return false;
+    if (k.cta == ~0u || !front_pays(g, S, k.clusters)) return false;
     cfg.cta = k.cta;
     cfg.clusters = std::max(1u, std::min(S, k.clusters));
     return true;

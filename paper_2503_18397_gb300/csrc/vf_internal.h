@@ -209,7 +209,7 @@ struct FrontArgs {
     const uint32_t* err_before;       // error bits of the incidence
 };
 // The launch's shape for S shards; false where the kernel does not apply (other
-// regimes, few shards, or a device without such clusters).
+// regimes, a device without such clusters) or the worklist is faster.
 bool front_config(const Geom& g, uint32_t S, FrontConfig& cfg);
 cudaError_t launch_front_peel(const FrontArgs& a, const FrontConfig& cfg, cudaStream_t st);
 // Assignment of the attempt's records round by round, last to first, straight in the

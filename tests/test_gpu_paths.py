@@ -190,3 +190,36 @@ def test_request_tiles(vf):  # noqa: F811
         reqs += [(s, dev(q[:m].copy()), None) for m in (1, 1023, 1024, 1025, 6000)]
     for (s, q, _), out in zip(reqs, vf.vf_query_batch(reqs)):
         assert (host(out) == host(s.query(q))).all()
+
+
+@pytest.mark.parametrize("n,arity,eps,shards,lg_seg,clusters", [
+    (3_571_428, 3, 0.0001, 1, 14, True), (4_999_999, 3, 0.0001, 1, 15, False),
+    (42_857_142, 3, 0.000364, 2, 16, True), (57_142_857, 3, 0.000315, 2, 17, False),
+    (228_571_428, 3, 0.000484, 8, 17, True),      # the waves begin with lists beyond shared memory
+    (5_185_185, 4, 0.0001, 1, 13, True), (7_407_407, 4, 0.0001, 1, 14, False),
+    (20_740_740, 4, 0.000946, 4, 13, True), (29_629_629, 4, 0.000781, 4, 14, False),
+    (237_037_037, 4, 0.000273, 4, 16, True),
+    (148_148, 4, 0.030999, 16, 8, False), (296_296, 4, 0.022183, 16, 8, True),
+    (10_666_666, 4, 0.008527, 64, 10, False), (21_333_333, 4, 0.006102, 64, 11, True),
+    (170_666_666, 4, 0.007388, 512, 11, True),    # many small shards assigned by rounds
+    (37_925_925, 4, 0.023269, 1024, 9, False)])
+def test_peel_by_clusters_or_worklist(vf, n, arity, eps, shards, lg_seg, clusters):  # noqa: F811
+    # both sides of each line of the rule, functions and filters
+    keys = synth.u64_keys_torch(0, n, 7)
+    vals = (keys & 0xFF).to(torch.uint8)
+    seeds = []
+    for v in (vals, None):
+        p = vf.vf_params_default(kind=vf.FILTER if v is None else vf.FUNC, b=8, mode=vf.MODE_FUSE, arity=arity, eps=eps,
+                                 seed=1, max_retries=40)
+        before = vf.vf_peel_attempts()
+        s = vf.vf_build(keys, v, params=p)
+        done = [a - b for a, b in zip(vf.vf_peel_attempts(), before)]
+        i = s.info
+        assert (i.shards, i.lg_seg) == (shards, lg_seg)
+        assert done == ([i.retries + 1, 0, 0] if clusters else [0, i.retries + 1, 0])
+        out = s.query(keys)
+        assert bool((out == vals).all()) if v is not None else bool(out.all())
+        seeds.append(i.seed)
+        s.free()
+        del out
+    assert seeds[0] == seeds[1]
