@@ -5,6 +5,8 @@
 // Each thread takes kQ keys spaced one grid-stride apart (coalesced key loads)
 // and issues all 3*kQ cell loads before using any, so every warp keeps 96
 // independent random 32-byte sector reads in flight.
+#include <algorithm>
+
 #include "vf_internal.h"
 
 namespace vf {
@@ -131,6 +133,7 @@ static void launch_w(bool bytes, const void* keys, const uint64_t* offs, uint64_
 // ------------------------------------------------------- cross-structure batch
 
 constexpr int kReqCache = 4096;
+constexpr uint32_t kFewRequests = 1024;  // k_query_few: requests it takes
 
 // The cells' XOR of key i of request r and its answer.
 __device__ __forceinline__ void query_one(const QueryReq& r, uint64_t i) {
@@ -154,13 +157,13 @@ __device__ __forceinline__ void query_one(const QueryReq& r, uint64_t i) {
     else put_answer<false>(r.out, i, x, local, r.g.b);
 }
 
-// kQ keys of one request per thread, spaced a block apart, with all their
-// cell loads in flight before any is used (as k_query).
-template <int WIDTH, bool FILTER, int K>
+// kQ keys of one request (of a 3-uniform structure) per thread, spaced a block
+// apart, with all their cell loads in flight before any is used (as k_query).
+template <int WIDTH, bool FILTER>
 __device__ __forceinline__ void query_tile(const QueryReq& r, uint64_t i0, uint32_t m) {
     const Geom g = r.g;
     const uint64_t* const keys = r.keys + i0;
-    uint64_t loc[kQ], cell[kQ][K];
+    uint64_t loc[kQ], cell[kQ][3];
 #pragma unroll
     for (int k = 0; k < kQ; k++) {
         const uint32_t i = threadIdx.x + k * kQThreads;
@@ -170,16 +173,15 @@ __device__ __forceinline__ void query_tile(const QueryReq& r, uint64_t i0, uint3
         uint64_t v[4];
         edge_of(g, loc[k], v);
 #pragma unroll
-        for (int j = 0; j < K; j++) cell[k][j] = base + v[j];
+        for (int j = 0; j < 3; j++) cell[k][j] = base + v[j];
     }
     uint32_t x[kQ];
 #pragma unroll
     for (int k = 0; k < kQ; k++) {
-        uint32_t c[K];
+        uint32_t c[3];
 #pragma unroll
-        for (int j = 0; j < K; j++) c[j] = threadIdx.x + k * kQThreads < m ? cell_q<WIDTH>(r.data, g.b, cell[k][j]) : 0u;
+        for (int j = 0; j < 3; j++) c[j] = threadIdx.x + k * kQThreads < m ? cell_q<WIDTH>(r.data, g.b, cell[k][j]) : 0u;
         x[k] = c[0] ^ c[1] ^ c[2];
-        if constexpr (K == 4) x[k] ^= c[3];
     }
 #pragma unroll
     for (int k = 0; k < kQ; k++) {
@@ -188,12 +190,37 @@ __device__ __forceinline__ void query_tile(const QueryReq& r, uint64_t i0, uint3
     }
 }
 
+// The request that key g of the launch belongs to; s_off: the offsets, where they fit
+// there (cached).
+__device__ __forceinline__ uint32_t request_of(const QueryReq* reqs, const uint64_t* s_off, bool cached, uint32_t count,
+                                               uint64_t g) {
+    uint32_t lo = 0, hi = count;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        const uint64_t o = cached ? s_off[mid] : reqs[mid].key_off;
+        if (o <= g) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // Requests against many resident structures in one launch: request r owns
-// keys [key_off, key_off + m) of the launch's key space. A block takes tiles of
-// consecutive keys; a tile almost always lies within one request, whose
-// descriptor is then looked up once for the block and whose keys go four a
-// thread (96 requests of 3*10^5 to 1.5*10^6 keys: 1.80 ms with a search and one key
-// a thread, 1.07 this way). A tile with a boundary in it is taken key by key.
+// keys [key_off, key_off + m) of the launch's key space. Few keys: one a thread,
+// each with its own search. At most kFewRequests.
+__global__ void __launch_bounds__(kQThreads) k_query_few(const QueryReq* __restrict__ reqs, uint32_t count, uint64_t total) {
+    __shared__ uint64_t s_off[kFewRequests];
+    for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) s_off[i] = reqs[i].key_off;
+    __syncthreads();
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    for (uint64_t g = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; g < total; g += stride) {
+        const QueryReq& q = reqs[request_of(reqs, s_off, true, count, g)];
+        query_one(q, g - q.key_off);
+    }
+}
+
+// Many: a block takes tiles of consecutive keys; a tile mostly lies within one
+// request, whose descriptor is then looked up once for the block and whose keys go
+// four a thread (96 requests of 3*10^5 to 1.5*10^6 keys: 1.80 ms with a search and one
+// key a thread, 1.07 this way). A tile with a boundary in it is taken key by key.
 __global__ void __launch_bounds__(kQThreads, 4) k_query_batch(const QueryReq* __restrict__ reqs, uint32_t count,
                                                            uint64_t total) {
     constexpr uint32_t kTileKeys = kQThreads * kQ;
@@ -202,46 +229,46 @@ __global__ void __launch_bounds__(kQThreads, 4) k_query_batch(const QueryReq* __
     if (cached)
         for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) s_off[i] = reqs[i].key_off;
     __syncthreads();
-    auto request_of = [&](uint64_t g) {
-        uint32_t lo = 0, hi = count;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            const uint64_t o = cached ? s_off[mid] : reqs[mid].key_off;
-            if (o <= g) lo = mid; else hi = mid;
-        }
-        return lo;
-    };
     for (uint64_t t0 = uint64_t(blockIdx.x) * kTileKeys; t0 < total; t0 += uint64_t(gridDim.x) * kTileKeys) {
         const uint32_t m = total - t0 < kTileKeys ? uint32_t(total - t0) : kTileKeys;
-        const uint32_t first = request_of(t0);
-        const QueryReq& r = reqs[first];
+        const QueryReq& r = reqs[request_of(reqs, s_off, cached, count, t0)];
         const uint64_t i0 = t0 - r.key_off;
         if (i0 + m <= r.m && r.g.k != 4 && (r.g.b == 8 || r.g.b == 16)) {
             if (r.g.kind == 1) {
-                if (r.g.b == 8) query_tile<8, true, 3>(r, i0, m);
-                else query_tile<16, true, 3>(r, i0, m);
+                if (r.g.b == 8) query_tile<8, true>(r, i0, m);
+                else query_tile<16, true>(r, i0, m);
             } else {
-                if (r.g.b == 8) query_tile<8, false, 3>(r, i0, m);
-                else query_tile<16, false, 3>(r, i0, m);
+                if (r.g.b == 8) query_tile<8, false>(r, i0, m);
+                else query_tile<16, false>(r, i0, m);
             }
         } else if (i0 + m <= r.m && r.g.k != 4 && r.g.b <= 32) {
-            if (r.g.kind == 1) query_tile<0, true, 3>(r, i0, m);
-            else query_tile<0, false, 3>(r, i0, m);
+            if (r.g.kind == 1) query_tile<0, true>(r, i0, m);
+            else query_tile<0, false>(r, i0, m);
         } else {
             for (uint32_t i = threadIdx.x; i < m; i += kQThreads) {
-                const QueryReq& q = reqs[request_of(t0 + i)];
+                const QueryReq& q = reqs[request_of(reqs, s_off, cached, count, t0 + i)];
                 query_one(q, t0 + i - q.key_off);
             }
         }
     }
 }
 
+// Up to five blocks of keys an SM, a key a thread: four keys of a thread after one
+// another on a quarter of the blocks cost more than they save. Device time, us, a key a
+// thread and tiles: one request of 1000 keys 5.6, 8.7 (wider than 32 bits 6.2, 10.3;
+// 4-uniform 6.1, 10.3), of 10^5 8.1, 8.5 (8.7, 11.7), of 2*10^5 10.6, 10.2, of 3*10^5 14.0, 10.1; 100 of
+// 500 9.9, 13.3; 300 of 500 10.6, 15.2; 700 of 500 22.5, 19.5; 10 of 20,000 10.9, 13.8, of
+// 30,000 14.8, 13.0. And not where every block would read thousands of offsets for a few
+// keys: 1000 of 64 13.4, 16.0; 3000 of 64 22.8, 18.6.
+constexpr uint32_t kFewBlocks = 5;
+
 cudaError_t launch_query_batch(const QueryReq* reqs, uint32_t count, uint64_t total, cudaStream_t st) {
     if (total == 0 || count == 0) return cudaSuccess;
-    uint64_t blocks = (total + kQThreads * kQ - 1) / (kQThreads * kQ);
-    const uint64_t cap = uint64_t(num_sms()) * 16;
-    if (blocks > cap) blocks = cap;
-    k_query_batch<<<unsigned(blocks < 1 ? 1 : blocks), kQThreads, 0, st>>>(reqs, count, total);
+    const bool few = count <= kFewRequests && total <= uint64_t(num_sms()) * kFewBlocks * kQThreads;
+    const uint64_t per = uint64_t(kQThreads) * (few ? 1 : kQ), cap = uint64_t(num_sms()) * 16;
+    const unsigned blocks = unsigned(std::min((total + per - 1) / per, cap));
+    if (few) k_query_few<<<blocks, kQThreads, 0, st>>>(reqs, count, total);
+    else k_query_batch<<<blocks, kQThreads, 0, st>>>(reqs, count, total);
     return cudaGetLastError();
 }
 

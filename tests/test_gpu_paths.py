@@ -223,3 +223,23 @@ def test_peel_by_clusters_or_worklist(vf, n, arity, eps, shards, lg_seg, cluster
         s.free()
         del out
     assert seeds[0] == seeds[1]
+
+
+@pytest.mark.parametrize("total,pieces", [(1, 1), (1000, 1), (194_560, 7), (194_561, 7), (30_000, 900), (30_000, 1400),
+                                          (500_000, 300)])
+def test_few_and_many_keys_of_requests(vf, total, pieces):  # noqa: F811
+    # a key a thread up to 5 * 152 * 256 keys and 1024 requests, tiles beyond; uneven requests of every kind
+    kinds = [(vf.FUNC, 8, {}), (vf.FILTER, 8, {}), (vf.FUNC, 16, {}), (vf.FUNC, 13, {}), (vf.FILTER, 33, {}),
+             (vf.FUNC, 40, {}), (vf.FUNC, 8, dict(mode=vf.MODE_FUSE, arity=4))]
+    kept = []
+    for i, (kind, b, kw) in enumerate(kinds):
+        n = 1_000_000 if kw else 20_000
+        k = synth.u64_keys(i << 32, n, 6)
+        v = synth.values(n, b, i) if kind == vf.FUNC else None
+        kept.append((vf.vf_build(dev(k), None if v is None else dev(v), params=vf.vf_params_default(kind=kind, b=b, seed=1, **kw)),
+                     dev(np.concatenate([k[:20_000], synth.u64_keys((1 << 50) + i, 20_000, 6)]))))
+    cuts = np.sort(np.random.default_rng(total).integers(0, total + 1, pieces - 1))
+    sizes = np.diff(np.concatenate([[0], cuts, [total]]))
+    reqs = [(kept[i % 7][0], kept[i % 7][1].repeat(5)[:m], None) for i, m in enumerate(sizes.tolist())]
+    for (s, q, _), out in zip(reqs, vf.vf_query_batch(reqs)):
+        assert len(q) == 0 or (host(out) == host(s.query(q))).all()
