@@ -166,12 +166,42 @@ __device__ __forceinline__ Sig sig_staged(const uint4* stage, uint32_t p, uint32
 
 // A block's tile of byte strings: their bytes, and their order by words.
 constexpr uint32_t kTileStrings = 256;  // the block's threads: a string each
+constexpr uint32_t kPartStrings = 48;   // strings too long for a stage together: as many as are staged at once, or none
 constexpr uint32_t kLenBins = 32;       // strings of as many words or more share the last bin
 struct StringTile {
     uint4 bytes[kStageBytes / 16];
     uint2 order[kTileStrings];  // staged offset | string << 16, length
     uint32_t bins[kLenBins];
 };
+
+// A tile of `count` strings from t0 on, bytes [lo, hi), that the stage does not hold: as
+// many strings at a time as fit, a string a thread (this one's bytes: [o0, o1)), while
+// these are kPartStrings at least; beyond that too few threads have one, and the rest is
+// hashed in place. Queries of 10^6 to 2*10^6 strings, us, in place and so: of 84 bytes on
+// average 162, 148, 150: 269, 221, 300: 272, 253 (all of 300: 238, 176), 500 (20 to 40 at a time):
+// 260, 300, 1000: 350, 616. Hash and histogram: 100: 190, 195, 150: 281, 246, 200: 198, 180, 300:
+// 294, 297.
+__device__ __forceinline__ Sig sig_parts(const uint8_t* buf, const uint64_t* __restrict__ offs, uint64_t total, uint64_t t0,
+                                 uint32_t count, uint64_t lo, uint64_t hi, uint64_t o0, uint64_t o1, uint4* stage,
+                                 uint64_t kh, uint64_t kl) {
+    const uint32_t tid = threadIdx.x;
+    // the offsets are the caller's: a tile of them out of order is hashed in place
+    const bool in_order = __syncthreads_and(o0 >= lo && o1 >= o0 && o1 <= hi && hi <= total);
+    Sig s{0, 0};
+    for (uint32_t a = 0, n; a < count; a += n) {
+        const uint64_t la = __ldg(offs + t0 + a);
+        n = in_order ? uint32_t(__syncthreads_count(tid >= a && tid < count && o1 - la <= kStageBytes - 48)) : 0u;
+        if (n < kPartStrings && a + n < count) {
+            if (tid >= a && tid < count) s = sig_bytes(buf, total, o0, o1 - o0, kh, kl);
+            break;
+        }
+        uint32_t at;
+        stage_bytes(buf, total, la, __ldg(offs + t0 + a + n), stage, at);
+        __syncthreads();
+        if (tid >= a && tid < a + n) s = sig_staged(stage, at + uint32_t(o0 - la), uint32_t(o1 - o0), kh, kl);
+    }
+    return s;
+}
 
 // Signature of one string of the tile [t0, t0 + kTileStrings) of m packed strings,
 // through `t`; i: which one, every string going to one thread (i >= m: none). Every
@@ -190,15 +220,15 @@ __device__ __forceinline__ Sig sig_tile(const uint8_t* buf, const uint64_t* __re
     if (tid < kLenBins) t.bins[tid] = 0;  // read by nobody since the barrier before the order was
     __syncthreads();                      // the tile before has been read
     uint32_t at;
-    bool staged = stage_bytes(buf, total, lo, hi, t.bytes, at);
+    if (!stage_bytes(buf, total, lo, hi, t.bytes, at))
+        return sig_parts(buf, offs, total, t0, uint32_t(t1 - t0), lo, hi, o0, o1, t.bytes, kh, kl);
     const uint32_t len = uint32_t(o1 - o0), p = at + uint32_t(o0 - lo);
     const uint32_t words = (len + 7) / 8, bin = words < kLenBins ? words : kLenBins - 1;
     // the offsets are the caller's: a tile of them out of order is hashed in place
-    const bool ok = staged && o0 >= lo && o1 >= o0 && o1 <= hi;
+    const bool ok = o0 >= lo && o1 >= o0 && o1 <= hi;
     uint32_t rank = 0;
     if (ok) rank = atomicAdd(&t.bins[bin], 1u);
-    staged = __syncthreads_and(ok);
-    if (!staged) return i < m ? sig_bytes(buf, total, o0, o1 - o0, kh, kl) : Sig{0, 0};
+    if (!__syncthreads_and(ok)) return i < m ? sig_bytes(buf, total, o0, o1 - o0, kh, kl) : Sig{0, 0};
     uint32_t upto = t.bins[lane];
     const uint32_t mine = upto;
 #pragma unroll
@@ -212,6 +242,27 @@ __device__ __forceinline__ Sig sig_tile(const uint8_t* buf, const uint64_t* __re
     const uint2 x = t.order[tid];
     i = t0 + (x.x >> 16);
     return i < m ? sig_staged(t.bytes, x.x & 0xFFFFu, x.y, kh, kl) : Sig{0, 0};
+}
+
+// Whether all strings seem to be of one length (a guess, which decides only how they
+// are read).
+__device__ __forceinline__ bool strings_alike(const uint64_t* __restrict__ offs, uint64_t n, uint64_t total) {
+    return total == n * (__ldg(offs + 1) - __ldg(offs));
+}
+
+// The same for kernels that do nothing but hash: strings of one length need no order,
+// and a warp's lanes read neighbouring lines at the same time, so in place they take
+// less (hash and histogram of 3*10^6 strings of 16 bytes 56 -> 43 us, of 64 bytes 113 ->
+// 98; a query, with six blocks' staged tiles and probes on an SM, gains 10% there but
+// loses 1.5% on strings of mixed lengths).
+__device__ __forceinline__ Sig sig_each(const uint8_t* buf, const uint64_t* __restrict__ offs, uint64_t total,
+                                        uint64_t t0, uint64_t m, StringTile& t, uint64_t kh, uint64_t kl, uint64_t& i,
+                                        bool alike) {
+    if (!alike) return sig_tile(buf, offs, total, t0, m, t, kh, kl, i);
+    i = t0 + threadIdx.x;
+    if (i >= m) return Sig{0, 0};
+    const uint64_t o = __ldg(offs + i);
+    return sig_bytes(buf, total, o, __ldg(offs + i + 1) - o, kh, kl);
 }
 
 // ------------------------------------------------------- shard, local, edges

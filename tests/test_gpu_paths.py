@@ -243,3 +243,21 @@ def test_few_and_many_keys_of_requests(vf, total, pieces):  # noqa: F811
     reqs = [(kept[i % 7][0], kept[i % 7][1].repeat(5)[:m], None) for i, m in enumerate(sizes.tolist())]
     for (s, q, _), out in zip(reqs, vf.vf_query_batch(reqs)):
         assert len(q) == 0 or (host(out) == host(s.query(q))).all()
+
+
+@pytest.mark.parametrize("name,lengths", [
+    ("alike", [16] * 1000), ("alike by sum", [24, 16, 32, 24] + [24] * 600),         # all of one length, or so it seems
+    ("parts", [100] * 700 + [9]), ("parts of 48", [425] * 300 + [8]), ("of 47", [426] * 300 + [8]),
+    ("last part", [300] * 255 + [20_000, 17]), ("mixed parts", list(range(8, 520, 2)) * 3),
+    ("too long inside", [90] * 200 + [30_000] + [90] * 200)])
+@pytest.mark.parametrize("shift", [0, 5])
+def test_strings_beyond_a_stage_and_of_one_length(vf, orc, name, lengths, shift):  # noqa: F811
+    data, offs = packed(lengths, len(lengths))
+    buf = torch.zeros(len(data) + 16, dtype=torch.uint8, device="cuda")
+    buf[shift:shift + len(data)] = torch.from_numpy(data).cuda()
+    k, o = buf[shift:shift + len(data)], dev(offs)
+    assert (host(vf.vf_signatures(k, 5, offsets=o)) == orc.sigs(data, 5, offsets=offs)).all()
+    vals = synth.values(len(lengths), 16, 3)
+    p = vf.vf_params_default(kind=vf.FUNC, b=16, seed=1, key_kind=vf.KEYS_BYTES)
+    s = vf.vf_build(k, dev(vals), offsets=o, params=p)
+    assert (host(s.query(k, offsets=o)) == vals).all()
