@@ -365,7 +365,7 @@ def run_gpu(args):
     h2d_gbs = host_to_device_gbs(torch)
     hbm, peak_kind = peaks()
     per_phase, dom, roof = phase_table(phases, n, args.steps, b, kind, hbm, peak_kind, args.workload,
-                                       info.regime == vf.REGIME_FUSE, int(info.k))
+                                       info.regime == vf.REGIME_FUSE, int(info.k), TRAFFIC_CLUSTERS)
     launches = sum(v[1] for v in phases.values())
     build_ns, qgps = job_rates(b_ms, q_ms, n, world)
     e2e_ns, e2e_qgps = job_rates(e2e_b_ms, e2e_q_ms, n, world)
@@ -452,7 +452,7 @@ def _algo(ph, b, kind, k):
     return ALGO_BYTES[ph](b, kind) + extra
 
 
-def phase_table(phases, n, steps, b, kind, hbm, peak_kind, workload, fuse, k=3):
+def phase_table(phases, n, steps, b, kind, hbm, peak_kind, workload, fuse, k=3, traffic=None):
     attempts = max(1, phases.get("hash_hist", (0, 0))[1])
     units = {"hash_hist": n * attempts, "scatter": n * attempts, "incidence": n * attempts,
              "peel": n * attempts, "lge": n * attempts, "assign": n * steps, "query": 2 * n * steps}
@@ -480,7 +480,7 @@ def phase_table(phases, n, steps, b, kind, hbm, peak_kind, workload, fuse, k=3):
         if dom == "incidence" and fuse:
             kb = 3 * 8.0 + 4.0 * 1.105
         roof = {"bound": "hbm", "kernel": dom, "achieved": d["achieved_gbs"], "peak": hbm, "unit": "GB/s",
-                "frac": round(d["achieved_gbs"] / hbm, 4), "traffic": TRAFFIC.get((workload, dom)),
+                "frac": round(d["achieved_gbs"] / hbm, 4), "traffic": (TRAFFIC if traffic is None else traffic).get((workload, dom)),
                 "peak_source": f"{peak_kind} hbm_gbs", "algorithmic_bytes_per_unit": _algo(dom, b, kind, k),
                 "kernel_model": {"bytes_per_unit": kb, "achieved": d["kernel_model_gbs"],
                                  "frac": round(d["kernel_model_gbs"] / hbm, 4)}}
@@ -489,10 +489,12 @@ def phase_table(phases, n, steps, b, kind, hbm, peak_kind, workload, fuse, k=3):
 
 # Per-launch DRAM traffic (bytes) from ncu captures of the same kernels, scaled
 # from the captured case by units processed; absent until a capture of the
-# current kernel exists (profiles/ holds the summaries).
-TRAFFIC = {("c2", "peel"): round(1120.07e6 / 2e7 * 1e8),   # k_flow_peel, one launch per attempt at 1e8 (the clusters'
-                                                           # eight head rounds and waves: 92 B an edge, not 56)
+# current kernel exists (profiles/ holds the summaries). The first table is that of
+# lines measured with the worklist peel (k_flow_peel, one launch per attempt at 1e8);
+# the second of what runs now: k_front_scan, eight k_front_head, k_front_peel.
+TRAFFIC = {("c2", "peel"): round(1120.07e6 / 2e7 * 1e8),
            ("c2", "query"): round(189.42e6 / 2e7 * 1e8)}  # k_query, one launch per 1e8 queries
+TRAFFIC_CLUSTERS = {**TRAFFIC, ("c2", "peel"): round(1908.71e6 / 2e7 * 1e8)}
 
 
 # ---------------------------------------------------------------- reference arm

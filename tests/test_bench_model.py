@@ -85,3 +85,17 @@ def test_random_sector_query_model():
 def test_job_rates_aggregate_over_replicas():
     ns, gq = bench.job_rates(65.0, 4.0, N, 4)  # 4 replicas of 1e8 keys
     assert ns == pytest.approx(65.0e6 / (4 * N)) and gq == pytest.approx(8 * N / 4e-3 / 1e9)
+
+
+def test_traffic_of_the_peel_that_runs():
+    # what the benchmark prints is the clusters' capture (2e7 keys, MB read + written), not the worklist's
+    rows = open(os.path.join(ROOT, "profiles", "cluster_peel.md")).read().splitlines()
+    mb = 0.0
+    for kernel in ("k_front_scan", "k_front_head<", "k_front_peel<"):
+        row = [r for r in rows if r.startswith("| `" + kernel) and " + " in r]
+        assert len(row) == 1, kernel
+        mb += sum(float(x) for x in row[0].split("|")[3].split("+"))
+    assert bench.TRAFFIC_CLUSTERS[("c2", "peel")] == pytest.approx(mb * 1e6 / 2e7 * 1e8, rel=1e-5)
+    _, dom, roof = bench.phase_table(PHASES, N, STEPS, 8, "filter", HBM, "measured", "c2", True, 3,
+                                     bench.TRAFFIC_CLUSTERS)
+    assert dom == "peel" and roof["traffic"] == bench.TRAFFIC_CLUSTERS[("c2", "peel")]
