@@ -58,7 +58,8 @@ enum { VF_REGIME_FUSE = 1, VF_REGIME_LGE = 2, VF_REGIME_MWHC = 3 };
  * and shards whose rounds outgrow the clusters' lists, by an asynchronous worklist.
  * Both record peeled edges in an order whose reverse is a valid assignment order;
  * the assignment goes back round by round or as a dataflow.
- * VF_SOLVER_ROUNDS: peeling in synchronous rounds with a grid barrier, assignment in reverse rounds. VF_SOLVER_WAVE: vertex words
+ * VF_SOLVER_ROUNDS: peeling in synchronous rounds with a grid barrier,
+ * assignment in reverse rounds. VF_SOLVER_WAVE: vertex words
  * that sum the degree, the other two vertices and the value of the incident
  * edges, so a peeling step is one fetch-and-add per vertex; grid-wide rounds
  * for the initial cascades, then one CTA per shard for the waves that sweep

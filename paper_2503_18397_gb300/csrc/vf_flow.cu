@@ -1031,7 +1031,7 @@ static cudaError_t launch_assign_words(const FlowArgs& a, cudaStream_t st) {
 // the narrowest word that holds b bits and the final bit is (10^9 keys, b = 8,
 // 0.8 GB of such 64-bit words: 90 -> 62 ms; 10^8, 50 MB: 10.1 -> 9.9 ms). Cells of 8,
 // 16 or 32 bits in that many shards are assigned round by round instead
-// (front_assign_fits); MWHC graphs and other widths come here.
+// (front_assign_fits); MWHC graphs, graphs the worklist peeled and other widths come here.
 constexpr uint64_t kWideWordsMB = 48;
 
 cudaError_t launch_flow_assign(const FlowArgs& a, cudaStream_t st) {

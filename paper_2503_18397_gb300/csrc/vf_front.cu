@@ -36,9 +36,9 @@
 // (front_uneven; every CTA sees the same sizes), the round's pushes are dealt out over the
 // cluster through distributed shared memory, behind a full cluster barrier.
 //
-// Measured (one GB300, b = 8; peel per attempt, worklist -> this): 2^20 keys 4.37 ->
-// 3.55 ms, 10^8 (8 shards) 31.8 -> 26.0, 3*10^8 (16) 50.3 -> 30.9, 10^9 (64) 201 -> 85;
-// 4-uniform 10^8 15.2 -> 13.3, 3*10^8 56.9 -> 28.0. A round takes ~4300 cycles at 10^8:
+// Measured (one GB300, b = 8; peel per attempt, worklist -> this): 2^20 keys 2.92 ->
+// 2.59 ms, 10^8 (8 shards) 32.2 -> 26.8, 3*10^8 (16) 49.7 -> 27.0, 10^9 (64) 188 -> 86;
+// 4-uniform 10^8 14.9 -> 13.1, 3*10^8 56.5 -> 24.7 (and where it is slower: front_pays). A round takes ~4300 cycles at 10^8:
 // ~1100 to the claims and signatures, ~1400 to the removals, ~450 waiting for
 // the slowest CTA, the rest between them (a remote fetch-and-add also costs an
 // SM ~3.3 cycles a lane, L2 or distributed shared memory alike, and a CTA has

@@ -707,6 +707,8 @@ __global__ void __launch_bounds__(kLT, kMinBlocks) k_lge(LgeArgs a) {
             __syncthreads();
             continue;
         }
+        // (S * AW is more than is stored: a limit of its own, which shards of random keys
+        // do not come to)
         if (uint64_t(S) * AW > o.lpool || cm_words + rows_words > o.lpool || small_words > kLgeSmemWords) {
             if (tid == 0) {
                 atomicOr(a.err, kErrLgeSize);
